@@ -1,7 +1,8 @@
 """Thin Python binding of libthc's C ABI (include/thc.h): argument marshalling only.
 
 Every step of the round runs in the library's CUDA kernels.  PyTorch is used here for
-device memory and the current stream; nothing in this module computes.  If libthc.so is
+device memory and the current stream; nothing in this module computes.  The launching calls go
+through csrc/binding.c, which collects the tensors' addresses in C.  If libthc.so is
 missing the import of the library fails loudly -- there is no fallback path.
 """
 from __future__ import annotations
@@ -13,6 +14,7 @@ from dataclasses import dataclass
 _HERE = os.path.dirname(os.path.abspath(__file__))
 _LIB_PATH = os.path.join(_HERE, "libthc.so")
 _lib = None
+_native = None
 
 THC_OK, THC_EINVAL, THC_EUNSUPPORTED, THC_ECUDA, THC_EWORKSPACE = 0, -1, -2, -3, -4
 THC_F32, THC_BF16 = 0, 1
@@ -110,20 +112,6 @@ def _check(code: int, where: str):
         raise ThcError(code, where)
 
 
-def _ptr_array(ptrs):
-    arr = (ctypes.c_void_p * len(ptrs))(*[ctypes.c_void_p(int(p)) for p in ptrs])
-    return arr
-
-
-def _dp(t) -> int:
-    """Device (or host) address of a torch tensor / raw integer address / None."""
-    if t is None:
-        return 0
-    if isinstance(t, int):
-        return t
-    return t.data_ptr()
-
-
 def _stream(stream) -> int:
     if stream is None:
         import torch
@@ -133,6 +121,16 @@ def _stream(stream) -> int:
     return stream.cuda_stream
 
 
+def _binding():
+    """The C marshalling module (csrc/binding.c), linked to the same libthc.so."""
+    global _native
+    if _native is None:
+        lib()
+        from . import _binding as native
+        _native = native
+    return _native
+
+
 def prepare_noalloc(grads, d: int, log2_block: int, in_dtype: int, t_p: float, scales,
                     status=None, stream=None):
     """thc_prepare_noalloc: the preliminary stage for callers that may not allocate device
@@ -140,9 +138,7 @@ def prepare_noalloc(grads, d: int, log2_block: int, in_dtype: int, t_p: float, s
     (NOALLOC_SCRATCH_BYTES per GPU).  `status` is an optional device uint32 tensor the status
     bits are OR-ed into.  Raises ThcError(THC_EWORKSPACE) when the input is too large for
     the built-in scratch."""
-    arr = _ptr_array([_dp(g) for g in grads])
-    _check(lib().thc_prepare_noalloc(arr, len(grads), d, log2_block, in_dtype, float(t_p),
-                                     _dp(scales), _dp(status), _stream(stream)),
+    _check(_binding().prepare_noalloc(0, grads, d, log2_block, in_dtype, t_p, scales, status, stream),
            "thc_prepare_noalloc")
 
 
@@ -163,11 +159,14 @@ class Context:
         _check(lib().thc_create(ctypes.byref(cfg), ctypes.byref(self._h)), "thc_create")
         self.bits, self.granularity, self.log2_block = bits, granularity, log2_block
         self.workers = workers
+        self._handle = self._h.value
+        self._call = _binding()
 
     def close(self):
         if getattr(self, "_h", None) is not None and self._h.value:
             lib().thc_destroy(self._h)
             self._h = ctypes.c_void_p()
+            self._handle = 0
 
     def __del__(self):
         try:
@@ -182,77 +181,46 @@ class Context:
                      s.workspace_bytes, s.acc_bits, s.fused_scales, s.scales_count)
 
     def prepare(self, grads, d: int, scales, workspace, stream=None):
-        arr = _ptr_array([_dp(g) for g in grads])
-        _check(lib().thc_prepare(self._h, arr, len(grads), d, _dp(scales), _dp(workspace),
-                                 workspace.numel() * workspace.element_size(), _stream(stream)),
-               "thc_prepare")
+        _check(self._call.prepare(self._handle, grads, d, scales, workspace, stream), "thc_prepare")
 
     def prepare_minmax(self, grads, d: int, rnd: int, scales, workspace, rotated=None, stream=None):
-        arr = _ptr_array([_dp(g) for g in grads])
-        ra = _ptr_array([_dp(r) for r in rotated]) if rotated is not None else None
-        _check(lib().thc_prepare_minmax(self._h, arr, len(grads), d, rnd, _dp(scales), ra, _dp(workspace),
-                                        workspace.numel() * workspace.element_size(), _stream(stream)),
+        _check(self._call.prepare_minmax(self._handle, grads, d, rnd, scales, rotated, workspace, stream),
                "thc_prepare_minmax")
 
     def compress(self, grads, d: int, rnd: int, scales, packed, workspace, rotated=None,
                  worker_base: int = 0, stream=None):
-        n = len(grads)
-        ga = _ptr_array([_dp(g) for g in grads])
-        pa = _ptr_array([_dp(p) for p in packed])
-        ra = _ptr_array([_dp(r) for r in rotated]) if rotated is not None else None
-        ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-        _check(lib().thc_compress(self._h, ga, n, worker_base, d, rnd, _dp(scales), pa, ra,
-                                  _dp(workspace), ws_bytes, _stream(stream)), "thc_compress")
+        _check(self._call.compress(self._handle, grads, worker_base, d, rnd, scales, packed, rotated,
+                                   workspace, stream), "thc_compress")
 
     def prepare_compress(self, grads, d: int, rnd: int, scales, packed, workspace, rotated=None,
                          worker_base: int = 0, stream=None):
-        n = len(grads)
-        ga = _ptr_array([_dp(g) for g in grads])
-        pa = _ptr_array([_dp(p) for p in packed])
-        ra = _ptr_array([_dp(r) for r in rotated]) if rotated is not None else None
-        _check(lib().thc_prepare_compress(self._h, ga, n, worker_base, d, rnd, _dp(scales), pa, ra,
-                                          _dp(workspace), workspace.numel() * workspace.element_size(),
-                                          _stream(stream)), "thc_prepare_compress")
+        _check(self._call.prepare_compress(self._handle, grads, worker_base, d, rnd, scales, packed,
+                                           rotated, workspace, stream), "thc_prepare_compress")
 
     def quantize_rotated(self, rotated, d: int, rnd: int, scales, packed, worker_base: int = 0,
                          stream=None):
-        ra = _ptr_array([_dp(r) for r in rotated])
-        pa = _ptr_array([_dp(p) for p in packed])
-        _check(lib().thc_quantize_rotated(self._h, ra, len(rotated), worker_base, d, rnd,
-                                          _dp(scales), pa, _stream(stream)), "thc_quantize_rotated")
+        _check(self._call.quantize_rotated(self._handle, rotated, worker_base, d, rnd, scales, packed,
+                                           stream), "thc_quantize_rotated")
 
     def aggregate(self, packed, d: int, total, stream=None):
-        pa = _ptr_array([_dp(p) for p in packed])
-        _check(lib().thc_aggregate(self._h, pa, len(packed), d, _dp(total), _stream(stream)),
-               "thc_aggregate")
+        _check(self._call.aggregate(self._handle, packed, d, total, stream), "thc_aggregate")
 
     def decompress(self, total, divisor: int, d: int, rnd: int, scales, out, workspace,
                    stream=None):
-        ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-        _check(lib().thc_decompress(self._h, _dp(total), divisor, d, rnd, _dp(scales), _dp(out),
-                                    _dp(workspace), ws_bytes, _stream(stream)), "thc_decompress")
+        _check(self._call.decompress(self._handle, total, divisor, d, rnd, scales, out, workspace,
+                                     stream), "thc_decompress")
 
     def aggregate_decompress(self, packed, d: int, rnd: int, scales, out, workspace, total=None,
                              stream=None):
-        pa = _ptr_array([_dp(p) for p in packed])
-        ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-        _check(lib().thc_aggregate_decompress(self._h, pa, len(packed), d, rnd, _dp(scales), _dp(out),
-                                              _dp(total), _dp(workspace), ws_bytes, _stream(stream)),
-               "thc_aggregate_decompress")
+        _check(self._call.aggregate_decompress(self._handle, packed, d, rnd, scales, out, total,
+                                               workspace, stream), "thc_aggregate_decompress")
 
     def error_feedback(self, grads, packed, d: int, rnd: int, scales, ef, workspace, stream=None):
-        ga = _ptr_array([_dp(g) for g in grads])
-        pa = _ptr_array([_dp(p) for p in packed])
-        ea = _ptr_array([_dp(e) for e in ef])
-        _check(lib().thc_error_feedback(self._h, ga, pa, len(grads), d, rnd, _dp(scales), ea,
-                                        _dp(workspace), workspace.numel() * workspace.element_size(),
-                                        _stream(stream)), "thc_error_feedback")
+        _check(self._call.error_feedback(self._handle, grads, packed, d, rnd, scales, ef, workspace,
+                                         stream), "thc_error_feedback")
 
     def accumulate_error(self, grads, ef, d: int, stream=None):
-        ga = _ptr_array([_dp(g) for g in grads])
-        ea = _ptr_array([_dp(e) for e in ef])
-        _check(lib().thc_accumulate_error(self._h, ga, ea, len(grads), d, _stream(stream)),
-               "thc_accumulate_error")
+        _check(self._call.accumulate_error(self._handle, grads, ef, d, stream), "thc_accumulate_error")
 
     def debug_skip_tasks(self, count: int):
         """Test hook: the next pipeline launch starts its task queue at `count`."""
