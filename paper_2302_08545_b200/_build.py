@@ -17,8 +17,8 @@ CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libthc.so")
 BINDING = os.path.join(HERE, "_binding.so")
 BINDING_SOURCE = os.path.join(CSRC, "binding.c")
-SOURCES = ["thc.cu", "thc_noalloc.cu"]
-HEADERS = ["thc_device.cuh", "thc_pipeline.cuh", os.path.join("..", "..", "include", "thc.h")]
+SOURCES = ["thc.cu", "thc_block.cu", "thc_noalloc.cu"]
+HEADERS = ["thc_device.cuh", "thc_pipeline.cuh", "thc_block.h", os.path.join("..", "..", "include", "thc.h")]
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a",
@@ -26,6 +26,7 @@ NVCC_FLAGS = [
     "-fmad=false", "-prec-div=true", "-prec-sqrt=true", "-ftz=false",
     "-Xcompiler", "-fPIC", "-shared",
     "-cudart", "shared",
+    "--threads", "3",                # the source files side by side
 ]
 
 

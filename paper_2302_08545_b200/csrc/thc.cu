@@ -1,11 +1,8 @@
 // libthc: kernels and C ABI.  See include/thc.h for the contract of every entry point.
 //
-// Structure of the transform.  An RHT block of B = 2^k coordinates with k <= 14 is handled by
-// rht_tile_kernel below: a CTA holds a tile of 2^14 consecutive coordinates (one block or
-// several small ones) in shared memory: load (+ sign flip or de-quantisation), stages of
-// stride 1 .. 2^(k-1), then the fused epilogue: scale by 1/sqrt(B) and either truncate +
-// quantise + pack (compress), sign flip + store (decompress) or min / max (exact range).
-// Larger blocks go through the persistent two-pass pipeline of thc_pipeline.cuh.
+// Structure of the transform.  RHT blocks of up to 2^16 coordinates are held in shared memory by one
+// CTA or a cluster (thc_block.cuh); larger blocks go through the persistent two-pass pipeline of
+// thc_pipeline.cuh.
 #include "../../include/thc.h"
 #include "thc_device.cuh"
 
@@ -19,294 +16,6 @@ namespace thc {
 
 struct PtrArray { const void *p[THC_MAX_WORKERS]; };
 struct MutPtrArray { void *p[THC_MAX_WORKERS]; };
-
-enum LoadKind { kLoadGradF32, kLoadGradBF16, kLoadSum8, kLoadSum16, kLoadSum32 };
-enum StoreKind { kStoreQuant, kStoreOut, kStoreRange };
-
-// Geometry of the tiles one launch walks.
-struct TileGeom {
-    uint64_t d;            // valid coordinates per worker
-    uint64_t d_pad;
-    uint64_t row_stride;   // coordinates between consecutive tile rows
-    uint32_t k;            // log2 of the RHT block
-    uint32_t row_log2;     // tile = 2^row_log2 rows ...
-    uint32_t col_log2;     // ... of 2^col_log2 consecutive coordinates (sum = 14)
-    uint32_t lo_cbit;      // chunk-index bits [lo_cbit, hi_cbit) are transformed
-    uint32_t hi_cbit;
-    uint32_t blocks_in_tile;   // RHT blocks a tile overlaps (1 if k >= 14)
-    uint32_t lut_rep;          // lane replication of the quantiser table in shared memory
-    uint32_t granularity;
-    uint32_t divisor;          // decompress: workers summed
-    uint32_t round;
-    uint32_t worker_base;
-    float    c_block;          // (float)(1/sqrt(B))
-    uint32_t exact_range;      // scales = nblocks minima then nblocks maxima (else M per block)
-};
-
-__device__ __forceinline__ uint64_t tile_base(const TileGeom &g, uint32_t tile)
-{
-    if (g.row_log2 == 0) return (uint64_t)tile << kTileLog2;
-    const uint32_t panels = 1u << g.row_log2;          // panels per RHT block
-    const uint64_t blk = tile >> g.row_log2;
-    const uint64_t panel = tile & (panels - 1);
-    return (blk << g.k) + (panel << g.col_log2);
-}
-
-__device__ __forceinline__ uint64_t chunk_coord(const TileGeom &g, uint64_t base, int c)
-{
-    const int ccl = (int)g.col_log2 - 2;
-    const uint64_t row = (uint64_t)(c >> ccl);
-    const uint64_t cc = (uint64_t)(c & ((1 << ccl) - 1));
-    return base + row * g.row_stride + cc * 4;
-}
-
-// Sign words of every row of the tile, 32 coordinates per word.
-__device__ __forceinline__ void fill_sign_words(uint32_t *sw, const TileGeom &g, uint64_t base,
-                                                const PhiloxKeys &keys, int tid,
-                                                int nthreads = kThreads)
-{
-    const int cols = 1 << g.col_log2;
-    const int words_per_row = max(1, cols >> 5);
-    const int calls_per_row = max(1, cols >> 7);
-    const int rows = 1 << g.row_log2;
-    const int words_per_call = min(4, words_per_row);
-    for (int q = tid; q < rows * calls_per_row; q += nthreads) {
-        const int row = q / calls_per_row;
-        const int cr = q - row * calls_per_row;
-        const uint64_t j0 = base + (uint64_t)row * g.row_stride + (uint64_t)cr * 128;
-        const uint4 ph = sign_call(j0, g.round, keys);
-        const int first = (int)((j0 >> 5) & 3);
-        for (int wi = 0; wi < words_per_call; ++wi) {
-            const int src = first + wi;
-            const uint32_t w = src == 0 ? ph.x : src == 1 ? ph.y : src == 2 ? ph.z : ph.w;
-            sw[row * words_per_row + cr * 4 + wi] = w;
-        }
-    }
-}
-
-__device__ __forceinline__ uint32_t sign_bits_of_chunk(const uint32_t *sw, const TileGeom &g,
-                                                       int c, uint64_t j)
-{
-    const int ccl = (int)g.col_log2 - 2;
-    const int row = c >> ccl;
-    const int cc = c & ((1 << ccl) - 1);
-    const int words_per_row = max(1, (1 << g.col_log2) >> 5);
-    return sw[row * words_per_row + (cc >> 3)] >> (uint32_t)(j & 31);
-}
-
-__device__ __forceinline__ float4 load_f32x4_masked(const float *x, uint64_t j, uint64_t d)
-{
-    if (j + 4 <= d) return __ldg(reinterpret_cast<const float4 *>(x + j));
-    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (j + 0 < d) v.x = __ldg(x + j + 0);
-    if (j + 1 < d) v.y = __ldg(x + j + 1);
-    if (j + 2 < d) v.z = __ldg(x + j + 2);
-    if (j + 3 < d) v.w = __ldg(x + j + 3);
-    return v;
-}
-
-// Eight 3-bit indices (24 bits, coordinate 0 in the low bits) go to bytes 3 (j/8) .. +2.
-__device__ __forceinline__ void store_packed3(unsigned char *pk, uint64_t j, uint32_t z)
-{
-    unsigned char *p = pk + 3 * (j >> 3);
-    p[0] = (unsigned char)z;
-    p[1] = (unsigned char)(z >> 8);
-    p[2] = (unsigned char)(z >> 16);
-}
-
-__device__ __forceinline__ float sum_to_float(uint32_t y)   // exact for y < 2^23
-{
-    return __uint_as_float(0x4B000000u | y) - 8388608.0f;
-}
-
-// One tile: load, butterfly rounds, store.  blockIdx.x = tile, blockIdx.y = local worker.
-template <int LOAD, int STORE, int BITS, bool IDENTITY>
-__global__ void __launch_bounds__(kThreads, 2)
-rht_tile_kernel(TileGeom g, PtrArray in, MutPtrArray out, MutPtrArray rotated,
-                const float *__restrict__ scales, DeviceBlock *dev, PhiloxKeys keys)
-{
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    float4 *tile = reinterpret_cast<float4 *>(smem_raw);
-    uint32_t *sw = reinterpret_cast<uint32_t *>(smem_raw + kTileElems * 4);
-    float2 *blk_const = reinterpret_cast<float2 *>(smem_raw + kTileElems * 4 + kSignWordsMax * 4);
-    unsigned char *lut = smem_raw + kTileElems * 4 + kSignWordsMax * 4 +
-                         (((size_t)g.blocks_in_tile * 8 + 15) & ~(size_t)15);
-
-    const int tid = threadIdx.x;
-    const uint32_t wl = blockIdx.y;
-    const uint64_t base = tile_base(g, blockIdx.x);
-    const uint64_t first_blk = base >> g.k;
-    const uint64_t nblocks = g.d_pad >> g.k;
-
-    // ---- per-tile constants
-    if (LOAD == kLoadGradF32 || LOAD == kLoadGradBF16 || STORE == kStoreOut)
-        fill_sign_words(sw, g, base, keys, tid);
-    if (STORE == kStoreQuant) {
-        // (1/(2M), 1/2) per block; (0, 0) for a degenerate block
-        for (uint32_t b = tid; b < g.blocks_in_tile; b += kThreads) {
-            float2 c = make_float2(0.f, 0.f);
-            if (first_blk + b < nblocks)
-                c = compress_constants(block_range(scales, first_blk + b, nblocks, g.exact_range));
-            blk_const[b] = c;
-        }
-        if (!IDENTITY) lut_fill<LutKind<BITS, IDENTITY>::k8>(lut, dev, g.granularity, tid, kThreads);
-    }
-    if (LOAD == kLoadSum8 || LOAD == kLoadSum16 || LOAD == kLoadSum32) {
-        // (step, -M) per block; (0, 0) for a degenerate block
-        for (uint32_t b = tid; b < g.blocks_in_tile; b += kThreads) {
-            float2 c = make_float2(0.f, 0.f);
-            if (first_blk + b < nblocks)
-                c = decode_constants(block_range(scales, first_blk + b, nblocks, g.exact_range),
-                                     g.granularity, g.divisor);
-            blk_const[b] = c;
-        }
-    }
-    __syncthreads();
-
-    // ---- load phase
-    if (LOAD == kLoadGradF32) {
-        const float *x = static_cast<const float *>(in.p[wl]);
-#pragma unroll 4
-        for (int i = 0; i < kTileChunks / kThreads; ++i) {
-            const int c = tid + i * kThreads;
-            const uint64_t j = base + (uint64_t)c * 4;
-            float4 v = load_f32x4_masked(x, j, g.d);
-            v = flip4(v, sw[c >> 3] >> ((c & 7) * 4));
-            tile[swz(c)] = stages01(v);
-        }
-    } else if (LOAD == kLoadGradBF16) {
-        const uint16_t *x = static_cast<const uint16_t *>(in.p[wl]);
-#pragma unroll 2
-        for (int i = 0; i < kTileChunks / 2 / kThreads; ++i) {
-            const int u = tid + i * kThreads;                 // 8 coordinates
-            const uint64_t j = base + (uint64_t)u * 8;
-            uint32_t w[4] = {0, 0, 0, 0};
-            if (j + 8 <= g.d) {
-                const uint4 q = __ldg(reinterpret_cast<const uint4 *>(x + j));
-                w[0] = q.x; w[1] = q.y; w[2] = q.z; w[3] = q.w;
-            } else {
-                for (int e = 0; e < 8; ++e)
-                    if (j + e < g.d) w[e >> 1] |= (uint32_t)__ldg(x + j + e) << ((e & 1) * 16);
-            }
-            float4 v0 = make_float4(__uint_as_float(w[0] << 16), __uint_as_float(w[0] & 0xFFFF0000u),
-                                    __uint_as_float(w[1] << 16), __uint_as_float(w[1] & 0xFFFF0000u));
-            float4 v1 = make_float4(__uint_as_float(w[2] << 16), __uint_as_float(w[2] & 0xFFFF0000u),
-                                    __uint_as_float(w[3] << 16), __uint_as_float(w[3] & 0xFFFF0000u));
-            const int c = 2 * u;
-            const uint32_t bits = sw[c >> 3] >> ((c & 7) * 4);
-            tile[swz(c)] = stages01(flip4(v0, bits));
-            tile[swz(c + 1)] = stages01(flip4(v1, bits >> 4));
-        }
-    } else if (LOAD == kLoadSum8 || LOAD == kLoadSum16 || LOAD == kLoadSum32) {
-        constexpr int kPer = LOAD == kLoadSum8 ? 16 : LOAD == kLoadSum16 ? 8 : 4;   // sums per 16 B
-        const unsigned char *y = static_cast<const unsigned char *>(in.p[0]);
-        for (int i = 0; i < kTileElems / kPer / kThreads; ++i) {
-            const int u = tid + i * kThreads;
-            const uint64_t j = base + (uint64_t)u * kPer;
-            uint4 q = make_uint4(0, 0, 0, 0);
-            if (j + kPer <= g.d_pad) {
-                q = __ldg(reinterpret_cast<const uint4 *>(y + j * (16 / kPer)));
-            } else if (j < g.d_pad) {          // only 8-bit sums with 8-coordinate blocks
-                const uint2 h = __ldg(reinterpret_cast<const uint2 *>(y + j * (16 / kPer)));
-                q.x = h.x; q.y = h.y;
-            }
-            const uint32_t w[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-            for (int cc = 0; cc < kPer / 4; ++cc) {
-                uint64_t bi = ((j + cc * 4) >> g.k) - first_blk;
-                if (bi >= g.blocks_in_tile) bi = 0;
-                const float2 bc = blk_const[bi];
-                float s[4];
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const int idx = cc * 4 + e;
-                    uint32_t val;
-                    if (LOAD == kLoadSum8) val = (w[idx >> 2] >> ((idx & 3) * 8)) & 0xFFu;
-                    else if (LOAD == kLoadSum16) val = (w[idx >> 1] >> ((idx & 1) * 16)) & 0xFFFFu;
-                    else val = w[idx];
-                    const float yf = LOAD == kLoadSum32 ? (float)val : sum_to_float(val);
-                    s[e] = fmaf(yf, bc.x, bc.y);
-                }
-                tile[swz(u * (kPer / 4) + cc)] = stages01(make_float4(s[0], s[1], s[2], s[3]));
-            }
-        }
-    }
-    __syncthreads();
-
-    // ---- butterflies
-    fwht_rounds(tile, (int)g.lo_cbit, (int)g.hi_cbit, tid);
-
-    // ---- store phase
-    if (STORE == kStoreQuant) {
-        unsigned char *pk = static_cast<unsigned char *>(out.p[wl]);
-        float *rot = static_cast<float *>(rotated.p[wl]);
-        const float gf = (float)g.granularity;
-        const uint32_t my_lut = lut_lane_addr<LutKind<BITS, IDENTITY>::k8>(lut, tid);
-#pragma unroll 1
-        for (int i = 0; i < kTileChunks / 2 / kThreads; ++i) {
-            const int u = tid + i * kThreads;
-            const int c = 2 * u;
-            const uint64_t j = chunk_coord(g, base, c);
-            if (j >= g.d_pad) continue;
-            const float4 a = scale4(tile[swz(c)], g.c_block);
-            const float4 b = scale4(tile[swz(c + 1)], g.c_block);
-            if (rot != nullptr) {
-                *reinterpret_cast<float4 *>(rot + j) = a;
-                *reinterpret_cast<float4 *>(rot + j + 4) = b;
-            }
-            const float r[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-            const float2 bc = blk_const[(j >> g.k) - first_blk];
-            const uint4 rnd = round_call(j, g.worker_base + wl, g.round, keys);
-            const uint64_t z = quantize8<BITS, IDENTITY>(r, bc.x, bc.y, gf, rnd, my_lut);
-            if constexpr (BITS == 8) *reinterpret_cast<uint2 *>(pk + j) = make_uint2((uint32_t)z, (uint32_t)(z >> 32));
-            else if constexpr (BITS == 4) *reinterpret_cast<uint32_t *>(pk + j / 2) = (uint32_t)z;
-            else if constexpr (BITS == 3) store_packed3(pk, j, (uint32_t)z);
-            else if constexpr (BITS == 2) *reinterpret_cast<uint16_t *>(pk + j / 4) = (uint16_t)z;
-            else pk[j / 8] = (unsigned char)z;
-        }
-    } else if (STORE == kStoreRange) {
-        // min / max of the rotated coordinates per RHT block, as ordered keys: out.p[0] holds
-        // nblocks min keys followed by nblocks max keys.  For blocks of at least 128
-        // coordinates the 32 chunks of a warp lie in one block and are reduced first.
-        uint32_t *rk = static_cast<uint32_t *>(out.p[0]);
-#pragma unroll 1
-        for (int i = 0; i < kTileChunks / kThreads; ++i) {
-            const int c = tid + i * kThreads;
-            const uint64_t j = chunk_coord(g, base, c);
-            if (j >= g.d_pad) continue;
-            const float4 v = scale4(tile[swz(c)], g.c_block);
-            if (rotated.p[wl] != nullptr) *reinterpret_cast<float4 *>(static_cast<float *>(rotated.p[wl]) + j) = v;
-            const uint32_t k0 = float_key(v.x), k1 = float_key(v.y), k2 = float_key(v.z), k3 = float_key(v.w);
-            uint32_t kmin = min(min(k0, k1), min(k2, k3));
-            uint32_t kmax = max(max(k0, k1), max(k2, k3));
-            const uint64_t blk = j >> g.k;
-            if (g.k >= 7) {
-                kmin = __reduce_min_sync(0xFFFFFFFFu, kmin);
-                kmax = __reduce_max_sync(0xFFFFFFFFu, kmax);
-                if ((tid & 31) != 0) continue;
-            }
-            atomicMin(rk + blk, kmin);
-            atomicMax(rk + nblocks + blk, kmax);
-        }
-    } else {   // kStoreOut
-        float *o = static_cast<float *>(out.p[0]);
-#pragma unroll 4
-        for (int i = 0; i < kTileChunks / kThreads; ++i) {
-            const int c = tid + i * kThreads;
-            const uint64_t j = chunk_coord(g, base, c);
-            if (j >= g.d) continue;
-            float4 v = scale4(tile[swz(c)], g.c_block);
-            v = flip4(v, sign_bits_of_chunk(sw, g, c, j));
-            if (j + 4 <= g.d) {
-                *reinterpret_cast<float4 *>(o + j) = v;
-            } else {
-                o[j] = v.x;
-                if (j + 1 < g.d) o[j + 1] = v.y;
-                if (j + 2 < g.d) o[j + 2] = v.z;
-            }
-        }
-    }
-}
 
 constexpr int kQrBlockCache = 1024;
 
@@ -344,11 +53,7 @@ quantize_rotated_kernel(PtrArray rotated, MutPtrArray packed, uint64_t d_pad, ui
         const float kappa = kc.x, offset = kc.y;
         const uint4 rnd = round_call(j, worker_base + wl, round, keys);
         const uint64_t z = quantize8<BITS, IDENTITY>(r, kappa, offset, gf, rnd, my_lut);
-        if constexpr (BITS == 8) *reinterpret_cast<uint2 *>(pk + j) = make_uint2((uint32_t)z, (uint32_t)(z >> 32));
-        else if constexpr (BITS == 4) *reinterpret_cast<uint32_t *>(pk + j / 2) = (uint32_t)z;
-        else if constexpr (BITS == 3) store_packed3(pk, j, (uint32_t)z);
-        else if constexpr (BITS == 2) *reinterpret_cast<uint16_t *>(pk + j / 4) = (uint16_t)z;
-        else pk[j / 8] = (unsigned char)z;
+        store_unit<BITS>(pk, j, z);
     }
 }
 
@@ -359,13 +64,6 @@ quantize_rotated_kernel(PtrArray rotated, MutPtrArray packed, uint64_t d_pad, ui
 // low half of the table answers indices 0-7 and, with bit 3 flipped, the high half answers
 // 8-15; the two results are disjoint and are added into packed byte accumulators (no byte
 // can overflow because workers * g <= 255).
-__device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel)
-{
-    uint32_t d;
-    asm("prmt.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(sel));
-    return d;
-}
-
 __global__ void __launch_bounds__(kThreads)
 aggregate_b4w8_kernel(PtrArray in, uint32_t n, uint64_t units32, const DeviceBlock *dev,
                       uint4 *__restrict__ sum)
@@ -542,23 +240,7 @@ aggregate_b8w16_kernel(PtrArray in, uint32_t n, uint64_t units16, uint4 *__restr
 }
 
 // ------------------------------------------------------------------------ error feedback
-// e <- x - e (e holds RHT^-1(X) on entry) and x <- x + e, 128-bit accesses with a scalar tail.
-__global__ void __launch_bounds__(kThreads)
-ef_subtract_kernel(const float *__restrict__ x, float *__restrict__ e, uint64_t d)
-{
-    const uint64_t n4 = d / 4;
-    for (uint64_t c = (uint64_t)blockIdx.x * kThreads + threadIdx.x; c < n4; c += (uint64_t)gridDim.x * kThreads) {
-        const float4 a = __ldg(reinterpret_cast<const float4 *>(x) + c);
-        float4 b = reinterpret_cast<float4 *>(e)[c];
-        b.x = a.x - b.x; b.y = a.y - b.y; b.z = a.z - b.z; b.w = a.w - b.w;
-        reinterpret_cast<float4 *>(e)[c] = b;
-    }
-    if (blockIdx.x == 0 && threadIdx.x < (d & 3)) {
-        const uint64_t j = n4 * 4 + threadIdx.x;
-        e[j] = x[j] - e[j];
-    }
-}
-
+// x <- x + e, 128-bit accesses with a scalar tail.
 __global__ void __launch_bounds__(kThreads)
 accumulate_kernel(float *__restrict__ x, const float *__restrict__ e, uint64_t d)
 {
@@ -782,6 +464,7 @@ aggregate_kernel(PtrArray in, uint32_t n, uint64_t units, uint64_t d_pad, const 
 }  // namespace thc
 
 #include "thc_pipeline.cuh"
+#include "thc_block.h"
 
 // =========================================================================== host side
 using namespace thc;
@@ -793,7 +476,7 @@ struct thc_ctx {
     int device;                 // -1: no CUDA device, host-only context
     DeviceBlock *dev;
     PhiloxKeys keys;
-    uint32_t lut_rep;
+    bool pipeline_next;         // the queue of the next pipeline launch is set (thc_debug_skip_tasks)
     int sm_count;
     // Encoded tensor maps of recent launches, keyed by what they describe: a training loop calls
     // with the same buffers every step, and encoding up to n + 1 maps per call costs more host
@@ -893,7 +576,7 @@ int thc_create(const thc_config *cfg, thc_ctx **out)
         k1 += 0xBB67AE85u;
     }
     const uint32_t g = cfg->granularity;
-    ctx->lut_rep = 8;
+    ctx->pipeline_next = false;
 
     // host copy of the device block
     DeviceBlock *h = new (std::nothrow) DeviceBlock;
@@ -1017,10 +700,10 @@ int thc_sizes(const thc_ctx *ctx, uint64_t d, uint32_t n_local, thc_sizes_t *s)
     s->rotated_bytes = s->d_pad * 4;
     s->acc_bits = ctx->acc_bits;
     s->scales_count = ctx->cfg.range_mode == THC_RANGE_MINMAX ? 2 * s->nblocks : s->nblocks;
-    const uint32_t chunk_log2 = k < (uint32_t)kTileLog2 ? k : (uint32_t)kTileLog2;
+    const uint32_t chunk_log2 = k < (uint32_t)kChunkLog2 ? k : (uint32_t)kChunkLog2;
     const uint64_t prepare_ws = (uint64_t)n_local * (s->d_pad >> chunk_log2) * 8;
     uint64_t two_pass_ws = 0;
-    if (k > (uint32_t)kTileLog2) {
+    if (k > (uint32_t)kChunkLog2) {
         const PipePlan pl = plan_pipeline(ctx, s->nblocks * n_local);
         two_pass_ws = (uint64_t)pl.ring * B * 4 + s->nblocks * 8;       // + range keys
         PipePlan pf;
@@ -1069,7 +752,7 @@ int thc_prepare(thc_ctx *ctx, const void *const *grads, uint32_t n, uint64_t d, 
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const uint32_t k = ctx->cfg.log2_block;
     if (ctx->cfg.range_mode == THC_RANGE_MINMAX) return THC_EUNSUPPORTED;   // thc_prepare_minmax
-    const uint32_t chunk_log2 = k < (uint32_t)kTileLog2 ? k : (uint32_t)kTileLog2;
+    const uint32_t chunk_log2 = k < (uint32_t)kChunkLog2 ? k : (uint32_t)kChunkLog2;
     const uint64_t chunks_per_worker = sz.d_pad >> chunk_log2;
     const uint64_t chunks_per_block = 1ull << (k - chunk_log2);
     if (chunks_per_worker > 0x7FFFFFFFull) return THC_EUNSUPPORTED;
@@ -1087,33 +770,6 @@ int thc_prepare(thc_ctx *ctx, const void *const *grads, uint32_t n, uint64_t d, 
         partial, n, sz.nblocks, chunks_per_block, chunks_per_worker, ctx->cfg.t_p, k, scales, ctx->dev);
     THC_CUDA(cudaGetLastError());
     return THC_OK;
-}
-
-// ---- tile-kernel dispatch
-typedef void (*tile_kernel_t)(TileGeom, PtrArray, MutPtrArray, MutPtrArray, const float *,
-                              DeviceBlock *, PhiloxKeys);
-
-template <int LOAD, int STORE>
-static tile_kernel_t pick_tile_kernel(uint32_t bits, bool identity)
-{
-    if constexpr (STORE != kStoreQuant) {
-        return rht_tile_kernel<LOAD, STORE, 4, true>;
-    } else {
-    switch (bits) {
-    case 1: return identity ? rht_tile_kernel<LOAD, STORE, 1, true> : rht_tile_kernel<LOAD, STORE, 1, false>;
-    case 2: return identity ? rht_tile_kernel<LOAD, STORE, 2, true> : rht_tile_kernel<LOAD, STORE, 2, false>;
-    case 3: return identity ? rht_tile_kernel<LOAD, STORE, 3, true> : rht_tile_kernel<LOAD, STORE, 3, false>;
-    case 4: return identity ? rht_tile_kernel<LOAD, STORE, 4, true> : rht_tile_kernel<LOAD, STORE, 4, false>;
-    default: return identity ? rht_tile_kernel<LOAD, STORE, 8, true> : rht_tile_kernel<LOAD, STORE, 8, false>;
-    }
-    }
-}
-
-static size_t tile_smem_bytes(const thc_ctx *ctx, const TileGeom &g)
-{
-    return (size_t)kTileElems * 4 + kSignWordsMax * 4 +
-           (((size_t)g.blocks_in_tile * 8 + 15) & ~(size_t)15) +
-           (size_t)(ctx->cfg.granularity + 1) * kLutEntryBytes;
 }
 
 // cudaFuncSetAttribute is needed once per kernel and dynamic shared-memory size; remember
@@ -1138,44 +794,6 @@ static int ensure_dynamic_smem(const void *kern, size_t smem)
     THC_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     if (seen < 96) { seen_kern[seen] = kern; seen_size[seen] = smem; seen_dev[seen] = dev; ++seen; }
     return THC_OK;
-}
-
-static int launch_tile(const thc_ctx *ctx, tile_kernel_t kern, const TileGeom &g, uint64_t tiles,
-                       uint32_t n_local, const PtrArray &in, const MutPtrArray &out,
-                       const MutPtrArray &rot, const float *scales, cudaStream_t st)
-{
-    if (tiles > 0x7FFFFFFFull) return THC_EUNSUPPORTED;
-    const size_t smem = tile_smem_bytes(ctx, g);
-    { const int rc = ensure_dynamic_smem(reinterpret_cast<const void *>(kern), smem); if (rc != THC_OK) return rc; }
-    kern<<<dim3((unsigned)tiles, n_local), kThreads, smem, st>>>(g, in, out, rot, scales, ctx->dev,
-                                                                 ctx->keys);
-    THC_CUDA(cudaGetLastError());
-    return THC_OK;
-}
-
-static TileGeom base_geom(const thc_ctx *ctx, const thc_sizes_t &sz, uint64_t d, uint32_t round)
-{
-    TileGeom g;
-    memset(&g, 0, sizeof g);
-    g.d = d;
-    g.d_pad = sz.d_pad;
-    g.k = ctx->cfg.log2_block;
-    g.lut_rep = ctx->lut_rep;
-    g.granularity = ctx->cfg.granularity;
-    g.round = round;
-    g.c_block = (float)(1.0 / sqrt((double)(1ull << g.k)));
-    g.exact_range = ctx->cfg.range_mode == THC_RANGE_MINMAX ? 1u : 0u;
-    return g;
-}
-
-static void geom_pass_a(TileGeom &g)
-{
-    g.row_log2 = 0;
-    g.col_log2 = kTileLog2;
-    g.row_stride = 0;
-    g.lo_cbit = 0;
-    g.hi_cbit = (g.k < (uint32_t)kTileLog2 ? g.k : (uint32_t)kTileLog2) - 2;
-    g.blocks_in_tile = g.k >= (uint32_t)kTileLog2 ? 1u : 1u << (kTileLog2 - g.k);
 }
 
 // ---- persistent pipeline dispatch (RHT blocks of 2^15 .. 2^24 coordinates)
@@ -1407,6 +1025,87 @@ static int launch_pipeline(const thc_ctx *ctx, pipe_kernel_t kern, bool compress
     return THC_OK;
 }
 
+// ---- blocks held in shared memory (RHT blocks of up to 2^16 coordinates)
+// Blocks up to 2^15 always; 2^16 up to 2^22 coordinates over all workers, where the two-pass pipeline
+// has less than a task per CTA and its chain of queue, ring and counters is all latency: 8.8 us
+// instead of 13.9 on a block or two, 21 instead of 23 on 2^22 coordinates; on 2^24 the cluster's
+// gather makes it 74 against 53.
+static bool use_block_kernel(const thc_ctx *ctx, uint64_t coords)
+{
+    if (ctx->pipeline_next) return false;
+    return ctx->cfg.log2_block < kBMaxLog2 || (ctx->cfg.log2_block == kBMaxLog2 && coords <= (1ull << 22));
+}
+
+// lut_bytes: table space in shared memory; keys: exact-range mode; agg_n: aggregate + decompress.
+static int launch_block(const thc_ctx *ctx, const void *kern, PipeMode mode, size_t lut_bytes, const thc_sizes_t &sz,
+                        uint64_t d, uint32_t n_local, uint32_t worker_base, uint32_t round, uint32_t divisor,
+                        const float *scales, const PtrArrayP &in, const MutPtrArrayP &out, const MutPtrArrayP &rot,
+                        cudaStream_t st, uint32_t *keys = nullptr, uint32_t agg_n = 0)
+{
+    const uint32_t k = ctx->cfg.log2_block;
+    BlockParams P;
+    memset(&P, 0, sizeof P);
+    const uint32_t tile_log2 = block_tile_log2(block_kind(k)), e = block_cluster_log2(block_kind(k));
+    const size_t tile = (size_t)1 << tile_log2;
+    const uint64_t units = e != 0u ? sz.nblocks : (sz.d_pad + tile - 1) >> tile_log2;
+    if ((units << e) * n_local >= 0x7FFFFFFFull || sz.nblocks >= 0xFFFFFFFFull) return THC_EUNSUPPORTED;
+    P.d = d;
+    P.d_pad = sz.d_pad;
+    P.scales = scales;
+    P.dev = ctx->dev;
+    P.tasks = (uint32_t)(units * n_local);
+    P.n_local = n_local;
+    P.k = k;
+    P.granularity = ctx->cfg.granularity;
+    P.divisor = divisor;
+    P.round = round;
+    P.worker_base = worker_base;
+    P.c_block = (float)(1.0 / sqrt((double)(1ull << k)));
+    P.exact_range = ctx->cfg.range_mode == THC_RANGE_MINMAX ? 1u : 0u;
+    P.nblocks = (uint32_t)sz.nblocks;
+    P.const_slots = k < tile_log2 ? 1u << (tile_log2 - k) : 1u;
+    P.range_keys = keys;
+    P.agg_n = agg_n;
+    P.agg_chunk = 255u / ctx->cfg.granularity;
+    P.agg_acc_bits = ctx->acc_bits;
+    const size_t smem = (size_t)1024 + tile * 4 + tile / 4 + (size_t)P.const_slots * 16 + lut_bytes;
+    { const int rc = ensure_dynamic_smem(kern, smem); if (rc != THC_OK) return rc; }
+    TmaMaps maps;
+    if ((d >> 5) >= 256) {
+        for (uint32_t i = 0; i < n_local; ++i) {
+            int rc = THC_OK;
+            if (mode == kCompressBF16) rc = cached_map(ctx, &maps.in[i], in.p[i], 32u, d >> 5, 64u, 64u, 32u, true);
+            else if (mode == kCompressF32 || mode == kRangeF32) rc = cached_map(ctx, &maps.in[i], in.p[i], 32u, d >> 5, 128u, 256u);
+            if (rc != THC_OK) return rc;
+        }
+    }
+    const uint32_t ctas_per_sm = tile_log2 == 13u ? 4u : 2u;
+    const uint32_t resident = ((uint32_t)ctx->sm_count * ctas_per_sm) >> e;       // clusters (CTAs where e = 0)
+    const uint32_t grid = (P.tasks < resident ? P.tasks : resident) << e;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = 1u << e;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof cfg);
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3((unsigned)(tile / 64));
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = e != 0u ? 1 : 0;
+    void *args[] = {&maps, &P, const_cast<PtrArrayP *>(&in), const_cast<MutPtrArrayP *>(&out), const_cast<MutPtrArrayP *>(&rot),
+                    const_cast<PhiloxKeys *>(&ctx->keys)};
+    THC_CUDA(cudaLaunchKernelExC(&cfg, kern, args));
+    return THC_OK;
+}
+
+// Table space of a launch that quantises.
+static size_t quant_lut_bytes(const thc_ctx *ctx)
+{
+    return ctx->identity ? 0 : (size_t)(ctx->cfg.granularity + 1) * kLutEntryBytes;
+}
+
 // thc_prepare in exact-range mode (Algorithm 1's preliminary stage on the rotated coordinates):
 // one transform pass over all workers whose epilogue only takes the minimum and maximum, then
 // the keys become the (lo, hi) planes of `scales`.  This costs about as much as the transform
@@ -1425,9 +1124,9 @@ int thc_prepare_minmax(thc_ctx *ctx, const void *const *grads, uint32_t n, uint6
     if (workspace_bytes < sz.workspace_bytes) return THC_EWORKSPACE;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const uint32_t k = ctx->cfg.log2_block;
-    const bool two_pass = k > (uint32_t)kTileLog2;
+    const bool in_block = use_block_kernel(ctx, sz.d_pad * n);
     uint32_t *keys = static_cast<uint32_t *>(workspace);
-    if (two_pass) {
+    if (!in_block) {
         const PipePlan pl = plan_pipeline(ctx, sz.nblocks * n);
         keys = reinterpret_cast<uint32_t *>(static_cast<unsigned char *>(workspace) + ((uint64_t)pl.ring << k) * 4);
     }
@@ -1435,41 +1134,24 @@ int thc_prepare_minmax(thc_ctx *ctx, const void *const *grads, uint32_t n, uint6
     range_init_kernel<<<init_blocks, 256, 0, st>>>(keys, sz.nblocks);
     THC_CUDA(cudaGetLastError());
     int rc;
-    if (!two_pass) {
-        PtrArray in;
-        MutPtrArray out, rot;
-        memset(&in, 0, sizeof in);
-        memset(&out, 0, sizeof out);
-        memset(&rot, 0, sizeof rot);
-        for (uint32_t i = 0; i < n; ++i) {
-            in.p[i] = grads[i];
-            if (rotated != nullptr && rotated[i] != nullptr) {
-                if (!aligned16(rotated[i])) return THC_EINVAL;
-                rot.p[i] = rotated[i];
-            }
+    PtrArrayP pin;
+    MutPtrArrayP pout, prot;
+    memset(&pin, 0, sizeof pin);
+    memset(&pout, 0, sizeof pout);
+    memset(&prot, 0, sizeof prot);
+    for (uint32_t i = 0; i < n; ++i) {
+        pin.p[i] = grads[i];
+        if (rotated != nullptr && rotated[i] != nullptr) {
+            if (!aligned16(rotated[i])) return THC_EINVAL;
+            prot.p[i] = rotated[i];
         }
-        out.p[0] = keys;
-        TileGeom g = base_geom(ctx, sz, d, round);
-        geom_pass_a(g);
-        const uint64_t tiles = (sz.d_pad + kTileElems - 1) / kTileElems;
-        rc = launch_tile(ctx, pick_tile_kernel<kLoadGradF32, kStoreRange>(4, true), g, tiles, n, in, out, rot,
-                         scales, st);
-    } else {
-        PtrArrayP pin;
-        MutPtrArrayP pout, prot;
-        memset(&pin, 0, sizeof pin);
-        memset(&pout, 0, sizeof pout);
-        memset(&prot, 0, sizeof prot);
-        for (uint32_t i = 0; i < n; ++i) {
-            pin.p[i] = grads[i];
-            if (rotated != nullptr && rotated[i] != nullptr) {
-                if (!aligned16(rotated[i])) return THC_EINVAL;
-                prot.p[i] = rotated[i];
-            }
-        }
+    }
+    if (in_block)
+        rc = launch_block(ctx, block_kernel(kRangeF32, 4, true, ctx->cfg.log2_block), kRangeF32, 0, sz, d, n, 0, round, 1, scales, pin, pout,
+                          prot, st, keys);
+    else
         rc = launch_pipeline(ctx, pick_pipe_kernel<kRangeF32>(4, true, k), true, sz, d, n, 0, round,
                              1, scales, workspace, pin, pout, prot, st);
-    }
     if (rc != THC_OK) return rc;
     range_final_kernel<<<init_blocks, 256, 0, st>>>(keys, sz.nblocks, scales, ctx->dev);
     THC_CUDA(cudaGetLastError());
@@ -1489,14 +1171,13 @@ int thc_compress(thc_ctx *ctx, const void *const *grads, uint32_t n_local, uint3
     if (scales == nullptr) return THC_EINVAL;
     if ((uint64_t)worker_base + n_local > 0xFFFFFFFFull) return THC_EINVAL;
     const uint32_t k = ctx->cfg.log2_block;
-    const bool two_pass = k > (uint32_t)kTileLog2;
-    if (two_pass) {
+    if (k > (uint32_t)kChunkLog2) {
         if (workspace == nullptr || !aligned16(workspace)) return THC_EINVAL;
         if (workspace_bytes < sz.workspace_bytes) return THC_EWORKSPACE;
     }
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    PtrArray in;
-    MutPtrArray out, rot;
+    PtrArrayP in;
+    MutPtrArrayP out, rot;
     memset(&in, 0, sizeof in);
     memset(&out, 0, sizeof out);
     memset(&rot, 0, sizeof rot);
@@ -1508,25 +1189,18 @@ int thc_compress(thc_ctx *ctx, const void *const *grads, uint32_t n_local, uint3
             rot.p[i] = rotated[i];
         }
     }
-    TileGeom g = base_geom(ctx, sz, d, round);
-    g.worker_base = worker_base;
     const bool bf16 = ctx->cfg.in_dtype == THC_BF16;
-    const uint64_t tiles = (sz.d_pad + kTileElems - 1) / kTileElems;
-    geom_pass_a(g);
-    if (!two_pass) {
-        tile_kernel_t kern = bf16 ? pick_tile_kernel<kLoadGradBF16, kStoreQuant>(ctx->cfg.bits, ctx->identity)
-                                  : pick_tile_kernel<kLoadGradF32, kStoreQuant>(ctx->cfg.bits, ctx->identity);
-        return launch_tile(ctx, kern, g, tiles, n_local, in, out, rot, scales, st);
+    if (use_block_kernel(ctx, sz.d_pad * n_local)) {
+        const void *kern = bf16 ? block_kernel(kCompressBF16, ctx->cfg.bits, ctx->identity, ctx->cfg.log2_block)
+                                   : block_kernel(kCompressF32, ctx->cfg.bits, ctx->identity, ctx->cfg.log2_block);
+        return launch_block(ctx, kern, bf16 ? kCompressBF16 : kCompressF32, quant_lut_bytes(ctx), sz, d, n_local, worker_base,
+                            round, 1, scales, in, out, rot, st);
     }
-    PtrArrayP pin;
-    MutPtrArrayP pout, prot;
-    memcpy(&pin, &in, sizeof pin);
-    memcpy(&pout, &out, sizeof pout);
-    memcpy(&prot, &rot, sizeof prot);
+    ctx->pipeline_next = false;
     pipe_kernel_t kern = bf16 ? pick_pipe_kernel<kCompressBF16>(ctx->cfg.bits, ctx->identity, k)
                               : pick_pipe_kernel<kCompressF32>(ctx->cfg.bits, ctx->identity, k);
     return launch_pipeline(ctx, kern, !bf16, sz, d, n_local, worker_base, round, 1, scales, workspace,
-                           pin, pout, prot, st, nullptr, bf16);
+                           in, out, rot, st, nullptr, bf16);
 }
 
 // Scales and compress in one launch (see thc.h).  Falls back to the two separate calls where
@@ -1580,36 +1254,27 @@ int thc_decompress(thc_ctx *ctx, const void *sum, uint32_t divisor, uint64_t d, 
     if (sum == nullptr || outp == nullptr || scales == nullptr || divisor == 0) return THC_EINVAL;
     if (!aligned16(sum) || !aligned16(outp)) return THC_EINVAL;
     const uint32_t k = ctx->cfg.log2_block;
-    const bool two_pass = k > (uint32_t)kTileLog2;
-    if (two_pass) {
+    if (k > (uint32_t)kChunkLog2) {
         if (workspace == nullptr || !aligned16(workspace)) return THC_EINVAL;
         if (workspace_bytes < pipeline_workspace_need(ctx, sz.nblocks, sz.nblocks)) return THC_EWORKSPACE;
     }
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    PtrArray in;
-    MutPtrArray out, rot;
-    memset(&in, 0, sizeof in);
-    memset(&out, 0, sizeof out);
-    memset(&rot, 0, sizeof rot);
-    in.p[0] = sum;
-    out.p[0] = outp;
-    TileGeom g = base_geom(ctx, sz, d, round);
-    g.divisor = divisor;
-    const uint64_t tiles = (sz.d_pad + kTileElems - 1) / kTileElems;
-    geom_pass_a(g);
     const uint32_t w = ctx->acc_bits;
-    tile_kernel_t k1;
-    if (!two_pass) {
-        k1 = w == 8 ? pick_tile_kernel<kLoadSum8, kStoreOut>(4, true)
-           : w == 16 ? pick_tile_kernel<kLoadSum16, kStoreOut>(4, true)
-                     : pick_tile_kernel<kLoadSum32, kStoreOut>(4, true);
-        return launch_tile(ctx, k1, g, tiles, 1, in, out, rot, scales, st);
-    }
     PtrArrayP pin;
     MutPtrArrayP pout, prot;
-    memcpy(&pin, &in, sizeof pin);
-    memcpy(&pout, &out, sizeof pout);
-    memcpy(&prot, &rot, sizeof prot);
+    memset(&pin, 0, sizeof pin);
+    memset(&pout, 0, sizeof pout);
+    memset(&prot, 0, sizeof prot);
+    pin.p[0] = sum;
+    pout.p[0] = outp;
+    if (use_block_kernel(ctx, sz.d_pad)) {
+        const void *kern = w == 8 ? block_kernel(kDecompress8, 4, true, ctx->cfg.log2_block)
+                            : w == 16 ? block_kernel(kDecompress16, 4, true, ctx->cfg.log2_block)
+                                      : block_kernel(kDecompress32, 4, true, ctx->cfg.log2_block);
+        return launch_block(ctx, kern, w == 8 ? kDecompress8 : w == 16 ? kDecompress16 : kDecompress32, 0, sz, d, 1, 0, round,
+                            divisor, scales, pin, pout, prot, st);
+    }
+    ctx->pipeline_next = false;
     pipe_kernel_t kern = w == 8 ? pick_pipe_kernel<kDecompress8>(4, true, k)
                        : w == 16 ? pick_pipe_kernel<kDecompress16>(4, true, k)
                                  : pick_pipe_kernel<kDecompress32>(4, true, k);
@@ -1634,8 +1299,8 @@ int thc_aggregate_decompress(thc_ctx *ctx, const void *const *packed, uint32_t n
     if (outp == nullptr || scales == nullptr || !aligned16(outp)) return THC_EINVAL;
     if (sum_or_null != nullptr && !aligned16(sum_or_null)) return THC_EINVAL;
     const uint32_t k = ctx->cfg.log2_block;
-    if (k <= (uint32_t)kTileLog2 || ctx->cfg.bits != 4 || ctx->cfg.granularity >= 128) {
-        // small blocks, and index widths without the byte-lane look-up (there the one launch is
+    if (ctx->cfg.bits != 4 || ctx->cfg.granularity >= 128 || sz.d_pad % 32 != 0) {
+        // index widths without the byte-lane look-up (there the one launch is
         // slower than the two): the two calls; the sums go to the caller's buffer or to the workspace
         // (without a buffer the sums take the end of the workspace; thc_decompress checks that what
         // is left in front of them is enough for it)
@@ -1651,8 +1316,14 @@ int thc_aggregate_decompress(thc_ctx *ctx, const void *const *packed, uint32_t n
         if ((rc = thc_aggregate(ctx, packed, n, d, sum, stream)) != THC_OK) return rc;
         return thc_decompress(ctx, sum, n, d, round, scales, outp, workspace, ws_for_decompress, stream);
     }
-    if (workspace == nullptr || !aligned16(workspace)) return THC_EINVAL;
-    if (workspace_bytes < pipeline_workspace_need(ctx, sz.nblocks, sz.nblocks)) return THC_EWORKSPACE;
+    if (k > (uint32_t)kChunkLog2) {
+        if (workspace == nullptr || !aligned16(workspace)) return THC_EINVAL;
+        if (workspace_bytes < pipeline_workspace_need(ctx, sz.nblocks, sz.nblocks)) return THC_EWORKSPACE;
+    } else if (sum_or_null == nullptr) {
+        // needed by configurations that run the two calls: the same rule for all
+        if (workspace == nullptr || !aligned16(workspace)) return THC_EINVAL;
+        if (workspace_bytes < round_up(sz.sum_bytes, 256)) return THC_EWORKSPACE;
+    }
     PtrArrayP pin;
     MutPtrArrayP pout, prot;
     memset(&pin, 0, sizeof pin);
@@ -1661,6 +1332,9 @@ int thc_aggregate_decompress(thc_ctx *ctx, const void *const *packed, uint32_t n
     for (uint32_t i = 0; i < n; ++i) pin.p[i] = packed[i];
     pout.p[0] = outp;
     pout.p[1] = sum_or_null;
+    if (use_block_kernel(ctx, sz.d_pad))
+        return launch_block(ctx, block_kernel(kAggDecompress, 4, true, ctx->cfg.log2_block), kAggDecompress, 0, sz, d, 1, 0, round, n, scales,
+                            pin, pout, prot, static_cast<cudaStream_t>(stream), nullptr, n);
     pipe_kernel_t kern = pick_pipe_kernel<kAggDecompress>(ctx->cfg.bits, true, k);
     return launch_pipeline(ctx, kern, false, sz, d, 1, 0, round, n, scales, workspace, pin, pout, prot,
                            static_cast<cudaStream_t>(stream), nullptr, false, n);
@@ -1804,38 +1478,26 @@ int thc_error_feedback(thc_ctx *ctx, const void *const *grads, const void *const
     if (scales == nullptr || workspace == nullptr || !aligned16(workspace)) return THC_EINVAL;
     if (workspace_bytes < sz.workspace_bytes) return THC_EWORKSPACE;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (ctx->cfg.log2_block > (uint32_t)kTileLog2) {
-        // one launch of the pipeline for all workers: indices in, x_i - RHT^-1(X_i) out
-        thc_sizes_t szn;
-        if ((rc = thc_sizes(ctx, d, n_local, &szn)) != THC_OK) return rc;
-        if (workspace_bytes < szn.workspace_bytes) return THC_EWORKSPACE;
-        PtrArrayP pin;
-        MutPtrArrayP pout, px;
-        memset(&pin, 0, sizeof pin);
-        memset(&pout, 0, sizeof pout);
-        memset(&px, 0, sizeof px);
-        for (uint32_t i = 0; i < n_local; ++i) {
-            pin.p[i] = packed[i];
-            pout.p[i] = ef[i];
-            px.p[i] = const_cast<void *>(grads[i]);
-        }
-        pipe_kernel_t kern = pick_pipe_kernel<kErrorFeedback>(ctx->cfg.bits, true, ctx->cfg.log2_block);
-        return launch_pipeline(ctx, kern, false, szn, d, n_local, 0, round, 1, scales, workspace, pin, pout, px, st);
-    }
-    const uint64_t ring_bytes = sz.workspace_bytes - round_up(sz.sum_bytes, 256);
-    void *values = static_cast<unsigned char *>(workspace) + ring_bytes;
-    uint64_t blocks = (d / 4 + kThreads - 1) / kThreads;
-    const uint64_t cap = (uint64_t)ctx->sm_count * 16;
-    if (blocks > cap) blocks = cap;
-    if (blocks == 0) blocks = 1;
+    // one launch for all workers: indices in, x_i - RHT^-1(X_i) out
+    thc_sizes_t szn;
+    if ((rc = thc_sizes(ctx, d, n_local, &szn)) != THC_OK) return rc;
+    if (ctx->cfg.log2_block > (uint32_t)kChunkLog2 && workspace_bytes < szn.workspace_bytes) return THC_EWORKSPACE;
+    PtrArrayP pin;
+    MutPtrArrayP pout, px;
+    memset(&pin, 0, sizeof pin);
+    memset(&pout, 0, sizeof pout);
+    memset(&px, 0, sizeof px);
     for (uint32_t i = 0; i < n_local; ++i) {
-        if ((rc = thc_aggregate(ctx, &packed[i], 1, d, values, stream)) != THC_OK) return rc;
-        if ((rc = thc_decompress(ctx, values, 1, d, round, scales, ef[i], workspace, ring_bytes, stream)) != THC_OK)
-            return rc;
-        ef_subtract_kernel<<<(unsigned)blocks, kThreads, 0, st>>>(static_cast<const float *>(grads[i]), ef[i], d);
-        THC_CUDA(cudaGetLastError());
+        pin.p[i] = packed[i];
+        pout.p[i] = ef[i];
+        px.p[i] = const_cast<void *>(grads[i]);
     }
-    return THC_OK;
+    const uint32_t bits = ctx->cfg.bits;
+    if (use_block_kernel(ctx, sz.d_pad * n_local))
+        return launch_block(ctx, block_kernel(kErrorFeedback, bits, true, ctx->cfg.log2_block), kErrorFeedback,
+                            ((size_t)4 << bits) * (bits <= 4 ? 32 : 8), szn, d, n_local, 0, round, 1, scales, pin, pout, px, st);
+    pipe_kernel_t kern = pick_pipe_kernel<kErrorFeedback>(bits, true, ctx->cfg.log2_block);
+    return launch_pipeline(ctx, kern, false, szn, d, n_local, 0, round, 1, scales, workspace, pin, pout, px, st);
 }
 
 int thc_accumulate_error(thc_ctx *ctx, float *const *grads, const float *const *ef, uint32_t n_local,
@@ -1866,6 +1528,7 @@ int thc_debug_skip_tasks(thc_ctx *ctx, uint32_t count)
     THC_CUDA(cudaDeviceSynchronize());
     PipeCounters *pc = reinterpret_cast<PipeCounters *>(ctx->dev->counters);
     THC_CUDA(cudaMemcpy(&pc->head, &count, sizeof count, cudaMemcpyHostToDevice));
+    ctx->pipeline_next = true;
     return THC_OK;
 }
 

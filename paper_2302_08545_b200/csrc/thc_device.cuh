@@ -12,13 +12,12 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "../../include/thc.h"
+
 namespace thc {
 
-constexpr int kTileLog2 = 14;                  // a CTA transforms 2^14 coordinates at a time
-constexpr int kTileElems = 1 << kTileLog2;
-constexpr int kTileChunks = kTileElems / 4;    // 16-byte chunks
+constexpr int kChunkLog2 = 14;                 // coordinates whose squares one CTA sums (prepare)
 constexpr int kThreads = 256;
-constexpr int kSignWordsMax = 1024;            // sign words a tile can need
 
 // Lives in the context's device block.
 struct DeviceBlock {
@@ -161,56 +160,6 @@ __device__ __forceinline__ float4 flip4(float4 v, uint32_t bits)
     return v;
 }
 
-// ------------------------------------------------------------------- shared-memory tile
-// The tile holds 4096 chunks.  Chunk c is stored at c ^ ((c >> 4) & 7): with this XOR every
-// access pattern below (consecutive chunks per lane, or one chunk per lane at any
-// power-of-two stride) touches eight distinct 16-byte bank groups per quarter warp.
-__device__ __forceinline__ int swz(int c) { return c ^ ((c >> 4) & 7); }
-
-// Butterfly stages on chunk-index bits [sp, sp+E) of the tile, ascending.  Each thread owns
-// whole groups of 2^E chunks, so the update is in place; callers separate rounds by a
-// block barrier.
-template <int E>
-__device__ __forceinline__ void fwht_round(float4 *tile, int sp, int tid)
-{
-    constexpr int N = 1 << E;
-    constexpr int kGroups = kTileChunks >> E;
-#pragma unroll 1
-    for (int G = tid; G < kGroups; G += kThreads) {
-        const int low = G & ((1 << sp) - 1);
-        const int base = ((G >> sp) << (sp + E)) | low;
-        float4 v[N];
-#pragma unroll
-        for (int m = 0; m < N; ++m) v[m] = tile[swz(base + (m << sp))];
-#pragma unroll
-        for (int t = 0; t < E; ++t) {
-#pragma unroll
-            for (int m = 0; m < N; ++m) {
-                if (!(m & (1 << t))) butterfly(v[m], v[m | (1 << t)]);
-            }
-        }
-#pragma unroll
-        for (int m = 0; m < N; ++m) tile[swz(base + (m << sp))] = v[m];
-    }
-}
-
-// All stages on chunk bits [lo, hi), in rounds of at most four bits.
-__device__ __forceinline__ void fwht_rounds(float4 *tile, int lo, int hi, int tid)
-{
-    int sp = lo;
-    while (sp < hi) {
-        const int e = min(4, hi - sp);
-        switch (e) {
-        case 4: fwht_round<4>(tile, sp, tid); break;
-        case 3: fwht_round<3>(tile, sp, tid); break;
-        case 2: fwht_round<2>(tile, sp, tid); break;
-        default: fwht_round<1>(tile, sp, tid); break;
-        }
-        sp += e;
-        __syncthreads();
-    }
-}
-
 // --------------------------------------------------------------------------- quantiser
 // The quantiser's table in shared memory, indexed by f = floor(u g): what the rounding rule
 // needs about the table interval [T[z0], T[z0+1]] that holds f.  Consecutive entries are 128
@@ -248,27 +197,29 @@ __device__ __forceinline__ uint32_t lut_lane_addr(const unsigned char *lut, int 
     return (uint32_t)__cvta_generic_to_shared(lut) + copy - 0x4B000000u * (uint32_t)kLutEntryBytes;
 }
 
-// Stochastic quantisation of eight consecutive rotated coordinates to table indices
+// Stochastic quantisation of four consecutive rotated coordinates to table indices
 // (Algorithm 2, worker lines; Section 4.1 for the rounding rule):
 //   u = sat(fma(r, kappa, offset))          position in [m, M] on the unit interval, truncated
 //   f = floor(u * g)                         (one round-down fma onto 2^23; exact)
 //   z0 = index of the table value at or below u*g, delta = fma(u, g, -T[z0])
 //   up iff u16 < RN(2^16 delta / gap)        (one fma onto 2^23, integer compare)
 // kappa = 1/(2M) and offset = 1/2; kappa = offset = 0 encodes a degenerate block (index 0).
-// `lut_addr` comes from lut_lane_addr (unused for the identity table).  Returns the indices
-// packed BITS apiece, coordinate 0 in the low bits.
+// w0, w1: the four 16-bit variates.  `lut_addr` comes from lut_lane_addr (unused for the identity
+// table).  Returns the indices packed BITS apiece, coordinate 0 in the low bits: the compare is the
+// carry of an addition, and a multiply-add with carry shifts the indices so far, appends z0 and
+// adds it (0.7 instructions per coordinate less than compare and select).  With the 8-byte entries
+// the whole second word is added in, so the bits above 4 BITS are not defined (join_units cuts
+// them off).
 template <int BITS, bool IDENTITY>
-__device__ __forceinline__ uint64_t quantize8(const float (&r)[8], float kappa, float offset,
-                                              float gf, uint4 rnd, uint32_t lut_addr)
+__device__ __forceinline__ uint32_t quantize4(float r0, float r1, float r2, float r3, float kappa, float offset,
+                                              float gf, uint32_t w0, uint32_t w1, uint32_t lut_addr)
 {
     constexpr bool kLut8 = LutKind<BITS, IDENTITY>::k8;
-    const uint32_t words[4] = {rnd.x, rnd.y, rnd.z, rnd.w};
-    // Indices are accumulated as z * 2^(BITS*slot) with multiply-adds into two 32-bit halves
-    // (coordinates 0-3 and 4-7).  With the 8-byte entries the whole second word is multiplied
-    // in: what its upper half leaves above bit 16 is cut off at the end (4 BITS <= 16 valid bits).
-    uint32_t acc[2] = {0u, 0u};
+    const float r[4] = {r0, r1, r2, r3};
+    const uint32_t words[2] = {w0, w1};
+    uint32_t acc = 0u;
 #pragma unroll
-    for (int e = 0; e < 8; ++e) {
+    for (int e = 3; e >= 0; --e) {
         float u;
         asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(u) : "f"(r[e]), "f"(kappa), "f"(offset));
         const float t = __fmaf_rd(u, gf, 8388608.0f);          // 2^23 + floor(u * g)
@@ -296,15 +247,105 @@ __device__ __forceinline__ uint64_t quantize8(const float (&r)[8], float kappa, 
             tau = fmaf(delta, __uint_as_float(y), 8388608.0f);
             zw = z;
         }
-        const int h = e >> 2;
-        const uint32_t weight = 1u << (BITS * (e & 3));
-        acc[h] = zw * weight + acc[h];
-        if (ub < __float_as_uint(tau)) acc[h] += weight;
+        // carry out of tau + ~ub: ub < tau
+        asm("{\n\t.reg .u32 t;\n\tadd.cc.u32 t, %1, %2;\n\tmadc.lo.u32 %0, %0, %4, %3;\n\t}"
+            : "+r"(acc) : "r"(__float_as_uint(tau)), "r"(~ub), "r"(zw), "n"(1 << BITS));
     }
-    if constexpr (BITS == 8) return (uint64_t)acc[0] | ((uint64_t)acc[1] << 32);
-    if constexpr (BITS == 4) return (uint64_t)__byte_perm(acc[0], acc[1], 0x5410);
-    constexpr uint32_t mask = (1u << (4 * BITS)) - 1u;
-    return (uint64_t)((acc[0] & mask) | ((acc[1] & mask) << (4 * BITS)));
+    return acc;
+}
+
+// Two groups of four indices as one unit of eight, coordinate 0 in the low bits.
+template <int BITS>
+__device__ __forceinline__ uint64_t join_units(uint32_t lo, uint32_t hi)
+{
+    if constexpr (BITS == 8) {
+        return (uint64_t)lo | ((uint64_t)hi << 32);
+    } else if constexpr (BITS == 4) {
+        return (uint64_t)__byte_perm(lo, hi, 0x5410);
+    } else {
+        constexpr uint32_t mask = (1u << (4 * BITS)) - 1u;
+        return (uint64_t)((lo & mask) | ((hi & mask) << (4 * BITS)));
+    }
+}
+
+// Eight consecutive coordinates (see quantize4).
+template <int BITS, bool IDENTITY>
+__device__ __forceinline__ uint64_t quantize8(const float (&r)[8], float kappa, float offset,
+                                              float gf, uint4 rnd, uint32_t lut_addr)
+{
+    const uint32_t lo = quantize4<BITS, IDENTITY>(r[0], r[1], r[2], r[3], kappa, offset, gf, rnd.x, rnd.y, lut_addr);
+    const uint32_t hi = quantize4<BITS, IDENTITY>(r[4], r[5], r[6], r[7], kappa, offset, gf, rnd.z, rnd.w, lut_addr);
+    return join_units<BITS>(lo, hi);
+}
+
+// Eight 3-bit indices (24 bits, coordinate 0 in the low bits) go to bytes 3 (j/8) .. +2.
+__device__ __forceinline__ void store_packed3(unsigned char *pk, uint64_t j, uint32_t z)
+{
+    unsigned char *p = pk + 3 * (j >> 3);
+    p[0] = (unsigned char)z;
+    p[1] = (unsigned char)(z >> 8);
+    p[2] = (unsigned char)(z >> 16);
+}
+
+// The eight indices of coordinates j .. j+7 (j a multiple of 8) to their place in the stream.
+template <int BITS>
+__device__ __forceinline__ void store_unit(unsigned char *pk, uint64_t j, uint64_t z)
+{
+    if constexpr (BITS == 8) *reinterpret_cast<uint2 *>(pk + j) = make_uint2((uint32_t)z, (uint32_t)(z >> 32));
+    else if constexpr (BITS == 4) *reinterpret_cast<uint32_t *>(pk + j / 2) = (uint32_t)z;
+    else if constexpr (BITS == 3) store_packed3(pk, j, (uint32_t)z);
+    else if constexpr (BITS == 2) *reinterpret_cast<uint16_t *>(pk + j / 4) = (uint16_t)z;
+    else pk[j / 8] = (unsigned char)z;
+}
+
+// ------------------------------------------------------------------------ small helpers
+__device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel)
+{
+    uint32_t d;
+    asm("prmt.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(sel));
+    return d;
+}
+
+__device__ __forceinline__ float4 load_f32x4_masked(const float *x, uint64_t j, uint64_t d)
+{
+    if (j + 4 <= d) return __ldg(reinterpret_cast<const float4 *>(x + j));
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (j + 0 < d) v.x = __ldg(x + j + 0);
+    if (j + 1 < d) v.y = __ldg(x + j + 1);
+    if (j + 2 < d) v.z = __ldg(x + j + 2);
+    if (j + 3 < d) v.w = __ldg(x + j + 3);
+    return v;
+}
+
+// Geometry of a tile: 2^row_log2 rows, row_stride coordinates apart, of 2^col_log2 consecutive ones.
+struct TileGeom {
+    uint64_t row_stride;
+    uint32_t row_log2, col_log2;
+    uint32_t round;
+};
+
+// Sign words of every row of the tile, 32 coordinates per word.
+__device__ __forceinline__ void fill_sign_words(uint32_t *sw, const TileGeom &g, uint64_t base,
+                                                const PhiloxKeys &keys, int tid,
+                                                int nthreads = kThreads)
+{
+    const int cols = 1 << g.col_log2;
+    const int words_per_row = max(1, cols >> 5);
+    const int calls_per_row = max(1, cols >> 7);
+    const int rows = 1 << g.row_log2;
+    const int words_per_call = min(4, words_per_row);
+    for (int q = tid; q < rows * calls_per_row; q += nthreads) {
+        const int row = q / calls_per_row;
+        const int cr = q - row * calls_per_row;
+        const uint64_t j0 = base + (uint64_t)row * g.row_stride + (uint64_t)cr * 128;
+        const uint4 ph = sign_call(j0, g.round, keys);
+        const int first = (int)((j0 >> 5) & 3);
+        for (int wi = 0; wi < words_per_call; ++wi) {
+            const int src = first + wi;
+            const uint32_t w = src == 0 ? ph.x : src == 1 ? ph.y : src == 2 ? ph.z : ph.w;
+            sw[row * words_per_row + cr * 4 + wi] = w;
+        }
+    }
 }
 
 }  // namespace thc

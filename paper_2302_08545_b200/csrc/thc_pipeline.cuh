@@ -359,7 +359,8 @@ __device__ __forceinline__ float2 block_constants(BlockRange b, uint32_t g, uint
 }
 
 // ------------------------------------------------------------------ in-place tile rounds
-// Butterfly stages on chunk-index bits [sp, sp+E) of a 2048-chunk tile (see fwht_round).
+// Butterfly stages on chunk-index bits [sp, sp+E) of a 2048-chunk tile: each thread owns whole groups of 2^E chunks, so the update
+// is in place; callers separate rounds by a block barrier.
 template <int E>
 __device__ __forceinline__ void p_round(float4 *tile, int sp, int tid, int mask)
 {
@@ -781,16 +782,7 @@ __device__ __forceinline__ void epilogue_unit(const float4 &va, const float4 &vb
         const float r[8] = {ra.x, ra.y, ra.z, ra.w, rb.x, rb.y, rb.z, rb.w};
         const uint4 rnd = round_call(j, ep.worker, ep.round, keys);
         const uint64_t z = quantize8<BITS, IDENTITY>(r, ep.kappa, ep.half_g, ep.gf, rnd, ep.lut);
-        if constexpr (BITS == 8)
-            *reinterpret_cast<uint2 *>(ep.packed + j) = make_uint2((uint32_t)z, (uint32_t)(z >> 32));
-        else if constexpr (BITS == 4)
-            *reinterpret_cast<uint32_t *>(ep.packed + j / 2) = (uint32_t)z;
-        else if constexpr (BITS == 3)
-            store_packed3(ep.packed, j, (uint32_t)z);
-        else if constexpr (BITS == 2)
-            *reinterpret_cast<uint16_t *>(ep.packed + j / 4) = (uint16_t)z;
-        else
-            ep.packed[j / 8] = (unsigned char)z;
+        store_unit<BITS>(ep.packed, j, z);
     } else {
         if (j >= ep.d) return;
         const uint32_t bits = ep.sw[row * ep.words_per_row + (uu >> 2)] >> (uint32_t)(j & 31);

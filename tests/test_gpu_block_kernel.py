@@ -1,0 +1,48 @@
+"""Blocks held in shared memory (thc_block.cu) at the edges of their tiles: one coordinate more or
+less than a tile, several tiles per CTA, clusters (2^15, 2^16) and the size from which 2^16 blocks
+take the two-pass pipeline, for fp32 and bf16 gradients: every step against the oracle."""
+import numpy as np
+import pytest
+
+from oracle import oracle as O
+from paper_2302_08545_b200 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("k,d,n,dtype,bits", [
+    (3, 8193, 2, "f32", 4), (5, 16_384 - 31, 2, "bf16", 3), (9, 8191, 3, "f32", 2), (11, 8192 * 3 + 1, 2, "bf16", 4),
+    (12, 5_000_001, 2, "f32", 4), (13, 8192, 1, "f32", 8), (13, 5_000_000, 2, "bf16", 1), (14, 16_385, 2, "f32", 4),
+    (14, 5_100_003, 2, "f32", 4), (15, 32_769, 3, "bf16", 4), (15, 10_000_019, 1, "f32", 2), (16, 65_535, 2, "f32", 4),
+    (16, 1 << 22, 1, "f32", 4), (16, (1 << 22) + 1, 1, "f32", 4), (16, 65_537, 20, "bf16", 4),
+])
+def test_edges_of_tiles_and_clusters(k, d, n, dtype, bits):
+    import torch
+    from paper_2302_08545_b200 import runner
+    g = {1: 5, 2: 3, 3: 12, 4: 30, 8: 255}[bits]
+    table = {1: (0, 5), 3: (0, 2, 4, 5, 6, 7, 9, 12)}.get(bits) or W.TABLES[(bits, g)]
+    w = W.Workload("cfg4_x" if dtype == "bf16" else "plain", n=n, d=d, log2_block=k, bits=bits, granularity=g,
+                   table=tuple(table), in_dtype=dtype, data_seed=k)
+    c = O.Config(bits=bits, granularity=g, table=tuple(table), t_p=w.t_p, log2_block=k, seed=w.seed)
+    ctx = runner.context_for(w)
+    r = runner.Round(ctx, n, d, dtype)
+    W.fill_torch(w, r.grads)
+    r.run(5)
+    tail = torch.zeros_like(r.out)
+    ctx.aggregate_decompress(r.packed, d, 5, r.scales, tail, r.workspace)
+    ef = [torch.zeros(d, dtype=torch.float32, device=r.device) for _ in range(n)]
+    if dtype == "f32":
+        ctx.error_feedback(r.grads, r.packed, d, 5, r.scales, ef, r.workspace)
+    torch.cuda.synchronize()
+    assert ctx.status() == 0
+    x = np.stack([t.float().cpu().numpy() for t in r.grads])
+    scl = r.scales.cpu().numpy()
+    ref = O.thc_round(x, c, 5, scl=scl)
+    assert np.array_equal(np.stack([p.cpu().numpy() for p in r.packed]), ref["packed"])
+    assert np.array_equal(r.sum_numpy(), ref["sum"])
+    assert np.array_equal(r.out.cpu().numpy().view(np.uint32), ref["out"].view(np.uint32))
+    assert torch.equal(tail.view(torch.int32), r.out.view(torch.int32))
+    if dtype == "f32":
+        z = O.unpack(r.packed[n - 1].cpu().numpy(), r.sz.d_pad, bits)
+        e = O.error_feedback(x[n - 1], z, scl, c, 5)
+        assert np.array_equal(ef[n - 1].cpu().numpy().view(np.uint32), e.view(np.uint32))
