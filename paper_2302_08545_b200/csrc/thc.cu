@@ -258,58 +258,187 @@ accumulate_kernel(float *__restrict__ x, const float *__restrict__ e, uint64_t d
 }
 
 // ------------------------------------------------------------------------------ prepare
-// Partial sums of squares in fp64: one CTA per (chunk of 2^chunk_log2 coordinates, worker).
+// Sums of squares in fp64.  HBM-bound: 16 bytes per load, all of a thread's loads for a worker in
+// flight together (4 x 2^26 fp32 coordinates: 5.8 -> 6.3 TB/s), and one launch where the second one
+// of a small call cost as much as the first.
+
+// 16 bytes of a gradient: 4 fp32 or 8 bf16 coordinates from j on, zero behind d.
+template <bool BF16>
+__device__ __forceinline__ uint4 load_unit(const void *x, uint64_t j, uint64_t d)
+{
+    constexpr int kPer = BF16 ? 8 : 4;
+    uint4 q = make_uint4(0u, 0u, 0u, 0u);
+    if (j + kPer <= d) {
+        const char *p = static_cast<const char *>(x) + j * (16 / kPer);
+        asm("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(q.x), "=r"(q.y), "=r"(q.z), "=r"(q.w) : "l"(p));
+    } else if (j < d) {
+        uint32_t w[4] = {0u, 0u, 0u, 0u};
+        for (int e = 0; e < kPer; ++e) {
+            if (j + e >= d) break;
+            if (BF16) w[e >> 1] |= (uint32_t)__ldg(static_cast<const uint16_t *>(x) + j + e) << ((e & 1) * 16);
+            else w[e & 3] = __ldg(static_cast<const uint32_t *>(x) + j + e);
+        }
+        q = make_uint4(w[0], w[1], w[2], w[3]);
+    }
+    return q;
+}
+
+template <bool BF16>
+__device__ __forceinline__ double add_squares(double s, uint4 q)
+{
+    const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        if (BF16) {
+            const double lo = (double)__uint_as_float(w[e] << 16), hi = (double)__uint_as_float(w[e] & 0xFFFF0000u);
+            s = fma(lo, lo, s);
+            s = fma(hi, hi, s);
+        } else {
+            const double v = (double)__uint_as_float(w[e]);
+            s = fma(v, v, s);
+        }
+    }
+    return s;
+}
+
+// M = t_p ell / sqrt(B) to scales[blk], and the status bits.
+__device__ __forceinline__ void store_scale(double ell, double t_p, uint32_t k, uint64_t blk, float *scales, DeviceBlock *dev)
+{
+    float M = (float)(t_p * ell / sqrt((double)((uint64_t)1 << k)));
+    uint32_t flags = 0;
+    if (!isfinite(M)) { M = 0.0f; flags |= THC_STATUS_NONFINITE; }
+    if (M == 0.0f) flags |= THC_STATUS_ZERO_BLOCK;
+    scales[blk] = M;
+    if (flags) atomicOr(&dev->status, flags);
+}
+
+__device__ __forceinline__ double max_norm(double a, double b) { return (b > a || b != b) ? b : a; }   // a NaN norm sticks
+
+// Blocks of up to 2^12: a CTA takes 2^12 coordinates of all workers and writes the scales of their blocks.
+// A warp takes 512 consecutive coordinates, in slabs of 32 loads; blocks of 2^9 and more are whole
+// warps (one reduction per worker and warp), smaller ones two slabs, one slab or 2^g lanes of it.
+constexpr int kSmallPrepLog2 = 12;
+template <bool BF16>
+__global__ void __launch_bounds__(kThreads)
+prepare_small_kernel(PtrArray in, uint32_t n, uint64_t d, uint64_t d_pad, uint32_t k, double t_p, float *__restrict__ scales,
+                     DeviceBlock *dev)
+{
+    constexpr uint32_t kPerLog2 = BF16 ? 3u : 2u;
+    constexpr int kSlabs = 1 << (9 - 5 - kPerLog2);
+    __shared__ double s_warp[THC_MAX_WORKERS][kThreads / 32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t g = min(k - kPerLog2, 5u);
+    const bool pairs = k == 6u + kPerLog2;             // a block is two slabs
+    const uint64_t j0 = ((uint64_t)blockIdx.x << kSmallPrepLog2) + 512u * warp + ((uint64_t)lane << kPerLog2);
+    double ell[kSlabs];
+#pragma unroll
+    for (int i = 0; i < kSlabs; ++i) ell[i] = 0.0;
+#pragma unroll 4
+    for (uint32_t w = 0; w < n; ++w) {
+        uint4 q[kSlabs];
+#pragma unroll
+        for (int i = 0; i < kSlabs; ++i) q[i] = load_unit<BF16>(in.p[w], j0 + ((uint64_t)i << (5 + kPerLog2)), d);
+        if (k >= 9u) {
+            double s = 0.0;
+#pragma unroll
+            for (int i = 0; i < kSlabs; ++i) s = add_squares<BF16>(s, q[i]);
+            for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, off);
+            if (lane == 0) s_warp[w][warp] = s;
+        } else {
+#pragma unroll
+            for (int i = 0; i < kSlabs; ++i) {
+                double s = add_squares<BF16>(0.0, q[i]);
+                if (pairs) {
+                    if (i & 1) continue;
+                    s = add_squares<BF16>(s, q[i + 1 < kSlabs ? i + 1 : i]);
+                }
+                for (uint32_t b = 0; b < g; ++b) s += __shfl_xor_sync(0xFFFFFFFFu, s, 1 << b);
+                ell[i] = max_norm(ell[i], sqrt(s));
+            }
+        }
+    }
+    if (k < 9u) {
+        if ((lane & ((1 << g) - 1)) != 0) return;
+#pragma unroll
+        for (int i = 0; i < kSlabs; ++i) {
+            const uint64_t j = j0 + ((uint64_t)i << (5 + kPerLog2));
+            if (j < d_pad && !(pairs && (i & 1))) store_scale(ell[i], t_p, k, j >> k, scales, dev);
+        }
+        return;
+    }
+    // a warp per block, the lanes share the workers
+    __syncthreads();
+    const int warps = 1 << (k - 9u);
+    if (warp >= (1 << (kSmallPrepLog2 - k))) return;
+    double m = 0.0;
+    for (uint32_t w = (uint32_t)lane; w < n; w += 32u) {
+        double s = 0.0;
+        for (int v = 0; v < warps; ++v) s += s_warp[w][warp * warps + v];
+        m = max_norm(m, sqrt(s));
+    }
+    for (int off = 16; off > 0; off >>= 1) m = max_norm(m, __shfl_xor_sync(0xFFFFFFFFu, m, off));
+    const uint64_t blk = ((uint64_t)blockIdx.x << (kSmallPrepLog2 - k)) + (uint32_t)warp;
+    if (lane == 0 && (blk << k) < d_pad) store_scale(m, t_p, k, blk, scales, dev);
+}
+
+// Larger blocks: partial sums of one (chunk of 2^chunk_log2 coordinates, worker) per CTA; with
+// `counters` the CTA that finishes the last chunk of an RHT block (over all workers) computes its scale
+// from the stored sums in a fixed order (atomicInc wraps, so the counters are zero again).
 template <bool BF16>
 __global__ void __launch_bounds__(kThreads)
 prepare_partial_kernel(PtrArray in, uint64_t d, uint32_t chunk_log2, uint64_t chunks_per_worker,
-                       double *__restrict__ partial)
+                       double *__restrict__ partial, uint32_t *counters, uint32_t chunks_per_block, double t_p, uint32_t k,
+                       float *__restrict__ scales, DeviceBlock *dev)
 {
+    constexpr uint32_t kPerLog2 = BF16 ? 3u : 2u;
     const uint64_t chunk = blockIdx.x;
     const uint32_t wl = blockIdx.y;
-    const uint64_t j0 = chunk << chunk_log2;
-    const int n4 = 1 << (chunk_log2 - 2);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint64_t j0 = (chunk << chunk_log2) + ((uint64_t)tid << kPerLog2);
+    const uint32_t units = 1u << (chunk_log2 - 8u - kPerLog2);           // per thread: a multiple of four
     double s = 0.0;
-    if (BF16) {
-        // eight bf16 (16 bytes) per load
-        const uint16_t *x = static_cast<const uint16_t *>(in.p[wl]);
-        for (int c = threadIdx.x; c < n4 / 2; c += kThreads) {
-            const uint64_t j = j0 + (uint64_t)c * 8;
-            if (j >= d) break;
-            uint32_t w[4] = {0u, 0u, 0u, 0u};
-            if (j + 8 <= d) {
-                const uint4 q = __ldg(reinterpret_cast<const uint4 *>(x + j));
-                w[0] = q.x; w[1] = q.y; w[2] = q.z; w[3] = q.w;
-            } else {
-                for (int e = 0; e < 8; ++e)
-                    if (j + e < d) w[e >> 1] |= (uint32_t)__ldg(x + j + e) << ((e & 1) * 16);
-            }
+#pragma unroll 1
+    for (uint32_t i = 0; i < units; i += 4) {
+        uint4 q[4];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const double lo = (double)__uint_as_float(w[q] << 16);
-                const double hi = (double)__uint_as_float(w[q] & 0xFFFF0000u);
-                s = fma(lo, lo, s);
-                s = fma(hi, hi, s);
-            }
-        }
-    } else {
-        for (int c = threadIdx.x; c < n4; c += kThreads) {
-            const uint64_t j = j0 + (uint64_t)c * 4;
-            if (j >= d) break;
-            const float4 v = load_f32x4_masked(static_cast<const float *>(in.p[wl]), j, d);
-            s = fma((double)v.x, (double)v.x, s);
-            s = fma((double)v.y, (double)v.y, s);
-            s = fma((double)v.z, (double)v.z, s);
-            s = fma((double)v.w, (double)v.w, s);
-        }
+        for (int e = 0; e < 4; ++e) q[e] = load_unit<BF16>(in.p[wl], j0 + ((uint64_t)(i + e) << (8 + kPerLog2)), d);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) s = add_squares<BF16>(s, q[e]);
     }
     __shared__ double red[kThreads / 32];
+    __shared__ uint32_t last;
     for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xFFFFFFFFu, s, off);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+    if (lane == 0) red[warp] = s;
     __syncthreads();
-    if (threadIdx.x == 0) {
+    const uint64_t blk = chunk / chunks_per_block;
+    if (tid == 0) {
         double t = 0.0;
         for (int w = 0; w < kThreads / 32; ++w) t += red[w];
-        partial[(uint64_t)wl * chunks_per_worker + chunk] = t;
+        __stcg(partial + (uint64_t)wl * chunks_per_worker + chunk, t);
+        last = 0u;
+        if (counters != nullptr) {
+            const uint32_t total = gridDim.y * chunks_per_block;
+            __threadfence();
+            last = atomicInc(counters + blk, total - 1u) == total - 1u;
+        }
+    }
+    __syncthreads();
+    if (!last) return;
+    // a warp per worker in turn
+    __threadfence();
+    double ell = 0.0;
+    for (uint32_t w = (uint32_t)warp; w < gridDim.y; w += kThreads / 32) {
+        const double *p = partial + (uint64_t)w * chunks_per_worker + blk * chunks_per_block;
+        double t = 0.0;
+        for (uint32_t c = (uint32_t)lane; c < chunks_per_block; c += 32u) t += __ldcg(p + c);
+        for (int off = 16; off > 0; off >>= 1) t += __shfl_xor_sync(0xFFFFFFFFu, t, off);
+        ell = max_norm(ell, sqrt(t));
+    }
+    if (lane == 0) red[warp] = ell;
+    __syncthreads();
+    if (tid == 0) {
+        for (int w = 1; w < kThreads / 32; ++w) ell = max_norm(ell, red[w]);
+        store_scale(ell, t_p, k, blk, scales, dev);
     }
 }
 
@@ -317,7 +446,7 @@ prepare_partial_kernel(PtrArray in, uint64_t d, uint32_t chunk_log2, uint64_t ch
 // per RHT block, eight workers at a time with four lanes per worker: a lane adds every fourth
 // partial sum of its worker (loads independent of each other), the four lanes are combined,
 // one square root per worker, then the maximum over workers.  The order is fixed, so the
-// result does not depend on timing.
+// result does not depend on timing.  For more blocks than there are counters.
 __global__ void __launch_bounds__(128)
 prepare_final_kernel(const double *__restrict__ partial, uint32_t n, uint64_t nblocks,
                      uint64_t chunks_per_block, uint64_t chunks_per_worker, double t_p, uint32_t k,
@@ -337,18 +466,12 @@ prepare_final_kernel(const double *__restrict__ partial, uint32_t n, uint64_t nb
         s += __shfl_xor_sync(0xFFFFFFFFu, s, 2);
         double norm = live ? sqrt(s) : 0.0;
         for (int off = 4; off < 32; off <<= 1) {
-            const double other = __shfl_xor_sync(0xFFFFFFFFu, norm, off);
-            if (other > norm || other != other) norm = other;      // a NaN norm sticks
+            norm = max_norm(norm, __shfl_xor_sync(0xFFFFFFFFu, norm, off));
         }
-        if (norm > ell || norm != norm) ell = norm;
+        ell = max_norm(ell, norm);
     }
     if (lane != 0) return;
-    float M = (float)(t_p * ell / sqrt((double)((uint64_t)1 << k)));
-    uint32_t flags = 0;
-    if (!isfinite(M)) { M = 0.0f; flags |= THC_STATUS_NONFINITE; }
-    if (M == 0.0f) flags |= THC_STATUS_ZERO_BLOCK;
-    scales[blk] = M;
-    if (flags) atomicOr(&dev->status, flags);
+    store_scale(ell, t_p, k, blk, scales, dev);
 }
 
 // Exact range (Algorithm 1's preliminary stage on the rotated coordinates): keys start at
@@ -752,23 +875,38 @@ int thc_prepare(thc_ctx *ctx, const void *const *grads, uint32_t n, uint64_t d, 
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const uint32_t k = ctx->cfg.log2_block;
     if (ctx->cfg.range_mode == THC_RANGE_MINMAX) return THC_EUNSUPPORTED;   // thc_prepare_minmax
-    const uint32_t chunk_log2 = k < (uint32_t)kChunkLog2 ? k : (uint32_t)kChunkLog2;
-    const uint64_t chunks_per_worker = sz.d_pad >> chunk_log2;
-    const uint64_t chunks_per_block = 1ull << (k - chunk_log2);
-    if (chunks_per_worker > 0x7FFFFFFFull) return THC_EUNSUPPORTED;
     PtrArray in;
     memset(&in, 0, sizeof in);
     for (uint32_t i = 0; i < n; ++i) in.p[i] = grads[i];
+    const double t_p = ctx->cfg.t_p;
+    const bool bf16 = ctx->cfg.in_dtype == THC_BF16;
+    if (k <= (uint32_t)kSmallPrepLog2) {
+        const uint64_t tiles = (sz.d_pad + (1u << kSmallPrepLog2) - 1) >> kSmallPrepLog2;
+        if (tiles > 0x7FFFFFFFull) return THC_EUNSUPPORTED;
+        if (bf16) prepare_small_kernel<true><<<(unsigned)tiles, kThreads, 0, st>>>(in, n, d, sz.d_pad, k, t_p, scales, ctx->dev);
+        else prepare_small_kernel<false><<<(unsigned)tiles, kThreads, 0, st>>>(in, n, d, sz.d_pad, k, t_p, scales, ctx->dev);
+        THC_CUDA(cudaGetLastError());
+        return THC_OK;
+    }
+    const uint32_t chunk_log2 = k < (uint32_t)kChunkLog2 ? k : (uint32_t)kChunkLog2;
+    const uint64_t chunks_per_worker = sz.d_pad >> chunk_log2;
+    const uint32_t chunks_per_block = 1u << (k - chunk_log2);
+    if (chunks_per_worker > 0x7FFFFFFFull) return THC_EUNSUPPORTED;
     double *partial = static_cast<double *>(workspace);
+    uint32_t *counters = sz.nblocks <= (uint64_t)kPrepCounters ? ctx->dev->prep_counters : nullptr;
     const dim3 grid((unsigned)chunks_per_worker, n);
-    if (ctx->cfg.in_dtype == THC_BF16)
-        prepare_partial_kernel<true><<<grid, kThreads, 0, st>>>(in, d, chunk_log2, chunks_per_worker, partial);
+    if (bf16)
+        prepare_partial_kernel<true><<<grid, kThreads, 0, st>>>(in, d, chunk_log2, chunks_per_worker, partial, counters,
+                                                                chunks_per_block, t_p, k, scales, ctx->dev);
     else
-        prepare_partial_kernel<false><<<grid, kThreads, 0, st>>>(in, d, chunk_log2, chunks_per_worker, partial);
+        prepare_partial_kernel<false><<<grid, kThreads, 0, st>>>(in, d, chunk_log2, chunks_per_worker, partial, counters,
+                                                                 chunks_per_block, t_p, k, scales, ctx->dev);
     THC_CUDA(cudaGetLastError());
-    prepare_final_kernel<<<(unsigned)((sz.nblocks + 3) / 4), 128, 0, st>>>(
-        partial, n, sz.nblocks, chunks_per_block, chunks_per_worker, ctx->cfg.t_p, k, scales, ctx->dev);
-    THC_CUDA(cudaGetLastError());
+    if (counters == nullptr) {
+        prepare_final_kernel<<<(unsigned)((sz.nblocks + 3) / 4), 128, 0, st>>>(
+            partial, n, sz.nblocks, chunks_per_block, chunks_per_worker, t_p, k, scales, ctx->dev);
+        THC_CUDA(cudaGetLastError());
+    }
     return THC_OK;
 }
 

@@ -19,11 +19,14 @@ namespace thc {
 constexpr int kChunkLog2 = 14;                 // coordinates whose squares one CTA sums (prepare)
 constexpr int kThreads = 256;
 
+constexpr int kPrepCounters = 4096;
+
 // Lives in the context's device block.
 struct DeviceBlock {
     uint32_t status;             // THC_STATUS_* bits
     uint32_t pad_[31];
     uint32_t counters[5632];     // scheduling counters (self-resetting), 128-byte aligned
+    uint32_t prep_counters[kPrepCounters];     // chunks done per RHT block in thc_prepare (self-resetting)
     uint4    lut[256];           // by floor(u*g): (-T[z0] as float, 65536/(T[z0+1]-T[z0]), z0, 0)
     uint32_t table[256];         // T
 };
