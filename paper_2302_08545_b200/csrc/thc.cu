@@ -1171,7 +1171,8 @@ static int launch_pipeline(const thc_ctx *ctx, pipe_kernel_t kern, bool compress
 static bool use_block_kernel(const thc_ctx *ctx, uint64_t coords)
 {
     if (ctx->pipeline_next) return false;
-    return ctx->cfg.log2_block < kBMaxLog2 || (ctx->cfg.log2_block == kBMaxLog2 && coords <= (1ull << 22));
+    const uint32_t k = ctx->cfg.log2_block;
+    return k <= 15u || (k == 16u && coords <= (1ull << 22)) || (k == 17u && coords <= (14ull << 17));
 }
 
 // lut_bytes: table space in shared memory; keys: exact-range mode; agg_n: aggregate + decompress.

@@ -1,9 +1,9 @@
-// RHT blocks of 2^3 .. 2^16 coordinates: transform, quantise or de-quantise without an intermediate
+// RHT blocks of 2^3 .. 2^17 coordinates: transform, quantise or de-quantise without an intermediate
 // in global memory.
 //
 // A CTA holds a tile of consecutive coordinates of one worker in shared memory: 2^13 of them (one
 // block, or several small ones; 128 threads, four CTAs per SM) or 2^14 (256 threads, two CTAs).  A
-// block of 2^15 is held by a cluster of two tiles of 2^14, one of 2^16 by eight of 2^13; the CTAs
+// block of 2^15 is held by a cluster of two tiles of 2^14, one of 2^16 (2^17) by eight of 2^13 (2^14); the CTAs
 // exchange the last stages through distributed shared memory.  A thread owns 64 coordinates (64
 // registers) at a time:
 //   round 1  strides 1 .. 32: two rows of 32 coordinates per lane, straight after the load
@@ -25,7 +25,7 @@
 // feedback 1310 -> 510 us; 2^14 681 -> 444, 155 -> 123, 1316 -> 531 us.  In a cluster the gather
 // binds (a tile of every CTA crosses the SM-to-SM network): 2^15 is as fast as the two-pass pipeline
 // on large inputs (672 us; error feedback 985 -> 770 us) and takes 9.4 instead of 14 us on a few
-// blocks; 2^16 pays only there (see use_block_kernel).
+// blocks; 2^16 and 2^17 pay only there (see use_block_kernel).
 #include "thc_block.h"
 
 namespace thc {
@@ -421,7 +421,7 @@ __device__ __forceinline__ void unit_gather(uint32_t own, uint32_t row, uint32_t
 }
 
 // ------------------------------------------------------------------------ the kernel
-// KIND 0: blocks up to 2^13; 1: 2^14; 2: 2^15, two tiles of 2^14; 3: 2^16, eight tiles of 2^13.
+// KIND: see block_kind.
 template <int MODE, int BITS, bool IDENTITY, int KIND>
 __global__ void __launch_bounds__(block_tile_log2(KIND) == 13 ? 128 : 256, block_tile_log2(KIND) == 13 ? 4 : 2)
 thc_block_kernel(const __grid_constant__ TmaMaps maps, const __grid_constant__ BlockParams P,
@@ -814,7 +814,8 @@ const void *block_kernel(PipeMode mode, uint32_t bits, bool identity, uint32_t k
     case 0: return pick_mode<0>(mode, bits, identity);
     case 1: return pick_mode<1>(mode, bits, identity);
     case 2: return pick_mode<2>(mode, bits, identity);
-    default: return pick_mode<3>(mode, bits, identity);
+    case 3: return pick_mode<3>(mode, bits, identity);
+    default: return pick_mode<4>(mode, bits, identity);
     }
 }
 

@@ -4,14 +4,12 @@
 
 namespace thc {
 
-constexpr uint32_t kBMaxLog2 = 16;
-
 // How a block size is held: 0 up to 2^13, one tile of 2^13; 1: 2^14, one tile of 2^14; 2: 2^15, a
-// cluster of two tiles of 2^14; 3: 2^16, a cluster of eight tiles of 2^13.  A tile of 2^13 has 128
+// cluster of two tiles of 2^14; 3 and 4: 2^16 and 2^17, a cluster of eight tiles of 2^13 or 2^14.  A tile of 2^13 has 128
 // threads and four CTAs per SM, one of 2^14 256 threads and two.
-__host__ __device__ constexpr int block_kind(uint32_t k) { return k <= 13u ? 0 : k == 14u ? 1 : k == 15u ? 2 : 3; }
-__host__ __device__ constexpr int block_tile_log2(int kind) { return kind == 1 || kind == 2 ? 14 : 13; }
-__host__ __device__ constexpr uint32_t block_cluster_log2(int kind) { return kind == 2 ? 1u : kind == 3 ? 3u : 0u; }
+__host__ __device__ constexpr int block_kind(uint32_t k) { return k <= 13u ? 0 : k == 14u ? 1 : k == 15u ? 2 : k == 16u ? 3 : 4; }
+__host__ __device__ constexpr int block_tile_log2(int kind) { return kind == 0 || kind == 3 ? 13 : 14; }
+__host__ __device__ constexpr uint32_t block_cluster_log2(int kind) { return kind == 2 ? 1u : kind >= 3 ? 3u : 0u; }
 
 struct BlockParams {
     uint64_t d;
