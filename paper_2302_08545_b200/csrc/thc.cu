@@ -64,6 +64,19 @@ quantize_rotated_kernel(PtrArray rotated, MutPtrArray packed, uint64_t d_pad, ui
 // low half of the table answers indices 0-7 and, with bit 3 flipped, the high half answers
 // 8-15; the two results are disjoint and are added into packed byte accumulators (no byte
 // can overflow because workers * g <= 255).
+// 32 bytes of sums to a 16-byte aligned address; in one store where it is 32-byte aligned, so that no
+// sector of 32 bytes reaches the L2 in two halves.
+__device__ __forceinline__ void store_sums32(uint4 *p, bool aligned32, const uint32_t (&v)[8])
+{
+    if (aligned32) {
+        asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" :: "l"(p), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]),
+                     "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]) : "memory");
+    } else {
+        p[0] = make_uint4(v[0], v[1], v[2], v[3]);
+        p[1] = make_uint4(v[4], v[5], v[6], v[7]);
+    }
+}
+
 __global__ void __launch_bounds__(kThreads)
 aggregate_b4w8_kernel(PtrArray in, uint32_t n, uint64_t units32, const DeviceBlock *dev,
                       uint4 *__restrict__ sum)
@@ -73,6 +86,7 @@ aggregate_b4w8_kernel(PtrArray in, uint32_t n, uint64_t units32, const DeviceBlo
     for (int q = 0; q < 4; ++q)
         t[q] = dev->table[4 * q] | (dev->table[4 * q + 1] << 8) | (dev->table[4 * q + 2] << 16) |
                (dev->table[4 * q + 3] << 24);
+    const bool aligned32 = (reinterpret_cast<uintptr_t>(sum) & 31u) == 0;
     // A thread sums 32 coordinates: 16 bytes of indices per worker, the loads of up to eight
     // workers in flight together, 32 bytes of sums out.
     for (uint64_t u = (uint64_t)blockIdx.x * kThreads + threadIdx.x; u < units32;
@@ -95,8 +109,7 @@ aggregate_b4w8_kernel(PtrArray in, uint32_t n, uint64_t units32, const DeviceBlo
                 }
             }
         }
-        __stcs(sum + 2 * u, make_uint4(acc[0], acc[1], acc[2], acc[3]));
-        __stcs(sum + 2 * u + 1, make_uint4(acc[4], acc[5], acc[6], acc[7]));
+        store_sums32(sum + 2 * u, aligned32, acc);
     }
 }
 
@@ -113,6 +126,7 @@ aggregate_b4w16_kernel(PtrArray in, uint32_t n, uint64_t units32, const DeviceBl
     for (int q = 0; q < 4; ++q)
         t[q] = dev->table[4 * q] | (dev->table[4 * q + 1] << 8) | (dev->table[4 * q + 2] << 16) |
                (dev->table[4 * q + 3] << 24);
+    const bool aligned32 = (reinterpret_cast<uintptr_t>(sum) & 31u) == 0;
     // A thread sums 32 coordinates: 16 bytes of indices per worker, 64 bytes of sums out.
     for (uint64_t u = (uint64_t)blockIdx.x * kThreads + threadIdx.x; u < units32;
          u += (uint64_t)gridDim.x * kThreads) {
@@ -141,14 +155,14 @@ aggregate_b4w16_kernel(PtrArray in, uint32_t n, uint64_t units32, const DeviceBl
             }
         }
 #pragma unroll
-        for (int q4 = 0; q4 < 4; ++q4) {
-            uint32_t o[4];
+        for (int q4 = 0; q4 < 2; ++q4) {
+            uint32_t o[8];
 #pragma unroll
-            for (int q = 0; q < 2; ++q) {
-                o[2 * q] = prmt(even[2 * q4 + q], odd[2 * q4 + q], 0x5410u);          // coordinates 4q, 4q+1
-                o[2 * q + 1] = prmt(even[2 * q4 + q], odd[2 * q4 + q], 0x7632u);      // coordinates 4q+2, 4q+3
+            for (int q = 0; q < 4; ++q) {
+                o[2 * q] = prmt(even[4 * q4 + q], odd[4 * q4 + q], 0x5410u);          // coordinates 4q, 4q+1
+                o[2 * q + 1] = prmt(even[4 * q4 + q], odd[4 * q4 + q], 0x7632u);      // coordinates 4q+2, 4q+3
             }
-            __stcs(sum + 4 * u + q4, make_uint4(o[0], o[1], o[2], o[3]));
+            store_sums32(sum + 4 * u + 2 * q4, aligned32, o);
         }
     }
 }
@@ -205,8 +219,80 @@ aggregate_small_w8_kernel(PtrArray in, uint32_t n, uint64_t units32, uint32_t g_
                 }
             }
         }
-        sum[2 * u] = make_uint4(o[0], o[1], o[2], o[3]);
-        sum[2 * u + 1] = make_uint4(o[4], o[5], o[6], o[7]);
+        store_sums32(sum + 2 * u, (reinterpret_cast<uintptr_t>(sum) & 31u) == 0, o);
+    }
+}
+
+// 3-bit indices, any table: eight bytes in two registers, looked up four at a time.  The 24 bits of eight
+// indices are spread into nibbles (three shift-and-mask steps); table values are summed in byte
+// lanes for `chunk` workers at a time (chunk * g <= 255) and, for 16-bit sums, widened into 16-bit lanes
+// in between.  A thread sums 64 coordinates: three 8-byte loads per worker, of four workers in flight.
+// (The shared-memory table of aggregate_kernel takes a look-up per index: 12.6 us on 10 workers x 2^22.)
+template <int W>
+__global__ void __launch_bounds__(128)
+aggregate_b3_kernel(PtrArray in, uint32_t n, uint64_t units64, uint32_t chunk, const DeviceBlock *dev, uint4 *__restrict__ sum)
+{
+    const uint32_t t0 = dev->table[0] | (dev->table[1] << 8) | (dev->table[2] << 16) | (dev->table[3] << 24);
+    const uint32_t t1 = dev->table[4] | (dev->table[5] << 8) | (dev->table[6] << 16) | (dev->table[7] << 24);
+    const bool aligned32 = (reinterpret_cast<uintptr_t>(sum) & 31u) == 0;
+    for (uint64_t u = (uint64_t)blockIdx.x * 128 + threadIdx.x; u < units64; u += (uint64_t)gridDim.x * 128) {
+        uint32_t wide[W == 16 ? 32 : 1];
+#pragma unroll
+        for (int q = 0; q < (W == 16 ? 32 : 1); ++q) wide[q] = 0u;
+        uint32_t acc[16];                              // 64 sums of 8 bits
+#pragma unroll
+        for (int q = 0; q < 16; ++q) acc[q] = 0u;
+#pragma unroll 1
+        for (uint32_t i0 = 0; i0 < n; i0 += chunk) {
+            const uint32_t i1 = min(n, i0 + chunk);
+#pragma unroll 4
+            for (uint32_t i = i0; i < i1; ++i) {
+                uint32_t w[7];
+#pragma unroll
+                for (int q = 0; q < 3; ++q) {
+                    const uint2 v = __ldg(reinterpret_cast<const uint2 *>(in.p[i]) + 3 * u + q);
+                    w[2 * q] = v.x; w[2 * q + 1] = v.y;
+                }
+                w[6] = 0u;
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    const uint32_t x = __funnelshift_r(w[24 * e / 32], w[24 * e / 32 + 1], 24 * e % 32);
+                    const uint32_t y = (x & 0x00000FFFu) | ((x << 4) & 0x0FFF0000u);
+                    const uint32_t z = (y & 0x003F003Fu) | ((y << 2) & 0x3F003F00u);
+                    const uint32_t s = (z & 0x07070707u) | ((z << 1) & 0x70707070u);
+                    acc[2 * e] += prmt(t0, t1, s);
+                    acc[2 * e + 1] += prmt(t0, t1, s >> 16);
+                }
+            }
+            if (W == 16) {
+#pragma unroll
+                for (int q = 0; q < 16; ++q) {
+                    wide[(2 * q) % (W == 16 ? 32 : 1)] += acc[q] & 0x00FF00FFu;
+                    wide[(2 * q + 1) % (W == 16 ? 32 : 1)] += (acc[q] >> 8) & 0x00FF00FFu;
+                    acc[q] = 0u;
+                }
+            }
+        }
+        if (W == 8) {
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const uint32_t o[8] = {acc[8 * q], acc[8 * q + 1], acc[8 * q + 2], acc[8 * q + 3],
+                                       acc[8 * q + 4], acc[8 * q + 5], acc[8 * q + 6], acc[8 * q + 7]};
+                store_sums32(sum + 4 * u + 2 * q, aligned32, o);
+            }
+        } else {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                uint32_t o[8];
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    const uint32_t even = wide[(8 * q + 2 * c) % (W == 16 ? 32 : 1)], odd = wide[(8 * q + 2 * c + 1) % (W == 16 ? 32 : 1)];
+                    o[2 * c] = prmt(even, odd, 0x5410u);
+                    o[2 * c + 1] = prmt(even, odd, 0x7632u);
+                }
+                store_sums32(sum + 8 * u + 2 * q, aligned32, o);
+            }
+        }
     }
 }
 
@@ -234,22 +320,32 @@ aggregate_b8w16_kernel(PtrArray in, uint32_t n, uint64_t units16, uint4 *__restr
             o[2 * q] = prmt(even[q], odd[q], 0x5410u);
             o[2 * q + 1] = prmt(even[q], odd[q], 0x7632u);
         }
-        sum[2 * u] = make_uint4(o[0], o[1], o[2], o[3]);
-        sum[2 * u + 1] = make_uint4(o[4], o[5], o[6], o[7]);
+        store_sums32(sum + 2 * u, (reinterpret_cast<uintptr_t>(sum) & 31u) == 0, o);
     }
 }
 
 // ------------------------------------------------------------------------ error feedback
-// x <- x + e, 128-bit accesses with a scalar tail.
+// x <- x + e of all workers in one launch: four 16-byte loads of each in flight per thread, a scalar tail.
+// (One launch per worker: 4 x 7,000,003 coordinates 62 us, now 50 us = 6.7 TB/s.)
+constexpr int kAccUnits = 4;
 __global__ void __launch_bounds__(kThreads)
-accumulate_kernel(float *__restrict__ x, const float *__restrict__ e, uint64_t d)
+accumulate_kernel(MutPtrArray xs, PtrArray es, uint64_t d)
 {
+    float *x = static_cast<float *>(xs.p[blockIdx.y]);
+    const float *e = static_cast<const float *>(es.p[blockIdx.y]);
     const uint64_t n4 = d / 4;
-    for (uint64_t c = (uint64_t)blockIdx.x * kThreads + threadIdx.x; c < n4; c += (uint64_t)gridDim.x * kThreads) {
-        float4 a = reinterpret_cast<float4 *>(x)[c];
-        const float4 b = __ldg(reinterpret_cast<const float4 *>(e) + c);
-        a.x = a.x + b.x; a.y = a.y + b.y; a.z = a.z + b.z; a.w = a.w + b.w;
-        reinterpret_cast<float4 *>(x)[c] = a;
+    const uint64_t c0 = (uint64_t)blockIdx.x * (kThreads * kAccUnits) + threadIdx.x;
+    float4 a[kAccUnits], b[kAccUnits];
+#pragma unroll
+    for (int i = 0; i < kAccUnits; ++i) {
+        const uint64_t c = c0 + (uint64_t)i * kThreads;
+        if (c < n4) { a[i] = reinterpret_cast<float4 *>(x)[c]; b[i] = __ldg(reinterpret_cast<const float4 *>(e) + c); }
+    }
+#pragma unroll
+    for (int i = 0; i < kAccUnits; ++i) {
+        const uint64_t c = c0 + (uint64_t)i * kThreads;
+        if (c < n4)
+            reinterpret_cast<float4 *>(x)[c] = make_float4(a[i].x + b[i].x, a[i].y + b[i].y, a[i].z + b[i].z, a[i].w + b[i].w);
     }
     if (blockIdx.x == 0 && threadIdx.x < (d & 3)) {
         const uint64_t j = n4 * 4 + threadIdx.x;
@@ -1167,7 +1263,8 @@ static int launch_pipeline(const thc_ctx *ctx, pipe_kernel_t kern, bool compress
 // Blocks up to 2^15 always; 2^16 up to 2^22 coordinates over all workers, where the two-pass pipeline
 // has less than a task per CTA and its chain of queue, ring and counters is all latency: 8.8 us
 // instead of 13.9 on a block or two, 21 instead of 23 on 2^22 coordinates; on 2^24 the cluster's
-// gather makes it 74 against 53.
+// gather makes it 74 against 53.  2^17 up to 14 blocks, the clusters of eight half SMs that are resident
+// at a time: 13.1 us instead of 19.1 on 12 blocks, 18.6 against 19.4 on 16.
 static bool use_block_kernel(const thc_ctx *ctx, uint64_t coords)
 {
     if (ctx->pipeline_next) return false;
@@ -1573,6 +1670,17 @@ int thc_aggregate(thc_ctx *ctx, const void *const *packed, uint32_t n, uint64_t 
         THC_CUDA(cudaGetLastError());
         return THC_OK;
     }
+    if (bits == 3 && w <= 16 && sz.d_pad % 64 == 0) {
+        const uint64_t units64 = sz.d_pad / 64;
+        uint64_t nb = (units64 + 127) / 128;
+        if (nb > (uint64_t)ctx->sm_count * 64) nb = (uint64_t)ctx->sm_count * 64;
+        uint4 *s4 = reinterpret_cast<uint4 *>(s);
+        const uint32_t chunk = w == 8 ? n : 255u / g;
+        if (w == 8) aggregate_b3_kernel<8><<<(unsigned)nb, 128, 0, st>>>(in, n, units64, chunk, ctx->dev, s4);
+        else aggregate_b3_kernel<16><<<(unsigned)nb, 128, 0, st>>>(in, n, units64, chunk, ctx->dev, s4);
+        THC_CUDA(cudaGetLastError());
+        return THC_OK;
+    }
     if (bits == 8 && ctx->identity && w == 16 && sz.d_pad % 16 == 0) {
         const uint64_t units16 = sz.d_pad / 16;
         uint64_t nb = (units16 + kThreads - 1) / kThreads;
@@ -1649,12 +1757,22 @@ int thc_accumulate_error(thc_ctx *ctx, float *const *grads, const float *const *
     if ((rc = check_ptr_array(reinterpret_cast<const void *const *>(grads), n_local)) != THC_OK) return rc;
     if ((rc = check_ptr_array(reinterpret_cast<const void *const *>(ef), n_local)) != THC_OK) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    uint64_t blocks = (d / 4 + kThreads - 1) / kThreads;
-    const uint64_t cap = (uint64_t)ctx->sm_count * 16;
-    if (blocks > cap) blocks = cap;
-    if (blocks == 0) blocks = 1;
-    for (uint32_t i = 0; i < n_local; ++i) {
-        accumulate_kernel<<<(unsigned)blocks, kThreads, 0, st>>>(grads[i], ef[i], d);
+    const uint64_t blocks = (d / 4 + kThreads * kAccUnits - 1) / (kThreads * kAccUnits);
+    if (blocks > 0x7FFFFFFFull) return THC_EUNSUPPORTED;
+    MutPtrArray x;
+    PtrArray e;
+    memset(&x, 0, sizeof x);
+    memset(&e, 0, sizeof e);
+    // buffers that overlap (one gradient that takes several residuals) are added in the order given
+    const auto overlap = [d](const float *a, const float *b) { return a < b + d && b < a + d; };
+    bool apart = true;
+    for (uint32_t i = 0; i < n_local; ++i)
+        for (uint32_t j = 0; j < n_local; ++j)
+            if (i != j && (overlap(grads[i], grads[j]) || overlap(grads[i], ef[j]))) apart = false;
+    const uint32_t per_launch = apart ? n_local : 1u;
+    for (uint32_t i0 = 0; i0 < n_local; i0 += per_launch) {
+        for (uint32_t i = 0; i < per_launch; ++i) { x.p[i] = grads[i0 + i]; e.p[i] = ef[i0 + i]; }
+        accumulate_kernel<<<dim3((unsigned)(blocks ? blocks : 1), per_launch), kThreads, 0, st>>>(x, e, d);
         THC_CUDA(cudaGetLastError());
     }
     return THC_OK;

@@ -69,19 +69,6 @@ __device__ __forceinline__ float4 *low_chunk(float4 *wtile, const LowRows &lr, i
     return wtile + row * 8 + ((m & 7) ^ (row & 7));
 }
 
-// A butterfly whose operands some lanes hold the other way round (x is the upper one where
-// s = -1): (x, y) <- (x + y, x - y) for s = 1 and (y - x, y + x) for s = -1, each one rounding of
-// the exact sum or difference.
-__device__ __forceinline__ void swapped_butterfly(float4 &x, float4 &y, float s)
-{
-    const float2 s2 = make_float2(s, s), n2 = make_float2(-s, -s);
-    const float2 xl = make_float2(x.x, x.y), xh = make_float2(x.z, x.w), yl = make_float2(y.x, y.y), yh = make_float2(y.z, y.w);
-    const float2 al = __ffma2_rn(xl, s2, yl), ah = __ffma2_rn(xh, s2, yh);
-    const float2 bl = __ffma2_rn(yl, n2, xl), bh = __ffma2_rn(yh, n2, xh);
-    x = make_float4(al.x, al.y, ah.x, ah.y);
-    y = make_float4(bl.x, bl.y, bh.x, bh.y);
-}
-
 // The stages of strides 1 .. 32 that lie inside the block, and the store back.  (Variants side by
 // side: stages under a condition, in place in 64 registers, cost the compiler 40 spilled ones.)
 __device__ __forceinline__ void low_stages_store(float4 *wtile, const LowRows &lr, float4 (&v)[16], uint32_t k)

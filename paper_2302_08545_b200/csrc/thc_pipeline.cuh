@@ -400,6 +400,26 @@ __device__ __forceinline__ void p_rounds(float4 *tile, int lo, int hi, int tid, 
     }
 }
 
+// A butterfly whose operands some lanes hold the other way round (x is the upper one where
+// s = -1): (x, y) <- (x + y, x - y) for s = 1 and (y - x, y + x) for s = -1, each one rounding of
+// the exact sum or difference.  Lets lanes that would meet in a bank walk their rows in another
+// order at no cost.
+__device__ __forceinline__ void swapped_butterfly(float2 &x, float2 &y, float s)
+{
+    const float2 a = __ffma2_rn(x, make_float2(s, s), y);
+    const float2 b = __ffma2_rn(y, make_float2(-s, -s), x);
+    x = a;
+    y = b;
+}
+__device__ __forceinline__ void swapped_butterfly(float4 &x, float4 &y, float s)
+{
+    float2 xl = make_float2(x.x, x.y), xh = make_float2(x.z, x.w), yl = make_float2(y.x, y.y), yh = make_float2(y.z, y.w);
+    swapped_butterfly(xl, yl, s);
+    swapped_butterfly(xh, yh, s);
+    x = make_float4(xl.x, xl.y, xh.x, xh.y);
+    y = make_float4(yl.x, yl.y, yh.x, yh.y);
+}
+
 // ------------------------------------------------------------------------------- pass A
 // A tile is 256 rows of 8 chunks (32 coordinates); row r, chunk cc sits at r*8 + (cc ^ (r&7)).
 //
@@ -906,6 +926,101 @@ __device__ __forceinline__ void pass_b_last_round_kb7(float4 *tile, int tid,
     }
 }
 
+// ---- panels of 2^21 and 2^22 blocks in compress: eight and nine stages in two rounds (4 + 4, 5 + 4).  (With
+// rounds of at most four stages and three in the last one it takes 4 + 1 + 3 and 4 + 2 + 3.)
+//
+// 2^22: 512 rows of 64 bytes in the 64-byte swizzle (16-byte chunk c of row r at c ^ ((r >> 1) & 3)).  Row
+// bits 0..4 on pairs of coordinates: thread (row group G = tid >> 3, pair f) owns rows 32 G + m.  The
+// two row groups of a half warp would meet in the same 64 bytes, so odd groups keep row m ^ 1 in
+// register m.
+__device__ __forceinline__ void pass_b_low5(float4 *tile, int tid)
+{
+    const int f = tid & 7, h = (tid >> 3) & 1;
+    unsigned char *b = reinterpret_cast<unsigned char *>(tile) + (tid >> 3) * 2048;
+    const int lane_bits = (h << 6) | ((f >> 1) << 4) | ((f & 1) << 3);
+    float2 *p[8];
+#pragma unroll
+    for (int x = 0; x < 8; ++x)
+        p[x] = reinterpret_cast<float2 *>(b + (x >> 1) * 128 + (lane_bits ^ (((x & 1) << 6) | ((x >> 1) << 4))));
+    float2 v[32];
+#pragma unroll
+    for (int m = 0; m < 32; ++m) v[m] = p[m & 7][(m >> 3) * 64];
+#pragma unroll
+    for (int m = 0; m < 32; m += 2) swapped_butterfly(v[m], v[m + 1], h ? -1.0f : 1.0f);
+#pragma unroll
+    for (int t = 1; t < 5; ++t) {
+#pragma unroll
+        for (int m = 0; m < 32; ++m)
+            if (!(m & (1 << t))) {
+                const float2 a = v[m], c = v[m | (1 << t)];
+                v[m] = add2(a, c);
+                v[m | (1 << t)] = sub2(a, c);
+            }
+    }
+#pragma unroll
+    for (int m = 0; m < 32; ++m) p[m & 7][(m >> 3) * 64] = v[m];
+}
+
+// Last round: the top four row bits, then the epilogue on the registers.  Thread tid owns chunk tid of the
+// panel's first sixteenth and the chunks 128 m behind it (m = 0..15), which are 2^(k-4) m
+// coordinates apart in the block.
+//
+// The two lanes of a unit of eight coordinates (chunks c, c ^ 1) keep the sixteen rows in another
+// order, m ^ 8 in the odd lane.  So registers 0..7 of the two lanes are the unit's sixteen rows:
+// each lane draws the Philox call of its own eight, keeps the half that belongs to its four columns
+// and hands the other half over; the indices of registers 8..15 then go the other way, and each
+// lane stores eight whole units.
+template <int BITS, bool IDENTITY, int KB>
+__device__ __forceinline__ void pass_b_high4(const float4 *tile, int tid, const EpilogueCtx &ep, const PhiloxKeys &keys)
+{
+    constexpr int ccl = 11 - KB, mask = KB == 9 ? 3 : 7;       // log2 chunks per row, swizzle
+    constexpr uint32_t step = 1u << (KB + kPLog2 - 4);
+    const int c = tid & ((1 << ccl) - 1), q = tid >> ccl;
+    const int hb = c & 1;
+    const float4 *lo = tile + (tid ^ ((tid >> 3) & mask)) + (hb ? 1024 : 0);
+    const float4 *hi = lo + (hb ? -1024 : 1024);
+    float4 v[16];
+#pragma unroll
+    for (int m = 0; m < 8; ++m) { v[m] = lo[m << 7]; v[8 + m] = hi[m << 7]; }
+#pragma unroll
+    for (int t = 0; t < 3; ++t) {
+#pragma unroll
+        for (int m = 0; m < 16; ++m)
+            if (!(m & (1 << t))) butterfly(v[m], v[m | (1 << t)]);
+    }
+#pragma unroll
+    for (int m = 0; m < 8; ++m) swapped_butterfly(v[m], v[8 + m], hb ? -1.0f : 1.0f);
+    // coordinates of registers 0 and 8, and the unit of register 0; register m: + m step
+    const uint64_t j_first = ep.j_tile + ((uint64_t)q << kPLog2) + 4 * c;
+    const uint64_t ja = j_first + (hb ? 8u * step : 0u), jb = j_first + (hb ? 0u : 8u * step);
+    const uint64_t unit = ja & ~(uint64_t)7;
+    const uint32_t call_lo = (uint32_t)(unit >> 3), call_hi = (uint32_t)(unit >> 35);   // a block's calls share the high word
+#pragma unroll 1
+    for (int half = 0; half < 2; ++half) {
+#pragma unroll
+        for (int mm = 0; mm < 4; ++mm) {
+            const uint32_t m = 4u * half + mm;
+            const float4 a = scale4(v[mm], ep.c_block), b = scale4(v[8 + mm], ep.c_block);
+            if (ep.rotated != nullptr) {
+                *reinterpret_cast<float4 *>(ep.rotated + ja + (uint64_t)(m * step)) = a;
+                *reinterpret_cast<float4 *>(ep.rotated + jb + (uint64_t)(m * step)) = b;
+            }
+            const uint4 rnd = philox4x32_10(call_lo + m * (step >> 3), call_hi, ep.worker, ep.round, keys);
+            const uint32_t own0 = hb ? rnd.z : rnd.x, own1 = hb ? rnd.w : rnd.y;
+            const uint32_t other0 = __shfl_xor_sync(0xFFFFFFFFu, hb ? rnd.x : rnd.z, 1);
+            const uint32_t other1 = __shfl_xor_sync(0xFFFFFFFFu, hb ? rnd.y : rnd.w, 1);
+            const uint32_t za = quantize4<BITS, IDENTITY>(a.x, a.y, a.z, a.w, ep.kappa, ep.half_g, ep.gf, own0, own1, ep.lut);
+            const uint32_t zb = quantize4<BITS, IDENTITY>(b.x, b.y, b.z, b.w, ep.kappa, ep.half_g, ep.gf, other0, other1, ep.lut);
+            const uint32_t zo = __shfl_xor_sync(0xFFFFFFFFu, zb, 1);
+            const uint64_t z = BITS == 4 ? (uint64_t)__byte_perm(za, zo, hb ? 0x1054 : 0x5410)
+                                         : join_units<BITS>(hb ? zo : za, hb ? za : zo);
+            store_unit<BITS>(ep.packed, unit + (uint64_t)(m * step), z);
+        }
+#pragma unroll
+        for (int mm = 0; mm < 4; ++mm) { v[mm] = v[mm + 4]; v[8 + mm] = v[12 + mm]; }
+    }
+}
+
 // ------------------------------------------------------------------------------ the kernel
 // KB = 7 specialises the k = 20 geometry at compile time; KB = 0 reads it from the params.
 template <int MODE, int BITS, bool IDENTITY, int KB>
@@ -1379,7 +1494,10 @@ thc_pipeline_kernel(const __grid_constant__ TmaMaps maps, PipeParams P, PtrArray
                     fill_sign_words(sw, g, j_tile, keys, tid, kPThreads);
                 }
                 const int e1 = kb < 4 ? kb : 4;
-                if (KB != 7) {
+                if (KB == 9) {
+                    pass_b_low5(tile, tid);
+                    compute_barrier();
+                } else if (KB != 7) {
                     switch (e1) {
                     case 4: p_round<4>(tile, ccl, tid, bmask); break;
                     case 3: p_round<3>(tile, ccl, tid, bmask); break;
@@ -1390,6 +1508,8 @@ thc_pipeline_kernel(const __grid_constant__ TmaMaps maps, PipeParams P, PtrArray
                 uint32_t kmin = 0xFFFFFFFFu, kmax = 0u;
                 if (KB == 7) {
                     pass_b_last_round_kb7<kCompress, BITS, IDENTITY, kRange>(tile, tid, ep, keys, kmin, kmax);
+                } else if constexpr (KB == 8 || KB == 9) {
+                    pass_b_high4<BITS, IDENTITY, KB>(tile, tid, ep, keys);
                 } else {
                     const int rem = kb - e1;
                     const int e_last = rem < 3 ? rem : 3;
