@@ -1308,15 +1308,16 @@ thc_pipeline_kernel(const __grid_constant__ TmaMaps maps, PipeParams P, PtrArray
                         tma = 1; phase = uses[s] & 1u; ++uses[s];
                     }
                 }
-                if (t.is_b && kEF && KB == 7) {
-                    // error feedback: the x values the epilogue will read (128 rows x 64 columns)
-                    const uint64_t j_panel = (uint64_t)r * B + ((uint64_t)t.idx << 6);
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        const uint64_t jr = j_panel + ((uint64_t)(lane + 32 * c) << kPLog2);
-                        const float *xr = static_cast<const float *>(rotated.p[t.wb - r * P.n_local]) + jr;
-                        if (jr < P.d) prefetch_l2(xr);
-                        if (jr + 32 < P.d) prefetch_l2(xr + 32);
+                if (t.is_b && kEF) {
+                    // error feedback: pull the x values the epilogue will read into L2, 256 lines in rows of
+                    // 2^(13-kb) coordinates
+                    const uint64_t j_panel = (uint64_t)r * B + ((uint64_t)t.idx << (kPLog2 - kb));
+                    const float *x = static_cast<const float *>(rotated.p[t.wb - r * P.n_local]);
+                    const int lpr = kb < 8 ? 8 - kb : 0;             // log2 of the 128-byte lines per row
+#pragma unroll 2
+                    for (int l = lane; l < (1 << (kb + lpr)); l += 32) {
+                        const uint64_t j = j_panel + ((uint64_t)(l >> lpr) << kPLog2) + 32u * (l & ((1 << lpr) - 1));
+                        if (j < P.d) prefetch_l2(x + j);
                     }
                 }
                 ti.tma = tma;
