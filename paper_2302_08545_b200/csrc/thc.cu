@@ -847,6 +847,17 @@ int thc_destroy(thc_ctx *ctx)
 
 static uint64_t round_up(uint64_t v, uint64_t a) { return (v + a - 1) / a * a; }
 
+// Which blocks are held in shared memory (thc_block.cu), by size and coordinates over all workers.
+// Blocks up to 2^15 always; 2^16 up to 2^22 coordinates over all workers, where the two-pass pipeline
+// has less than a task per CTA and its chain of queue, ring and counters is all latency: 8.8 us
+// instead of 13.9 on a block or two, 21 instead of 23 on 2^22 coordinates; on 2^24 the cluster's
+// gather makes it 74 against 53.  2^17 up to 14 blocks, the clusters of eight half SMs that are resident
+// at a time: 13.1 us instead of 19.1 on 12 blocks, 18.6 against 19.4 on 16.
+static bool block_kernel_serves(uint32_t k, uint64_t coords)
+{
+    return k <= 15u || (k == 16u && coords <= (1ull << 22)) || (k == 17u && coords <= (14ull << 17));
+}
+
 // Schedule of the persistent pipeline for `wb_count` worker-blocks of 2^k coordinates:
 // how far pass B trails pass A (lag, in worker-blocks) and how many ring slots that needs.
 struct PipePlan { uint32_t grid, lag, ring; };
@@ -877,10 +888,11 @@ static PipePlan plan_pipeline(const thc_ctx *ctx, uint64_t wb_count)
 // The same for the fused-scales kernel: pass B of a block can start only when all n workers'
 // tiles of the block are done, so it trails by n - 1 more worker-blocks and the ring grows by
 // as many slots.  Used only where that ring still fits comfortably in L2 and the per-block
-// counters (16 residues) cannot alias; otherwise the caller runs prepare and compress apart.
+// counters (160 residues) cannot alias; otherwise the caller runs prepare and compress apart.
 static bool plan_pipeline_fused(const thc_ctx *ctx, uint64_t nblocks, uint32_t n, PipePlan *out)
 {
-    if (ctx->cfg.log2_block != 20 || ctx->cfg.in_dtype != THC_F32) return false;
+    const uint32_t k = ctx->cfg.log2_block;
+    if (k > 20u || ctx->cfg.in_dtype != THC_F32 || block_kernel_serves(k, (nblocks * n) << k)) return false;
     if (ctx->cfg.range_mode != THC_RANGE_NORM) return false;
     const uint64_t wb_count = nblocks * n;
     PipePlan p = plan_pipeline(ctx, wb_count);
@@ -888,8 +900,8 @@ static bool plan_pipeline_fused(const thc_ctx *ctx, uint64_t nblocks, uint32_t n
     const uint64_t lag = (uint64_t)p.lag + n - 1;
     const uint64_t ring = lag + window;
     if (ring > wb_count || ring > (uint64_t)kMaxRing) return false;
-    if (ring * ((uint64_t)4 << 20) > ((uint64_t)96 << 20)) return false;
-    if ((ring + n - 1) / n + 2 > 16) return false;
+    if (((ring << k) * 4) > ((uint64_t)96 << 20)) return false;
+    if ((ring + n - 1) / n + 2 > (uint64_t)kFusedBlocks) return false;
     p.lag = (uint32_t)lag;
     p.ring = (uint32_t)ring;
     *out = p;
@@ -1260,16 +1272,9 @@ static int launch_pipeline(const thc_ctx *ctx, pipe_kernel_t kern, bool compress
 }
 
 // ---- blocks held in shared memory (RHT blocks of up to 2^16 coordinates)
-// Blocks up to 2^15 always; 2^16 up to 2^22 coordinates over all workers, where the two-pass pipeline
-// has less than a task per CTA and its chain of queue, ring and counters is all latency: 8.8 us
-// instead of 13.9 on a block or two, 21 instead of 23 on 2^22 coordinates; on 2^24 the cluster's
-// gather makes it 74 against 53.  2^17 up to 14 blocks, the clusters of eight half SMs that are resident
-// at a time: 13.1 us instead of 19.1 on 12 blocks, 18.6 against 19.4 on 16.
 static bool use_block_kernel(const thc_ctx *ctx, uint64_t coords)
 {
-    if (ctx->pipeline_next) return false;
-    const uint32_t k = ctx->cfg.log2_block;
-    return k <= 15u || (k == 16u && coords <= (1ull << 22)) || (k == 17u && coords <= (14ull << 17));
+    return !ctx->pipeline_next && block_kernel_serves(ctx->cfg.log2_block, coords);
 }
 
 // lut_bytes: table space in shared memory; keys: exact-range mode; agg_n: aggregate + decompress.
@@ -1474,7 +1479,8 @@ int thc_prepare_compress(thc_ctx *ctx, const void *const *grads, uint32_t n, uin
             prot.p[i] = rotated[i];
         }
     }
-    pipe_kernel_t kern = pick_pipe_kernel_kb<kCompressF32Fused, 7>(ctx->cfg.bits, ctx->identity);
+    pipe_kernel_t kern = ctx->cfg.log2_block == 20 ? pick_pipe_kernel_kb<kCompressF32Fused, 7>(ctx->cfg.bits, ctx->identity)
+                                                    : pick_pipe_kernel_kb<kCompressF32Fused, 0>(ctx->cfg.bits, ctx->identity);
     return launch_pipeline(ctx, kern, true, sz, d, n, worker_base, round, 1, scales, workspace, pin, pout,
                            prot, static_cast<cudaStream_t>(stream), scales);
 }

@@ -40,8 +40,8 @@
 // n_local * T tiles computes M = t_p * max_i ||x_i|| / sqrt(B) from the stored sums in a fixed
 // order, writes it to `scales` and releases the block's pass-B tasks.  The queue trails pass B
 // behind pass A by n_local - 1 more worker-blocks so that this is normally done in time.
-// In this mode a_done[0..15] count finished tiles of block r in entry r mod 16 and
-// a_done[16..31] count finished blocks of that residue.
+// In this mode a_done[0..159] count finished tiles of block r in entry r mod 160 and
+// a_done[160..319] count finished blocks of that residue.
 //
 // Counters (in the context's device block, all zero between launches; the last CTA to leave
 // clears them):  head, exited, abort, a_done[R], b_done[R].  a_done[s] counts finished A tiles
@@ -60,6 +60,8 @@ constexpr int kPThreads = 128;                // compute threads of a CTA
 constexpr int kPCtaThreads = 160;             // plus one control warp that runs the queue
 constexpr int kPSignWords = 512;            // sign words: two slots of 256 (pass A) or one of 512
 constexpr int kMaxRing = 320;                // ring slots: blocks of 2^15 need up to 280 to cover the tasks in flight
+constexpr uint32_t kFusedBlocks = 160;       // fused scales: blocks in flight have counters of their own
+static_assert(2 * kFusedBlocks <= (uint32_t)kMaxRing, "the block counters share the tile counters' array");
 constexpr int kBlockConstMax = 256;         // per-block constants cached in shared memory
 constexpr uint32_t kMaxPolls = 1u << 21;
 
@@ -1114,13 +1116,13 @@ thc_pipeline_kernel(const __grid_constant__ TmaMaps maps, PipeParams P, PtrArray
             if (lane == 0) {
                 const double tile_sum = (s_sq[sq][0] + s_sq[sq][1]) + (s_sq[sq][2] + s_sq[sq][3]);
                 __stcg(P.tile_sq + (((size_t)t.wb << kb) + t.idx), tile_sum);
-                old = atom_release_add(&pc->a_done[r & 15u].v, 1u);
+                old = atom_release_add(&pc->a_done[r % kFusedBlocks].v, 1u);
             }
             return true;
         };
         auto complete_finish = [&](uint32_t old, uint32_t r) {
             old = __shfl_sync(0xFFFFFFFFu, old, 0);
-            if (old + 1u != (r / 16u + 1u) * P.n_local * T) return;
+            if (old + 1u != (r / kFusedBlocks + 1u) * P.n_local * T) return;
             __threadfence();                           // the other tiles' sums, after seeing the count
             // Eight workers at a time, four lanes per worker: each lane adds every fourth of
             // its worker's T tile sums (all loads in flight together), the four lanes are
@@ -1156,7 +1158,7 @@ thc_pipeline_kernel(const __grid_constant__ TmaMaps maps, PipeParams P, PtrArray
                 br.hi = M; br.lo = -M;
                 __stcg(P.fused_const + r, compress_constants(br));
                 if (flags) atomicOr(&P.dev->status, flags);
-                red_release_add(&pc->a_done[16u + (r & 15u)].v, 1u);
+                red_release_add(&pc->a_done[kFusedBlocks + r % kFusedBlocks].v, 1u);
             }
         };
         auto complete = [&](const TaskId &t, int sq) {
@@ -1235,8 +1237,8 @@ thc_pipeline_kernel(const __grid_constant__ TmaMaps maps, PipeParams P, PtrArray
                 // pass B needs its worker-block's tiles (fused scales: the block's M, which
                 // implies them); pass A needs the previous tenant of its ring slot consumed
                 const uint32_t *ctr = !t.is_b ? &pc->b_done[t.slot].v
-                                      : kFused ? &pc->a_done[16u + (r & 15u)].v : &pc->a_done[t.slot].v;
-                const uint32_t target = !t.is_b ? t.gen * T : kFused ? r / 16u + 1u : (t.gen + 1) * T;
+                                      : kFused ? &pc->a_done[kFusedBlocks + r % kFusedBlocks].v : &pc->a_done[t.slot].v;
+                const uint32_t target = !t.is_b ? t.gen * T : kFused ? r / kFusedBlocks + 1u : (t.gen + 1) * T;
                 if (target != 0) {
                     have = false;
                     bool expired = true;
