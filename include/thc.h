@@ -20,7 +20,7 @@
  *     pointers; the library copies them into kernel arguments, so they may be freed or
  *     reused as soon as the call returns.
  *   - Every device buffer is owned by the caller.  Device buffers must be 16-byte aligned.
- *     The library owns only the context (some 45 KB of device memory for the
+ *     The library owns only the context (some 80 KB of device memory for the
  *     status word and scheduling counters, allocated by thc_create).
  *   - The round calls (and thc_quantize_rotated, thc_prepare_compress, thc_prepare_minmax,
  *     thc_error_feedback, thc_accumulate_error) only enqueue work on `stream`

@@ -570,26 +570,12 @@ prepare_final_kernel(const double *__restrict__ partial, uint32_t n, uint64_t nb
     store_scale(ell, t_p, k, blk, scales, dev);
 }
 
-// Exact range (Algorithm 1's preliminary stage on the rotated coordinates): keys start at
-// (+max, 0); afterwards they become nblocks minima followed by nblocks maxima in `scales`.
-// A block with a non-finite rotated coordinate gets (0, 0) and THC_STATUS_NONFINITE.
-__global__ void range_init_kernel(uint32_t *keys, uint64_t nblocks)
+// Exact range (Algorithm 1's preliminary stage on the rotated coordinates) of more blocks than the context
+// has keys for: keys in the workspace, cleared before and turned into the ranges after the transform.
+__global__ void range_final_kernel(uint32_t *keys, uint64_t nblocks, float *scales, DeviceBlock *dev)
 {
-    const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < nblocks) { keys[i] = 0xFFFFFFFFu; keys[nblocks + i] = 0u; }
-}
-
-__global__ void range_final_kernel(const uint32_t *keys, uint64_t nblocks, float *scales, DeviceBlock *dev)
-{
-    const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= nblocks) return;
-    float lo = key_float(keys[i]), hi = key_float(keys[nblocks + i]);
-    uint32_t flags = 0;
-    if (!isfinite(lo) || !isfinite(hi)) { lo = 0.0f; hi = 0.0f; flags |= THC_STATUS_NONFINITE; }
-    if (hi == 0.0f && lo == 0.0f) flags |= THC_STATUS_ZERO_BLOCK;   // a constant block decodes exactly
-    scales[i] = lo;
-    scales[nblocks + i] = hi;
-    if (flags) atomicOr(&dev->status, flags);
+    const uint64_t r = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (r < nblocks) finish_range(keys, nblocks, r, scales, dev);
 }
 
 // ---------------------------------------------------------------------------- aggregate
@@ -1176,7 +1162,8 @@ static int launch_pipeline(const thc_ctx *ctx, pipe_kernel_t kern, bool compress
                            const thc_sizes_t &sz, uint64_t d, uint32_t n_local, uint32_t worker_base, uint32_t round, uint32_t divisor,
                            const float *scales, void *workspace, const PtrArrayP &in,
                            const MutPtrArrayP &out, const MutPtrArrayP &rot, cudaStream_t st,
-                           float *fused_scales_out = nullptr, bool compress_bf16 = false, uint32_t agg_n = 0)
+                           float *fused_scales_out = nullptr, bool compress_bf16 = false, uint32_t agg_n = 0,
+                           uint32_t *range_keys = nullptr, float *range_out = nullptr)
 {
     const uint32_t k = ctx->cfg.log2_block;
     PipeParams P;
@@ -1190,8 +1177,6 @@ static int launch_pipeline(const thc_ctx *ctx, pipe_kernel_t kern, bool compress
     PipePlan pl = plan_pipeline(ctx, P.wb_count);
     // Compress of 2^22 blocks: pass B trails by two worker-blocks in a ring of four slots
     // (64 MB stay in L2 better than the planned six slots of 16 MB; the workspace holds those).
-    // The exact-range keys stay where the planned ring ends: thc_prepare_minmax looks there.
-    const uint32_t planned_ring = pl.ring;
     if ((compress_f32 || compress_bf16) && k == 22 && pl.ring > 4) { pl.lag = 2; pl.ring = 4; }
     if (fused_scales_out != nullptr) {
         if (!plan_pipeline_fused(ctx, sz.nblocks, n_local, &pl)) return THC_EUNSUPPORTED;
@@ -1218,8 +1203,8 @@ static int launch_pipeline(const thc_ctx *ctx, pipe_kernel_t kern, bool compress
     P.nblocks = (uint32_t)sz.nblocks;
     P.agg_n = agg_n;
     P.agg_acc_bits = ctx->acc_bits;
-    P.range_keys = reinterpret_cast<uint32_t *>(static_cast<unsigned char *>(workspace) +
-                                                ((uint64_t)planned_ring << k) * 4);
+    P.range_keys = range_keys;
+    P.range_out = range_out;
     const uint64_t nblk_cached = sz.nblocks < (uint64_t)kBlockConstMax ? sz.nblocks : (uint64_t)kBlockConstMax;
     const size_t smem = (size_t)1024 + (size_t)2 * kPElems * 4 + kPSignWords * 4 +
                         (size_t)(ctx->cfg.granularity + 1) * kLutEntryBytes + (size_t)nblk_cached * 8;
@@ -1281,7 +1266,7 @@ static bool use_block_kernel(const thc_ctx *ctx, uint64_t coords)
 static int launch_block(const thc_ctx *ctx, const void *kern, PipeMode mode, size_t lut_bytes, const thc_sizes_t &sz,
                         uint64_t d, uint32_t n_local, uint32_t worker_base, uint32_t round, uint32_t divisor,
                         const float *scales, const PtrArrayP &in, const MutPtrArrayP &out, const MutPtrArrayP &rot,
-                        cudaStream_t st, uint32_t *keys = nullptr, uint32_t agg_n = 0)
+                        cudaStream_t st, uint32_t *keys = nullptr, uint32_t agg_n = 0, float *range_out = nullptr)
 {
     const uint32_t k = ctx->cfg.log2_block;
     BlockParams P;
@@ -1306,6 +1291,8 @@ static int launch_block(const thc_ctx *ctx, const void *kern, PipeMode mode, siz
     P.nblocks = (uint32_t)sz.nblocks;
     P.const_slots = k < tile_log2 ? 1u << (tile_log2 - k) : 1u;
     P.range_keys = keys;
+    P.range_out = range_out;
+    P.exited = &reinterpret_cast<PipeCounters *>(ctx->dev->counters)->exited;
     P.agg_n = agg_n;
     P.agg_chunk = 255u / ctx->cfg.granularity;
     P.agg_acc_bits = ctx->acc_bits;
@@ -1366,14 +1353,18 @@ int thc_prepare_minmax(thc_ctx *ctx, const void *const *grads, uint32_t n, uint6
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const uint32_t k = ctx->cfg.log2_block;
     const bool in_block = use_block_kernel(ctx, sz.d_pad * n);
-    uint32_t *keys = static_cast<uint32_t *>(workspace);
-    if (!in_block) {
-        const PipePlan pl = plan_pipeline(ctx, sz.nblocks * n);
-        keys = reinterpret_cast<uint32_t *>(static_cast<unsigned char *>(workspace) + ((uint64_t)pl.ring << k) * 4);
+    // up to kPrepCounters blocks the keys are the context's own, zero between calls, and the last CTA
+    // of the transform writes the ranges: one launch (three took 3.7 us more on 65 blocks)
+    const bool own_keys = sz.nblocks <= (uint64_t)kPrepCounters;
+    uint32_t *keys = own_keys ? ctx->dev->range_keys : static_cast<uint32_t *>(workspace);
+    if (!own_keys) {
+        if (!in_block) {
+            const PipePlan pl = plan_pipeline(ctx, sz.nblocks * n);
+            keys = reinterpret_cast<uint32_t *>(static_cast<unsigned char *>(workspace) + ((uint64_t)pl.ring << k) * 4);
+        }
+        THC_CUDA(cudaMemsetAsync(keys, 0, sz.nblocks * 8, st));
     }
-    const unsigned init_blocks = (unsigned)((sz.nblocks + 255) / 256);
-    range_init_kernel<<<init_blocks, 256, 0, st>>>(keys, sz.nblocks);
-    THC_CUDA(cudaGetLastError());
+    float *range_out = own_keys ? scales : nullptr;
     int rc;
     PtrArrayP pin;
     MutPtrArrayP pout, prot;
@@ -1389,13 +1380,15 @@ int thc_prepare_minmax(thc_ctx *ctx, const void *const *grads, uint32_t n, uint6
     }
     if (in_block)
         rc = launch_block(ctx, block_kernel(kRangeF32, 4, true, ctx->cfg.log2_block), kRangeF32, 0, sz, d, n, 0, round, 1, scales, pin, pout,
-                          prot, st, keys);
+                          prot, st, keys, 0, range_out);
     else
         rc = launch_pipeline(ctx, pick_pipe_kernel<kRangeF32>(4, true, k), true, sz, d, n, 0, round,
-                             1, scales, workspace, pin, pout, prot, st);
+                             1, scales, workspace, pin, pout, prot, st, nullptr, false, 0, keys, range_out);
     if (rc != THC_OK) return rc;
-    range_final_kernel<<<init_blocks, 256, 0, st>>>(keys, sz.nblocks, scales, ctx->dev);
-    THC_CUDA(cudaGetLastError());
+    if (!own_keys) {
+        range_final_kernel<<<(unsigned)((sz.nblocks + 255) / 256), 256, 0, st>>>(keys, sz.nblocks, scales, ctx->dev);
+        THC_CUDA(cudaGetLastError());
+    }
     return THC_OK;
 }
 

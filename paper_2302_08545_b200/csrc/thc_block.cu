@@ -699,10 +699,7 @@ thc_block_kernel(const __grid_constant__ TmaMaps maps, const __grid_constant__ B
                                 lo = __reduce_min_sync(0xFFFFFFFFu, lo);
                                 hi = __reduce_max_sync(0xFFFFFFFFu, hi);
                             }
-                            if (j < P.d_pad && (k < 8u || lane == 0)) {
-                                atomicMin(P.range_keys + (j >> k), lo);
-                                atomicMax(P.range_keys + P.nblocks + (j >> k), hi);
-                            }
+                            if (j < P.d_pad && (k < 8u || lane == 0)) add_range(P.range_keys, P.nblocks, j >> k, lo, hi);
                         }
                     } else {
                         const float2 kc = bc[KIND != 0 ? 0u : ((32u * rl + 8u * u + off) >> k)];
@@ -745,10 +742,19 @@ thc_block_kernel(const __grid_constant__ TmaMaps maps, const __grid_constant__ B
         if (kRange && (KIND != 0 || k >= (uint32_t)kBLog2)) {
             kmin = __reduce_min_sync(0xFFFFFFFFu, kmin);
             kmax = __reduce_max_sync(0xFFFFFFFFu, kmax);
-            if (lane == 0) {
-                atomicMin(P.range_keys + (j_out >> k), kmin);
-                atomicMax(P.range_keys + P.nblocks + (j_out >> k), kmax);
-            }
+            if (lane == 0) add_range(P.range_keys, P.nblocks, j_out >> k, kmin, kmax);
+        }
+    }
+    if (kRange && P.range_out != nullptr) {
+        __shared__ uint32_t s_left;
+        __threadfence();
+        __syncthreads();
+        if (thread == 0) s_left = atomicAdd(P.exited, 1u);
+        __syncthreads();
+        if (s_left == gridDim.x - 1) {
+            __threadfence();
+            finish_ranges(P.range_keys, P.nblocks, P.range_out, P.dev, thread, kBThreads);
+            if (thread == 0) *P.exited = 0u;
         }
     }
 }

@@ -27,6 +27,7 @@ struct DeviceBlock {
     uint32_t pad_[31];
     uint32_t counters[5632];     // scheduling counters (self-resetting), 128-byte aligned
     uint32_t prep_counters[kPrepCounters];     // chunks done per RHT block in thc_prepare (self-resetting)
+    uint32_t range_keys[2 * kPrepCounters];    // exact range, up to as many blocks (self-resetting)
     uint4    lut[256];           // by floor(u*g): (-T[z0] as float, 65536/(T[z0+1]-T[z0]), z0, 0)
     uint32_t table[256];         // T
 };
@@ -112,6 +113,33 @@ __device__ __forceinline__ uint32_t float_key(float f)
 __device__ __forceinline__ float key_float(uint32_t k)
 {
     return __uint_as_float(k ^ ((k >> 31) ? 0x80000000u : 0xFFFFFFFFu));
+}
+
+// Exact range: the keys are nblocks complements of the smallest key, then nblocks largest keys, so that
+// both start at 0 and are raised by atomicMax.
+__device__ __forceinline__ void add_range(uint32_t *keys, uint64_t nblocks, uint64_t r, uint32_t kmin, uint32_t kmax)
+{
+    atomicMax(keys + r, ~kmin);
+    atomicMax(keys + nblocks + r, kmax);
+}
+
+// The keys of block r become its minimum and maximum in `scales` and are 0 again.  A block with a
+// non-finite rotated coordinate gets (0, 0) and THC_STATUS_NONFINITE.
+__device__ __forceinline__ void finish_range(uint32_t *keys, uint64_t nblocks, uint64_t r, float *scales, DeviceBlock *dev)
+{
+    float lo = key_float(~__ldcg(keys + r)), hi = key_float(__ldcg(keys + nblocks + r));
+    keys[r] = 0u;
+    keys[nblocks + r] = 0u;
+    uint32_t flags = 0;
+    if (!isfinite(lo) || !isfinite(hi)) { lo = 0.0f; hi = 0.0f; flags |= THC_STATUS_NONFINITE; }
+    if (hi == 0.0f && lo == 0.0f) flags |= THC_STATUS_ZERO_BLOCK;   // a constant block decodes exactly
+    scales[r] = lo;
+    scales[nblocks + r] = hi;
+    if (flags) atomicOr(&dev->status, flags);
+}
+__device__ __forceinline__ void finish_ranges(uint32_t *keys, uint64_t nblocks, float *scales, DeviceBlock *dev, int tid, int threads)
+{
+    for (uint64_t r = tid; r < nblocks; r += threads) finish_range(keys, nblocks, r, scales, dev);
 }
 
 // ---------------------------------------------------------------- packed fp32 arithmetic

@@ -110,7 +110,8 @@ struct PipeParams {
     double   t_p;
     uint32_t exact_range;      // scales = nblocks minima then nblocks maxima (else M per block)
     uint32_t nblocks;
-    uint32_t *range_keys;      // range mode: nblocks min keys then nblocks max keys
+    uint32_t *range_keys;      // range mode: see add_range
+    float   *range_out;        // ... finished by the last CTA (or null: by range_final_kernel)
     uint32_t b_swz_mask;       // run-time geometry, pass-B tiles: chunk c sits at c ^ ((c >> 3) & mask)
     uint32_t agg_n;            // kAggDecompress: workers whose table values are summed
     uint32_t agg_acc_bits;     // ... and the width of the sums written on request (outp.p[1])
@@ -1527,10 +1528,7 @@ thc_pipeline_kernel(const __grid_constant__ TmaMaps maps, PipeParams P, PtrArray
                 if (kRange) {
                     kmin = __reduce_min_sync(0xFFFFFFFFu, kmin);
                     kmax = __reduce_max_sync(0xFFFFFFFFu, kmax);
-                    if ((tid & 31) == 0) {
-                        atomicMin(P.range_keys + r, kmin);
-                        atomicMax(P.range_keys + P.nblocks + r, kmax);
-                    }
+                    if ((tid & 31) == 0) add_range(P.range_keys, P.nblocks, r, kmin, kmax);
                 }
             }
             // Finished: tell the control warp (it signals the completion to the other CTAs),
@@ -1545,17 +1543,25 @@ thc_pipeline_kernel(const __grid_constant__ TmaMaps maps, PipeParams P, PtrArray
     }
     __syncthreads();
 
-    // ---- leave: the last CTA clears the counters for the next launch
+    // ---- leave: the last CTA clears the counters for the next launch (and finishes the ranges)
+    __shared__ uint32_t s_left;
     if (tid == 0) {
         __threadfence();
-        const uint32_t left = atomicAdd(&pc->exited, 1u);
-        if (left == gridDim.x - 1) {
-            for (int sl = 0; sl < kMaxRing; ++sl) { pc->a_done[sl].v = 0; pc->b_done[sl].v = 0; }
+        s_left = atomicAdd(&pc->exited, 1u);
+    }
+    __syncthreads();
+    if (s_left == gridDim.x - 1) {
+        __threadfence();
+        const uint32_t used = kFused ? max(P.ring_slots, 2u * kFusedBlocks) : P.ring_slots;
+        for (uint32_t sl = tid; sl < used; sl += kPCtaThreads) { pc->a_done[sl].v = 0; pc->b_done[sl].v = 0; }
+        if (kRange && P.range_out != nullptr) finish_ranges(P.range_keys, P.nblocks, P.range_out, P.dev, tid, kPCtaThreads);
+        if (tid == 0) {
             pc->abort = 0;
             pc->head = 0;
-            __threadfence();
-            pc->exited = 0;
         }
+        __threadfence();
+        __syncthreads();
+        if (tid == 0) pc->exited = 0;
     }
 }
 
