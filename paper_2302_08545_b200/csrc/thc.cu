@@ -24,7 +24,7 @@ template <int BITS, bool IDENTITY>
 __global__ void __launch_bounds__(kThreads)
 quantize_rotated_kernel(PtrArray rotated, MutPtrArray packed, uint64_t d_pad, uint32_t k,
                         uint32_t granularity, uint32_t round, uint32_t worker_base, uint32_t exact_range,
-                        const float *__restrict__ scales, const DeviceBlock *dev, PhiloxKeys keys)
+                        const float *scales, const DeviceBlock *dev, PhiloxKeys keys)
 {
     // dynamic shared memory: the quantiser table, one copy per lane group, then the block
     // constants of the first kQrBlockCache RHT blocks (the fp64 division is done once per block)
@@ -32,6 +32,7 @@ quantize_rotated_kernel(PtrArray rotated, MutPtrArray packed, uint64_t d_pad, ui
     unsigned char *lut = qr_smem;
     float2 *bc = reinterpret_cast<float2 *>(qr_smem + (size_t)(granularity + 1) * kLutEntryBytes);
     if (!IDENTITY) lut_fill<LutKind<BITS, IDENTITY>::k8>(lut, dev, granularity, threadIdx.x, kThreads);
+    depend_on_previous();
     const uint64_t nblocks = d_pad >> k;
     const uint32_t cached = nblocks < (uint64_t)kQrBlockCache ? (uint32_t)nblocks : (uint32_t)kQrBlockCache;
     for (uint32_t b = threadIdx.x; b < cached; b += kThreads)
@@ -45,8 +46,8 @@ quantize_rotated_kernel(PtrArray rotated, MutPtrArray packed, uint64_t d_pad, ui
     for (uint64_t u = (uint64_t)blockIdx.x * kThreads + threadIdx.x; u < d_pad / 8;
          u += (uint64_t)gridDim.x * kThreads) {
         const uint64_t j = u * 8;
-        const float4 a = __ldg(reinterpret_cast<const float4 *>(rot + j));
-        const float4 b = __ldg(reinterpret_cast<const float4 *>(rot + j + 4));
+        const float4 a = ld_global_once(reinterpret_cast<const float4 *>(rot + j));
+        const float4 b = ld_global_once(reinterpret_cast<const float4 *>(rot + j + 4));
         const float r[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
         const uint64_t blk = j >> k;
         const float2 kc = blk < cached ? bc[blk] : compress_constants(block_range(scales, blk, nblocks, exact_range));
@@ -86,6 +87,7 @@ aggregate_b4w8_kernel(PtrArray in, uint32_t n, uint64_t units32, const DeviceBlo
     for (int q = 0; q < 4; ++q)
         t[q] = dev->table[4 * q] | (dev->table[4 * q + 1] << 8) | (dev->table[4 * q + 2] << 16) |
                (dev->table[4 * q + 3] << 24);
+    depend_on_previous();
     const bool aligned32 = (reinterpret_cast<uintptr_t>(sum) & 31u) == 0;
     // A thread sums 32 coordinates: 16 bytes of indices per worker, the loads of up to eight
     // workers in flight together, 32 bytes of sums out.
@@ -97,7 +99,7 @@ aggregate_b4w8_kernel(PtrArray in, uint32_t n, uint64_t units32, const DeviceBlo
             uint4 w[8];
 #pragma unroll
             for (int j = 0; j < 8; ++j)         // index 0 everywhere adds T[0] = 0
-                w[j] = i0 + j < n ? __ldcs(reinterpret_cast<const uint4 *>(in.p[i0 + j]) + u) : make_uint4(0u, 0u, 0u, 0u);
+                w[j] = i0 + j < n ? ld_global_once(reinterpret_cast<const uint4 *>(in.p[i0 + j]) + u) : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
                 const uint32_t words[4] = {w[j].x, w[j].y, w[j].z, w[j].w};
@@ -126,6 +128,7 @@ aggregate_b4w16_kernel(PtrArray in, uint32_t n, uint64_t units32, const DeviceBl
     for (int q = 0; q < 4; ++q)
         t[q] = dev->table[4 * q] | (dev->table[4 * q + 1] << 8) | (dev->table[4 * q + 2] << 16) |
                (dev->table[4 * q + 3] << 24);
+    depend_on_previous();
     const bool aligned32 = (reinterpret_cast<uintptr_t>(sum) & 31u) == 0;
     // A thread sums 32 coordinates: 16 bytes of indices per worker, 64 bytes of sums out.
     for (uint64_t u = (uint64_t)blockIdx.x * kThreads + threadIdx.x; u < units32;
@@ -136,7 +139,7 @@ aggregate_b4w16_kernel(PtrArray in, uint32_t n, uint64_t units32, const DeviceBl
             uint4 w[CHUNK];
 #pragma unroll
             for (int j = 0; j < CHUNK; ++j)      // index 0 everywhere adds T[0] = 0
-                w[j] = i0 + j < n ? __ldcs(reinterpret_cast<const uint4 *>(in.p[i0 + j]) + u) : make_uint4(0u, 0u, 0u, 0u);
+                w[j] = i0 + j < n ? ld_global_once(reinterpret_cast<const uint4 *>(in.p[i0 + j]) + u) : make_uint4(0u, 0u, 0u, 0u);
             uint32_t acc[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
 #pragma unroll
             for (int j = 0; j < CHUNK; ++j) {
@@ -177,6 +180,7 @@ __global__ void __launch_bounds__(kThreads)
 aggregate_small_w8_kernel(PtrArray in, uint32_t n, uint64_t units32, uint32_t g_mult,
                           uint4 *__restrict__ sum)
 {
+    depend_on_previous();
     constexpr int kWords = BITS;                       // 32 coordinates = BITS words
     constexpr int kSpread = 8 / BITS;                  // spreads per word
     constexpr uint32_t kMask = BITS == 1 ? 0x01010101u : 0x03030303u;
@@ -191,9 +195,9 @@ aggregate_small_w8_kernel(PtrArray in, uint32_t n, uint64_t units32, uint32_t g_
         for (uint32_t i = 0; i < n; ++i) {
             uint32_t words[kWords];
             if constexpr (BITS == 1) {
-                words[0] = __ldg(reinterpret_cast<const uint32_t *>(in.p[i]) + u);
+                words[0] = ld_global(reinterpret_cast<const uint32_t *>(in.p[i]) + u);
             } else {
-                const uint2 w = __ldg(reinterpret_cast<const uint2 *>(in.p[i]) + u);
+                const uint2 w = ld_global(reinterpret_cast<const uint2 *>(in.p[i]) + u);
                 words[0] = w.x; words[1] = w.y;
             }
 #pragma unroll
@@ -234,6 +238,7 @@ aggregate_b3_kernel(PtrArray in, uint32_t n, uint64_t units64, uint32_t chunk, c
 {
     const uint32_t t0 = dev->table[0] | (dev->table[1] << 8) | (dev->table[2] << 16) | (dev->table[3] << 24);
     const uint32_t t1 = dev->table[4] | (dev->table[5] << 8) | (dev->table[6] << 16) | (dev->table[7] << 24);
+    depend_on_previous();
     const bool aligned32 = (reinterpret_cast<uintptr_t>(sum) & 31u) == 0;
     for (uint64_t u = (uint64_t)blockIdx.x * 128 + threadIdx.x; u < units64; u += (uint64_t)gridDim.x * 128) {
         uint32_t wide[W == 16 ? 32 : 1];
@@ -250,7 +255,7 @@ aggregate_b3_kernel(PtrArray in, uint32_t n, uint64_t units64, uint32_t chunk, c
                 uint32_t w[7];
 #pragma unroll
                 for (int q = 0; q < 3; ++q) {
-                    const uint2 v = __ldg(reinterpret_cast<const uint2 *>(in.p[i]) + 3 * u + q);
+                    const uint2 v = ld_global(reinterpret_cast<const uint2 *>(in.p[i]) + 3 * u + q);
                     w[2 * q] = v.x; w[2 * q + 1] = v.y;
                 }
                 w[6] = 0u;
@@ -301,12 +306,13 @@ aggregate_b3_kernel(PtrArray in, uint32_t n, uint64_t units64, uint32_t chunk, c
 __global__ void __launch_bounds__(kThreads)
 aggregate_b8w16_kernel(PtrArray in, uint32_t n, uint64_t units16, uint4 *__restrict__ sum)
 {
+    depend_on_previous();
     for (uint64_t u = (uint64_t)blockIdx.x * kThreads + threadIdx.x; u < units16;
          u += (uint64_t)gridDim.x * kThreads) {
         uint32_t even[4] = {0u, 0u, 0u, 0u}, odd[4] = {0u, 0u, 0u, 0u};
 #pragma unroll 4
         for (uint32_t i = 0; i < n; ++i) {
-            const uint4 w = __ldg(reinterpret_cast<const uint4 *>(in.p[i]) + u);
+            const uint4 w = ld_global(reinterpret_cast<const uint4 *>(in.p[i]) + u);
             const uint32_t words[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
@@ -331,6 +337,7 @@ constexpr int kAccUnits = 4;
 __global__ void __launch_bounds__(kThreads)
 accumulate_kernel(MutPtrArray xs, PtrArray es, uint64_t d)
 {
+    depend_on_previous();
     float *x = static_cast<float *>(xs.p[blockIdx.y]);
     const float *e = static_cast<const float *>(es.p[blockIdx.y]);
     const uint64_t n4 = d / 4;
@@ -339,7 +346,7 @@ accumulate_kernel(MutPtrArray xs, PtrArray es, uint64_t d)
 #pragma unroll
     for (int i = 0; i < kAccUnits; ++i) {
         const uint64_t c = c0 + (uint64_t)i * kThreads;
-        if (c < n4) { a[i] = reinterpret_cast<float4 *>(x)[c]; b[i] = __ldg(reinterpret_cast<const float4 *>(e) + c); }
+        if (c < n4) { a[i] = reinterpret_cast<float4 *>(x)[c]; b[i] = ld_global_once(reinterpret_cast<const float4 *>(e) + c); }
     }
 #pragma unroll
     for (int i = 0; i < kAccUnits; ++i) {
@@ -366,13 +373,13 @@ __device__ __forceinline__ uint4 load_unit(const void *x, uint64_t j, uint64_t d
     uint4 q = make_uint4(0u, 0u, 0u, 0u);
     if (j + kPer <= d) {
         const char *p = static_cast<const char *>(x) + j * (16 / kPer);
-        asm("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(q.x), "=r"(q.y), "=r"(q.z), "=r"(q.w) : "l"(p));
+        asm volatile("ld.global.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(q.x), "=r"(q.y), "=r"(q.z), "=r"(q.w) : "l"(p));
     } else if (j < d) {
         uint32_t w[4] = {0u, 0u, 0u, 0u};
         for (int e = 0; e < kPer; ++e) {
             if (j + e >= d) break;
-            if (BF16) w[e >> 1] |= (uint32_t)__ldg(static_cast<const uint16_t *>(x) + j + e) << ((e & 1) * 16);
-            else w[e & 3] = __ldg(static_cast<const uint32_t *>(x) + j + e);
+            if (BF16) w[e >> 1] |= (uint32_t)ld_global(static_cast<const uint16_t *>(x) + j + e) << ((e & 1) * 16);
+            else w[e & 3] = ld_global(static_cast<const uint32_t *>(x) + j + e);
         }
         q = make_uint4(w[0], w[1], w[2], w[3]);
     }
@@ -419,6 +426,7 @@ __global__ void __launch_bounds__(kThreads)
 prepare_small_kernel(PtrArray in, uint32_t n, uint64_t d, uint64_t d_pad, uint32_t k, double t_p, float *__restrict__ scales,
                      DeviceBlock *dev)
 {
+    depend_on_previous();
     constexpr uint32_t kPerLog2 = BF16 ? 3u : 2u;
     constexpr int kSlabs = 1 << (9 - 5 - kPerLog2);
     __shared__ double s_warp[THC_MAX_WORKERS][kThreads / 32];
@@ -486,6 +494,7 @@ prepare_partial_kernel(PtrArray in, uint64_t d, uint32_t chunk_log2, uint64_t ch
                        double *__restrict__ partial, uint32_t *counters, uint32_t chunks_per_block, double t_p, uint32_t k,
                        float *__restrict__ scales, DeviceBlock *dev)
 {
+    depend_on_previous();
     constexpr uint32_t kPerLog2 = BF16 ? 3u : 2u;
     const uint64_t chunk = blockIdx.x;
     const uint32_t wl = blockIdx.y;
@@ -544,10 +553,11 @@ prepare_partial_kernel(PtrArray in, uint64_t d, uint32_t chunk_log2, uint64_t ch
 // one square root per worker, then the maximum over workers.  The order is fixed, so the
 // result does not depend on timing.  For more blocks than there are counters.
 __global__ void __launch_bounds__(128)
-prepare_final_kernel(const double *__restrict__ partial, uint32_t n, uint64_t nblocks,
+prepare_final_kernel(const double *partial, uint32_t n, uint64_t nblocks,
                      uint64_t chunks_per_block, uint64_t chunks_per_worker, double t_p, uint32_t k,
                      float *__restrict__ scales, DeviceBlock *dev)
 {
+    depend_on_previous();
     const uint64_t blk = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (blk >= nblocks) return;
@@ -574,6 +584,7 @@ prepare_final_kernel(const double *__restrict__ partial, uint32_t n, uint64_t nb
 // has keys for: keys in the workspace, cleared before and turned into the ranges after the transform.
 __global__ void range_final_kernel(uint32_t *keys, uint64_t nblocks, float *scales, DeviceBlock *dev)
 {
+    depend_on_previous();
     const uint64_t r = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (r < nblocks) finish_range(keys, nblocks, r, scales, dev);
 }
@@ -587,6 +598,7 @@ aggregate_kernel(PtrArray in, uint32_t n, uint64_t units, uint64_t d_pad, const 
 {
     __shared__ uint32_t T[256];
     for (int z = threadIdx.x; z < (1 << BITS); z += kThreads) T[z] = dev->table[z];
+    depend_on_previous();
     __syncthreads();
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         // coordinates past the last whole group of 32 (blocks of 8 or 16 coordinates only)
@@ -615,20 +627,20 @@ aggregate_kernel(PtrArray in, uint32_t n, uint64_t units, uint64_t d_pad, const 
                 static_cast<const unsigned char *>(in.p[i]) + u * (4 * BITS));
             uint32_t w[kInWords];
             if constexpr (BITS == 8) {
-                const uint4 a = __ldg(reinterpret_cast<const uint4 *>(src));
-                const uint4 b = __ldg(reinterpret_cast<const uint4 *>(src) + 1);
+                const uint4 a = ld_global(reinterpret_cast<const uint4 *>(src));
+                const uint4 b = ld_global(reinterpret_cast<const uint4 *>(src) + 1);
                 w[0] = a.x; w[1] = a.y; w[2] = a.z; w[3] = a.w;
                 w[4] = b.x; w[5] = b.y; w[6] = b.z; w[7] = b.w;
             } else if constexpr (BITS == 4) {
-                const uint4 a = __ldg(reinterpret_cast<const uint4 *>(src));
+                const uint4 a = ld_global(reinterpret_cast<const uint4 *>(src));
                 w[0] = a.x; w[1] = a.y; w[2] = a.z; w[3] = a.w;
             } else if constexpr (BITS == 3) {
-                w[0] = __ldg(src); w[1] = __ldg(src + 1); w[2] = __ldg(src + 2);
+                w[0] = ld_global(src); w[1] = ld_global(src + 1); w[2] = ld_global(src + 2);
             } else if constexpr (BITS == 2) {
-                const uint2 a = __ldg(reinterpret_cast<const uint2 *>(src));
+                const uint2 a = ld_global(reinterpret_cast<const uint2 *>(src));
                 w[0] = a.x; w[1] = a.y;
             } else {
-                w[0] = __ldg(src);
+                w[0] = ld_global(src);
             }
 #pragma unroll
             for (int e = 0; e < 32; ++e) {
@@ -702,11 +714,30 @@ static int cuda_fail(cudaError_t e)
     return THC_ECUDA;
 }
 
-#define THC_CUDA(call)                                        \
+#define THC_CUDA(...)                                         \
     do {                                                      \
-        cudaError_t e__ = (call);                             \
+        cudaError_t e__ = (__VA_ARGS__);                      \
         if (e__ != cudaSuccess) return cuda_fail(e__);        \
     } while (0)
+
+// A launch that may start while the one before it on the stream is still running (depend_on_previous):
+// 1 to 1.5 us less between two launches of a round.
+template <class... P, class... A>
+static cudaError_t launch_after(void (*kern)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st, A... args)
+{
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof cfg);
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, P(args)...);
+}
 
 static bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
@@ -977,9 +1008,8 @@ int thc_prepare(thc_ctx *ctx, const void *const *grads, uint32_t n, uint64_t d, 
     if (k <= (uint32_t)kSmallPrepLog2) {
         const uint64_t tiles = (sz.d_pad + (1u << kSmallPrepLog2) - 1) >> kSmallPrepLog2;
         if (tiles > 0x7FFFFFFFull) return THC_EUNSUPPORTED;
-        if (bf16) prepare_small_kernel<true><<<(unsigned)tiles, kThreads, 0, st>>>(in, n, d, sz.d_pad, k, t_p, scales, ctx->dev);
-        else prepare_small_kernel<false><<<(unsigned)tiles, kThreads, 0, st>>>(in, n, d, sz.d_pad, k, t_p, scales, ctx->dev);
-        THC_CUDA(cudaGetLastError());
+        if (bf16) THC_CUDA(launch_after(prepare_small_kernel<true>, dim3((unsigned)tiles), kThreads, 0, st, in, n, d, sz.d_pad, k, t_p, scales, ctx->dev));
+        else THC_CUDA(launch_after(prepare_small_kernel<false>, dim3((unsigned)tiles), kThreads, 0, st, in, n, d, sz.d_pad, k, t_p, scales, ctx->dev));
         return THC_OK;
     }
     const uint32_t chunk_log2 = k < (uint32_t)kChunkLog2 ? k : (uint32_t)kChunkLog2;
@@ -990,16 +1020,14 @@ int thc_prepare(thc_ctx *ctx, const void *const *grads, uint32_t n, uint64_t d, 
     uint32_t *counters = sz.nblocks <= (uint64_t)kPrepCounters ? ctx->dev->prep_counters : nullptr;
     const dim3 grid((unsigned)chunks_per_worker, n);
     if (bf16)
-        prepare_partial_kernel<true><<<grid, kThreads, 0, st>>>(in, d, chunk_log2, chunks_per_worker, partial, counters,
-                                                                chunks_per_block, t_p, k, scales, ctx->dev);
+        THC_CUDA(launch_after(prepare_partial_kernel<true>, grid, kThreads, 0, st, in, d, chunk_log2, chunks_per_worker, partial, counters,
+                                                                chunks_per_block, t_p, k, scales, ctx->dev));
     else
-        prepare_partial_kernel<false><<<grid, kThreads, 0, st>>>(in, d, chunk_log2, chunks_per_worker, partial, counters,
-                                                                 chunks_per_block, t_p, k, scales, ctx->dev);
-    THC_CUDA(cudaGetLastError());
+        THC_CUDA(launch_after(prepare_partial_kernel<false>, grid, kThreads, 0, st, in, d, chunk_log2, chunks_per_worker, partial, counters,
+                                                                 chunks_per_block, t_p, k, scales, ctx->dev));
     if (counters == nullptr) {
-        prepare_final_kernel<<<(unsigned)((sz.nblocks + 3) / 4), 128, 0, st>>>(
-            partial, n, sz.nblocks, chunks_per_block, chunks_per_worker, t_p, k, scales, ctx->dev);
-        THC_CUDA(cudaGetLastError());
+        THC_CUDA(launch_after(prepare_final_kernel, dim3((unsigned)((sz.nblocks + 3) / 4)), 128, 0, st, 
+            partial, n, sz.nblocks, chunks_per_block, chunks_per_worker, t_p, k, scales, ctx->dev));
     }
     return THC_OK;
 }
@@ -1251,8 +1279,7 @@ static int launch_pipeline(const thc_ctx *ctx, pipe_kernel_t kern, bool compress
             if (rc != THC_OK) return rc;
         }
     }
-    kern<<<pl.grid, kPCtaThreads, smem, st>>>(maps, P, in, out, rot, ctx->keys);
-    THC_CUDA(cudaGetLastError());
+    THC_CUDA(launch_after(kern, dim3(pl.grid), kPCtaThreads, smem, st, maps, P, in, out, rot, ctx->keys));
     return THC_OK;
 }
 
@@ -1310,18 +1337,20 @@ static int launch_block(const thc_ctx *ctx, const void *kern, PipeMode mode, siz
     const uint32_t ctas_per_sm = tile_log2 == 13u ? 4u : 2u;
     const uint32_t resident = ((uint32_t)ctx->sm_count * ctas_per_sm) >> e;       // clusters (CTAs where e = 0)
     const uint32_t grid = (P.tasks < resident ? P.tasks : resident) << e;
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = 1u << e;
-    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = 1u << e;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof cfg);
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3((unsigned)(tile / 64));
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cfg.attrs = &attr;
-    cfg.numAttrs = e != 0u ? 1 : 0;
+    cfg.attrs = attr;
+    cfg.numAttrs = e != 0u ? 2 : 1;
     void *args[] = {&maps, &P, const_cast<PtrArrayP *>(&in), const_cast<MutPtrArrayP *>(&out), const_cast<MutPtrArrayP *>(&rot),
                     const_cast<PhiloxKeys *>(&ctx->keys)};
     THC_CUDA(cudaLaunchKernelExC(&cfg, kern, args));
@@ -1386,8 +1415,7 @@ int thc_prepare_minmax(thc_ctx *ctx, const void *const *grads, uint32_t n, uint6
                              1, scales, workspace, pin, pout, prot, st, nullptr, false, 0, keys, range_out);
     if (rc != THC_OK) return rc;
     if (!own_keys) {
-        range_final_kernel<<<(unsigned)((sz.nblocks + 255) / 256), 256, 0, st>>>(keys, sz.nblocks, scales, ctx->dev);
-        THC_CUDA(cudaGetLastError());
+        THC_CUDA(launch_after(range_final_kernel, dim3((unsigned)((sz.nblocks + 255) / 256)), 256, 0, st, keys, sz.nblocks, scales, ctx->dev));
     }
     return THC_OK;
 }
@@ -1599,9 +1627,9 @@ int thc_quantize_rotated(thc_ctx *ctx, const float *const *rotated, uint32_t n_l
     const dim3 grid((unsigned)blocks, n_local);
     const uint32_t k = ctx->cfg.log2_block, g = ctx->cfg.granularity;
     const size_t qr_smem = (size_t)(g + 1) * kLutEntryBytes + (size_t)kQrBlockCache * 8;
-#define THC_QR(B, I) quantize_rotated_kernel<B, I><<<grid, kThreads, qr_smem, st>>>( \
+#define THC_QR(B, I) THC_CUDA(launch_after(quantize_rotated_kernel<B, I>, grid, kThreads, qr_smem, st, \
         in, out, sz.d_pad, k, g, round, worker_base,                         \
-        ctx->cfg.range_mode == THC_RANGE_MINMAX ? 1u : 0u, scales, ctx->dev, ctx->keys)
+        ctx->cfg.range_mode == THC_RANGE_MINMAX ? 1u : 0u, scales, ctx->dev, ctx->keys))
     switch (ctx->cfg.bits) {
     case 1: if (ctx->identity) THC_QR(1, true); else THC_QR(1, false); break;
     case 2: if (ctx->identity) THC_QR(2, true); else THC_QR(2, false); break;
@@ -1610,7 +1638,6 @@ int thc_quantize_rotated(thc_ctx *ctx, const float *const *rotated, uint32_t n_l
     default: if (ctx->identity) THC_QR(8, true); else THC_QR(8, false); break;
     }
 #undef THC_QR
-    THC_CUDA(cudaGetLastError());
     return THC_OK;
 }
 
@@ -1639,9 +1666,8 @@ int thc_aggregate(thc_ctx *ctx, const void *const *packed, uint32_t n, uint64_t 
         uint64_t nb = (units32 + kThreads - 1) / kThreads;
         const uint64_t cap32 = (uint64_t)ctx->sm_count * 64;     // a unit or two per thread: no uneven tail
         if (nb > cap32) nb = cap32;
-        aggregate_b4w8_kernel<<<(unsigned)nb, kThreads, 0, st>>>(in, n, units32, ctx->dev,
-                                                                  reinterpret_cast<uint4 *>(s));
-        THC_CUDA(cudaGetLastError());
+        THC_CUDA(launch_after(aggregate_b4w8_kernel, dim3((unsigned)nb), kThreads, 0, st, in, n, units32, ctx->dev,
+                                                                  reinterpret_cast<uint4 *>(s)));
         return THC_OK;
     }
     const uint32_t bits = ctx->cfg.bits, g = ctx->cfg.granularity, w = ctx->acc_bits;
@@ -1650,10 +1676,9 @@ int thc_aggregate(thc_ctx *ctx, const void *const *packed, uint32_t n, uint64_t 
         uint64_t nb = (units32 + kThreads - 1) / kThreads;
         if (nb > (uint64_t)ctx->sm_count * 64) nb = (uint64_t)ctx->sm_count * 64;
         uint4 *s4 = reinterpret_cast<uint4 *>(s);
-        if (g <= 31) aggregate_b4w16_kernel<8><<<(unsigned)nb, kThreads, 0, st>>>(in, n, units32, ctx->dev, s4);
-        else if (g <= 63) aggregate_b4w16_kernel<4><<<(unsigned)nb, kThreads, 0, st>>>(in, n, units32, ctx->dev, s4);
-        else aggregate_b4w16_kernel<2><<<(unsigned)nb, kThreads, 0, st>>>(in, n, units32, ctx->dev, s4);
-        THC_CUDA(cudaGetLastError());
+        if (g <= 31) THC_CUDA(launch_after(aggregate_b4w16_kernel<8>, dim3((unsigned)nb), kThreads, 0, st, in, n, units32, ctx->dev, s4));
+        else if (g <= 63) THC_CUDA(launch_after(aggregate_b4w16_kernel<4>, dim3((unsigned)nb), kThreads, 0, st, in, n, units32, ctx->dev, s4));
+        else THC_CUDA(launch_after(aggregate_b4w16_kernel<2>, dim3((unsigned)nb), kThreads, 0, st, in, n, units32, ctx->dev, s4));
         return THC_OK;
     }
     if ((bits == 1 || (bits == 2 && ctx->identity)) && w == 8 && sz.d_pad % 32 == 0) {
@@ -1661,12 +1686,11 @@ int thc_aggregate(thc_ctx *ctx, const void *const *packed, uint32_t n, uint64_t 
         uint64_t nb = (units32 + kThreads - 1) / kThreads;
         if (nb > (uint64_t)ctx->sm_count * 8) nb = (uint64_t)ctx->sm_count * 8;
         if (bits == 1)
-            aggregate_small_w8_kernel<1><<<(unsigned)nb, kThreads, 0, st>>>(in, n, units32, g,
-                                                                            reinterpret_cast<uint4 *>(s));
+            THC_CUDA(launch_after(aggregate_small_w8_kernel<1>, dim3((unsigned)nb), kThreads, 0, st, in, n, units32, g,
+                                                                            reinterpret_cast<uint4 *>(s)));
         else
-            aggregate_small_w8_kernel<2><<<(unsigned)nb, kThreads, 0, st>>>(in, n, units32, 1u,
-                                                                            reinterpret_cast<uint4 *>(s));
-        THC_CUDA(cudaGetLastError());
+            THC_CUDA(launch_after(aggregate_small_w8_kernel<2>, dim3((unsigned)nb), kThreads, 0, st, in, n, units32, 1u,
+                                                                            reinterpret_cast<uint4 *>(s)));
         return THC_OK;
     }
     if (bits == 3 && w <= 16 && sz.d_pad % 64 == 0) {
@@ -1675,20 +1699,18 @@ int thc_aggregate(thc_ctx *ctx, const void *const *packed, uint32_t n, uint64_t 
         if (nb > (uint64_t)ctx->sm_count * 64) nb = (uint64_t)ctx->sm_count * 64;
         uint4 *s4 = reinterpret_cast<uint4 *>(s);
         const uint32_t chunk = w == 8 ? n : 255u / g;
-        if (w == 8) aggregate_b3_kernel<8><<<(unsigned)nb, 128, 0, st>>>(in, n, units64, chunk, ctx->dev, s4);
-        else aggregate_b3_kernel<16><<<(unsigned)nb, 128, 0, st>>>(in, n, units64, chunk, ctx->dev, s4);
-        THC_CUDA(cudaGetLastError());
+        if (w == 8) THC_CUDA(launch_after(aggregate_b3_kernel<8>, dim3((unsigned)nb), 128, 0, st, in, n, units64, chunk, ctx->dev, s4));
+        else THC_CUDA(launch_after(aggregate_b3_kernel<16>, dim3((unsigned)nb), 128, 0, st, in, n, units64, chunk, ctx->dev, s4));
         return THC_OK;
     }
     if (bits == 8 && ctx->identity && w == 16 && sz.d_pad % 16 == 0) {
         const uint64_t units16 = sz.d_pad / 16;
         uint64_t nb = (units16 + kThreads - 1) / kThreads;
         if (nb > (uint64_t)ctx->sm_count * 8) nb = (uint64_t)ctx->sm_count * 8;
-        aggregate_b8w16_kernel<<<(unsigned)nb, kThreads, 0, st>>>(in, n, units16, reinterpret_cast<uint4 *>(s));
-        THC_CUDA(cudaGetLastError());
+        THC_CUDA(launch_after(aggregate_b8w16_kernel, dim3((unsigned)nb), kThreads, 0, st, in, n, units16, reinterpret_cast<uint4 *>(s)));
         return THC_OK;
     }
-#define THC_AG(B, W) aggregate_kernel<B, W><<<(unsigned)blocks, kThreads, 0, st>>>(in, n, units, sz.d_pad, ctx->dev, s)
+#define THC_AG(B, W) THC_CUDA(launch_after(aggregate_kernel<B, W>, dim3((unsigned)blocks), kThreads, 0, st, in, n, units, sz.d_pad, ctx->dev, s))
 #define THC_AGW(B)                                       \
     do {                                                 \
         if (ctx->acc_bits == 8) THC_AG(B, 8);            \
@@ -1704,7 +1726,6 @@ int thc_aggregate(thc_ctx *ctx, const void *const *packed, uint32_t n, uint64_t 
     }
 #undef THC_AGW
 #undef THC_AG
-    THC_CUDA(cudaGetLastError());
     return THC_OK;
 }
 
@@ -1771,8 +1792,7 @@ int thc_accumulate_error(thc_ctx *ctx, float *const *grads, const float *const *
     const uint32_t per_launch = apart ? n_local : 1u;
     for (uint32_t i0 = 0; i0 < n_local; i0 += per_launch) {
         for (uint32_t i = 0; i < per_launch; ++i) { x.p[i] = grads[i0 + i]; e.p[i] = ef[i0 + i]; }
-        accumulate_kernel<<<dim3((unsigned)(blocks ? blocks : 1), per_launch), kThreads, 0, st>>>(x, e, d);
-        THC_CUDA(cudaGetLastError());
+        THC_CUDA(launch_after(accumulate_kernel, dim3((unsigned)(blocks ? blocks : 1), per_launch), kThreads, 0, st, x, e, d));
     }
     return THC_OK;
 }

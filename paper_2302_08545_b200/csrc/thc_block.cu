@@ -193,15 +193,15 @@ __device__ __forceinline__ void low_round_inverse(float4 *wtile, const unsigned 
             if constexpr (IN_BITS >= 4) {
 #pragma unroll
                 for (int q = 0; q < IN_BITS / 4; ++q) {
-                    const uint4 t4 = __ldg(reinterpret_cast<const uint4 *>(p) + q);
+                    const uint4 t4 = ld_global(reinterpret_cast<const uint4 *>(p) + q);
                     w[4 * q] = t4.x; w[4 * q + 1] = t4.y; w[4 * q + 2] = t4.z; w[4 * q + 3] = t4.w;
                 }
             } else if constexpr (IN_BITS == 2) {
-                const uint2 t2 = __ldg(reinterpret_cast<const uint2 *>(p));
+                const uint2 t2 = ld_global(reinterpret_cast<const uint2 *>(p));
                 w[0] = t2.x; w[1] = t2.y;
             } else {
 #pragma unroll
-                for (int q = 0; q < IN_BITS; ++q) w[q] = __ldg(reinterpret_cast<const uint32_t *>(p) + q);
+                for (int q = 0; q < IN_BITS; ++q) w[q] = ld_global(reinterpret_cast<const uint32_t *>(p) + q);
             }
         } else if (row * 32 < coords) {
             // 8, 16 or 24 coordinates (blocks of 2^3 and 2^4): byte by byte
@@ -210,7 +210,7 @@ __device__ __forceinline__ void low_round_inverse(float4 *wtile, const unsigned 
             for (int q = 0; q < IN_BITS; ++q)
 #pragma unroll
                 for (int y = 0; y < 4; ++y)
-                    if (4 * q + y < bytes) w[q] |= (uint32_t)__ldg(p + 4 * q + y) << (8 * y);
+                    if (4 * q + y < bytes) w[q] |= (uint32_t)ld_global(p + 4 * q + y) << (8 * y);
         }
 #pragma unroll
         for (int m = 0; m < 8; ++m) {
@@ -293,7 +293,7 @@ __device__ __forceinline__ void low_round_aggregate(float4 *wtile, const PtrArra
 #pragma unroll 4
                 for (uint32_t i = i0; i < i1; ++i) {
                     const unsigned char *src = static_cast<const unsigned char *>(in.p[i]) + byte_off;
-                    const uint4 t4 = __ldg(reinterpret_cast<const uint4 *>(src + (size_t)row * 16));
+                    const uint4 t4 = ld_global(reinterpret_cast<const uint4 *>(src + (size_t)row * 16));
                     const uint32_t words[4] = {t4.x, t4.y, t4.z, t4.w};
 #pragma unroll
                     for (int h = 0; h < 4; ++h) {
@@ -488,9 +488,7 @@ thc_block_kernel(const __grid_constant__ TmaMaps maps, const __grid_constant__ B
     if (thread == 0) {
         mbar_init(&s_full, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        if (task < P.tasks && by_tma(unit)) start_load(unit, wl);
     }
-    if (!kForward && task < P.tasks) prefetch_inputs(unit, wl);
     if (kQuant && !IDENTITY) lut_fill<LutKind<BITS, IDENTITY>::k8>(lut, P.dev, P.granularity, thread, kBThreads);
     if (kEF) {
         // table values as floats, one copy per lane (8 copies for 8-bit indices)
@@ -503,6 +501,11 @@ thc_block_kernel(const __grid_constant__ TmaMaps maps, const __grid_constant__ B
         for (int q = 0; q < 4; ++q)
             agg_tb[q] = P.dev->table[4 * q] | (P.dev->table[4 * q + 1] << 8) | (P.dev->table[4 * q + 2] << 16) |
                         (P.dev->table[4 * q + 3] << 24);
+    }
+    depend_on_previous();
+    if (task < P.tasks) {
+        if (thread == 0 && by_tma(unit)) start_load(unit, wl);
+        if (!kForward) prefetch_inputs(unit, wl);
     }
     __syncthreads();
 
@@ -566,11 +569,11 @@ thc_block_kernel(const __grid_constant__ TmaMaps maps, const __grid_constant__ B
                         const uint64_t j = jw + 8u * u;
                         uint32_t w[4] = {0, 0, 0, 0};
                         if (j + 8 <= P.d) {
-                            const uint4 q4 = __ldg(reinterpret_cast<const uint4 *>(x + j));
+                            const uint4 q4 = ld_global(reinterpret_cast<const uint4 *>(x + j));
                             w[0] = q4.x; w[1] = q4.y; w[2] = q4.z; w[3] = q4.w;
                         } else {
                             for (int e = 0; e < 8; ++e)
-                                if (j + e < P.d) w[e >> 1] |= (uint32_t)__ldg(x + j + e) << ((e & 1) * 16);
+                                if (j + e < P.d) w[e >> 1] |= (uint32_t)ld_global(x + j + e) << ((e & 1) * 16);
                         }
                         const int c = 2 * u;
                         wtile[c ^ ((c >> 3) & 7)] = make_float4(__uint_as_float(w[0] << 16), __uint_as_float(w[0] & 0xFFFF0000u),
@@ -715,8 +718,8 @@ thc_block_kernel(const __grid_constant__ TmaMaps maps, const __grid_constant__ B
                     float4 oa = flip4(ra, bits), ob = flip4(rb, bits >> 4);
                     if (j + 8 <= P.d) {
                         if (kEF) {
-                            const float4 xa = __ldcs(reinterpret_cast<const float4 *>(xs + j));
-                            const float4 xb = __ldcs(reinterpret_cast<const float4 *>(xs + j + 4));
+                            const float4 xa = ld_global_once(reinterpret_cast<const float4 *>(xs + j));
+                            const float4 xb = ld_global_once(reinterpret_cast<const float4 *>(xs + j + 4));
                             oa = make_float4(xa.x - oa.x, xa.y - oa.y, xa.z - oa.z, xa.w - oa.w);
                             ob = make_float4(xb.x - ob.x, xb.y - ob.y, xb.z - ob.z, xb.w - ob.w);
                         }

@@ -32,6 +32,60 @@ struct DeviceBlock {
     uint32_t table[256];         // T
 };
 
+// ------------------------------------------------------------------------ dependent launches
+// Every kernel is launched so that it may start before the launch before it is complete (launch_after in
+// thc.cu): the launch itself, the tables and the barriers are set up while the other's writes drain.  Each CTA
+// calls depend_on_previous() before it touches anything that a launch writes; it returns when the previous
+// launch, which called it too, is complete and its writes are visible.  No kernel releases the next one
+// early (griddepcontrol.launch_dependents): CTAs that move in beside a kernel with another split of
+// shared memory and L1 keep that split (a pipeline kernel next to a streaming one: 8 us of 144 lost).
+__device__ __forceinline__ void depend_on_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// Loads of what other launches wrote: volatile and coherent, so that none of them is moved in front of
+// depend_on_previous() (loads through the read-only path may be).
+__device__ __forceinline__ uint4 ld_global(const uint4 *p)
+{
+    uint4 v;
+    asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ uint4 ld_global_once(const uint4 *p)
+{
+    uint4 v;
+    asm volatile("ld.global.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float4 ld_global_once(const float4 *p)
+{
+    const uint4 v = ld_global_once(reinterpret_cast<const uint4 *>(p));
+    return make_float4(__uint_as_float(v.x), __uint_as_float(v.y), __uint_as_float(v.z), __uint_as_float(v.w));
+}
+__device__ __forceinline__ uint2 ld_global(const uint2 *p)
+{
+    uint2 v;
+    asm volatile("ld.global.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ uint32_t ld_global(const uint32_t *p)
+{
+    uint32_t v;
+    asm volatile("ld.global.u32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ uint32_t ld_global(const uint16_t *p)
+{
+    uint16_t v;
+    asm volatile("ld.global.u16 %0, [%1];" : "=h"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ uint32_t ld_global(const unsigned char *p)
+{
+    uint32_t v;
+    asm volatile("ld.global.u8 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float ld_global(const float *p) { return __uint_as_float(ld_global(reinterpret_cast<const uint32_t *>(p))); }
+
 struct PhiloxKeys { uint32_t k[20]; };         // the ten round keys, precomputed on the host
 
 // Philox4x32-10 (Salmon et al., SC'11).
@@ -80,8 +134,8 @@ __device__ __forceinline__ BlockRange block_range(const float *scales, uint64_t 
                                                   uint32_t exact)
 {
     BlockRange b;
-    if (exact) { b.lo = scales[r]; b.hi = scales[nblocks + r]; }
-    else { b.hi = scales[r]; b.lo = -b.hi; }
+    if (exact) { b.lo = ld_global(scales + r); b.hi = ld_global(scales + nblocks + r); }
+    else { b.hi = ld_global(scales + r); b.lo = -b.hi; }
     return b;
 }
 
@@ -339,12 +393,12 @@ __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel)
 
 __device__ __forceinline__ float4 load_f32x4_masked(const float *x, uint64_t j, uint64_t d)
 {
-    if (j + 4 <= d) return __ldg(reinterpret_cast<const float4 *>(x + j));
+    if (j + 4 <= d) return ld_global_once(reinterpret_cast<const float4 *>(x + j));
     float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (j + 0 < d) v.x = __ldg(x + j + 0);
-    if (j + 1 < d) v.y = __ldg(x + j + 1);
-    if (j + 2 < d) v.z = __ldg(x + j + 2);
-    if (j + 3 < d) v.w = __ldg(x + j + 3);
+    if (j + 0 < d) v.x = ld_global(x + j + 0);
+    if (j + 1 < d) v.y = ld_global(x + j + 1);
+    if (j + 2 < d) v.z = ld_global(x + j + 2);
+    if (j + 3 < d) v.w = ld_global(x + j + 3);
     return v;
 }
 

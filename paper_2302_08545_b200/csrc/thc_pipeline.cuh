@@ -546,18 +546,18 @@ __device__ __forceinline__ void pass_a_round1_inverse(float4 *tile, const unsign
         if constexpr (IN_BITS >= 4) {
 #pragma unroll
             for (int q = 0; q < IN_BITS / 4; ++q) {
-                const uint4 t4 = __ldg(reinterpret_cast<const uint4 *>(p) + q);
+                const uint4 t4 = ld_global(reinterpret_cast<const uint4 *>(p) + q);
                 wg[4 * q] = t4.x; wg[4 * q + 1] = t4.y; wg[4 * q + 2] = t4.z; wg[4 * q + 3] = t4.w;
             }
         } else if constexpr (IN_BITS == 3) {
-            wg[0] = __ldg(reinterpret_cast<const uint32_t *>(p));
-            wg[1] = __ldg(reinterpret_cast<const uint32_t *>(p) + 1);
-            wg[2] = __ldg(reinterpret_cast<const uint32_t *>(p) + 2);
+            wg[0] = ld_global(reinterpret_cast<const uint32_t *>(p));
+            wg[1] = ld_global(reinterpret_cast<const uint32_t *>(p) + 1);
+            wg[2] = ld_global(reinterpret_cast<const uint32_t *>(p) + 2);
         } else if constexpr (IN_BITS == 2) {
-            const uint2 t2 = __ldg(reinterpret_cast<const uint2 *>(p));
+            const uint2 t2 = ld_global(reinterpret_cast<const uint2 *>(p));
             wg[0] = t2.x; wg[1] = t2.y;
         } else {
-            wg[0] = __ldg(reinterpret_cast<const uint32_t *>(p));
+            wg[0] = ld_global(reinterpret_cast<const uint32_t *>(p));
         }
     }
 #pragma unroll 1
@@ -629,7 +629,7 @@ __device__ __forceinline__ void pass_a_round1_aggregate(float4 *tile, const PtrA
                 const unsigned char *src = static_cast<const unsigned char *>(in.p[i]) + byte_off;
 #pragma unroll
                 for (int g = 0; g < 2; ++g) {
-                    const uint4 t4 = __ldg(reinterpret_cast<const uint4 *>(src + (size_t)(r0 + 32 * g) * 16));
+                    const uint4 t4 = ld_global(reinterpret_cast<const uint4 *>(src + (size_t)(r0 + 32 * g) * 16));
                     const uint32_t words[4] = {t4.x, t4.y, t4.z, t4.w};
 #pragma unroll
                     for (int h = 0; h < 4; ++h) {
@@ -813,8 +813,8 @@ __device__ __forceinline__ void epilogue_unit(const float4 &va, const float4 &vb
         float4 ob = flip4(rb, bits >> 4);
         if (j + 8 <= ep.d) {
             if (ep.xsub != nullptr) {
-                const float4 xa = __ldcs(reinterpret_cast<const float4 *>(ep.xsub + j));
-                const float4 xb = __ldcs(reinterpret_cast<const float4 *>(ep.xsub + j + 4));
+                const float4 xa = ld_global_once(reinterpret_cast<const float4 *>(ep.xsub + j));
+                const float4 xb = ld_global_once(reinterpret_cast<const float4 *>(ep.xsub + j + 4));
                 oa = make_float4(xa.x - oa.x, xa.y - oa.y, xa.z - oa.z, xa.w - oa.w);
                 ob = make_float4(xb.x - ob.x, xb.y - ob.y, xb.z - ob.z, xb.w - ob.w);
             }
@@ -1076,6 +1076,7 @@ thc_pipeline_kernel(const __grid_constant__ TmaMaps maps, PipeParams P, PtrArray
         for (int idx = tid; idx < (1 << BITS) * kFRep; idx += kPCtaThreads)
             ftab[idx] = (float)P.dev->table[idx / kFRep];
     }
+    depend_on_previous();
     const uint32_t nblk_total = (uint32_t)(P.d_pad >> P.k);
     const uint32_t nblk_cached = nblk_total < (uint32_t)kBlockConstMax ? nblk_total : (uint32_t)kBlockConstMax;
     if (!kFused && !kRange) {
@@ -1372,11 +1373,11 @@ thc_pipeline_kernel(const __grid_constant__ TmaMaps maps, PipeParams P, PtrArray
                     const uint64_t j = j0 + 8ull * u;
                     uint32_t w[4] = {0, 0, 0, 0};
                     if (j + 8 <= P.d) {
-                        const uint4 q = __ldg(reinterpret_cast<const uint4 *>(x + j));
+                        const uint4 q = ld_global(reinterpret_cast<const uint4 *>(x + j));
                         w[0] = q.x; w[1] = q.y; w[2] = q.z; w[3] = q.w;
                     } else {
                         for (int e = 0; e < 8; ++e)
-                            if (j + e < P.d) w[e >> 1] |= (uint32_t)__ldg(x + j + e) << ((e & 1) * 16);
+                            if (j + e < P.d) w[e >> 1] |= (uint32_t)ld_global(x + j + e) << ((e & 1) * 16);
                     }
                     tile[pswz(2 * u)] = make_float4(__uint_as_float(w[0] << 16), __uint_as_float(w[0] & 0xFFFF0000u),
                                                     __uint_as_float(w[1] << 16), __uint_as_float(w[1] & 0xFFFF0000u));
