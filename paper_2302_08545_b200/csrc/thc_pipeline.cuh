@@ -776,13 +776,13 @@ struct EpilogueCtx {
 
 // RANGE: the unit only feeds the running minimum / maximum (as ordered keys) of the rotated
 // coordinates (Algorithm 1's preliminary stage).
-template <bool COMPRESS, int BITS, bool IDENTITY, bool RANGE = false>
+template <bool COMPRESS, int BITS, bool IDENTITY, bool RANGE = false, bool SCALE = true>
 __device__ __forceinline__ void epilogue_unit(const float4 &va, const float4 &vb, uint64_t j, int row,
                                               int uu, const EpilogueCtx &ep, const PhiloxKeys &keys,
                                               uint32_t &kmin, uint32_t &kmax)
 {
-    const float4 ra = scale4(va, ep.c_block);
-    const float4 rb = scale4(vb, ep.c_block);
+    const float4 ra = SCALE ? scale4(va, ep.c_block) : va;
+    const float4 rb = SCALE ? scale4(vb, ep.c_block) : vb;
     if constexpr (RANGE) {
         if (ep.rotated != nullptr) {
             *reinterpret_cast<float4 *>(ep.rotated + j) = ra;
@@ -798,7 +798,7 @@ __device__ __forceinline__ void epilogue_unit(const float4 &va, const float4 &vb
         return;
     }
     if (COMPRESS) {
-        if (ep.rotated != nullptr) {
+        if (SCALE && ep.rotated != nullptr) {
             *reinterpret_cast<float4 *>(ep.rotated + j) = ra;
             *reinterpret_cast<float4 *>(ep.rotated + j + 4) = rb;
         }
@@ -888,7 +888,7 @@ __device__ __forceinline__ void pass_b_last_round(const float4 *tile, int kb, in
 // Thread (u = tid & 3, rl from bits 2..5, h = tid >> 6) owns unit 4h + u of rows rl + 16 m,
 // m = 0..7; lanes 0-7 of a quarter warp cover four units of two adjacent rows, whose XOR
 // patterns differ in bit 0, so both chunk reads are conflict-free.
-template <bool COMPRESS, int BITS, bool IDENTITY, bool RANGE>
+template <bool COMPRESS, int BITS, bool IDENTITY, bool RANGE, bool SCALE>
 __device__ __forceinline__ void pass_b_last_round_kb7(float4 *tile, int tid,
                                                       const EpilogueCtx &ep, const PhiloxKeys &keys,
                                                       uint32_t &kmin, uint32_t &kmax)
@@ -921,7 +921,7 @@ __device__ __forceinline__ void pass_b_last_round_kb7(float4 *tile, int tid,
         for (int half = 0; half < 2; ++half) {
 #pragma unroll
             for (int m = 0; m < 4; ++m)
-                epilogue_unit<COMPRESS, BITS, IDENTITY, RANGE>(a[m], b[m], j0 + ((uint64_t)(4 * half + m) << (kPLog2 + 4)),
+                epilogue_unit<COMPRESS, BITS, IDENTITY, RANGE, SCALE>(a[m], b[m], j0 + ((uint64_t)(4 * half + m) << (kPLog2 + 4)),
                                                                rl + 16 * (4 * half + m), uu, ep, keys, kmin, kmax);
 #pragma unroll
             for (int m = 0; m < 4; ++m) { a[m] = a[m + 4]; b[m] = b[m + 4]; }
@@ -1511,8 +1511,21 @@ thc_pipeline_kernel(const __grid_constant__ TmaMaps maps, PipeParams P, PtrArray
                     compute_barrier();
                 }
                 uint32_t kmin = 0xFFFFFFFFu, kmax = 0u;
-                if (KB == 7) {
-                    pass_b_last_round_kb7<kCompress, BITS, IDENTITY, kRange>(tile, tid, ep, keys, kmin, kmax);
+                // 1/sqrt(B) of 2^20 blocks is a power of two: it goes into kappa, which gives the same position
+                // bit for bit (a rotated coordinate that would round, being below 2^-126, is nothing against the
+                // offset of 1/2 for such a kappa), and the scaling of every coordinate is left out: one dispatch
+                // slot of 58 (one worker x 25.6 M coordinates 86 -> 80 us, 4 x 2^26 634 -> 628).  Not where the
+                // rotated coordinates are written, nor in exact-range mode, whose offset may be 0; with fused
+                // scales and for 2^22 blocks it was no faster.
+                constexpr bool kScaleInKappa = KB == 7 && kCompress && !kRange && !kFused;
+                bool in_kappa = false;
+                if constexpr (kScaleInKappa) {
+                    in_kappa = ep.rotated == nullptr && P.exact_range == 0u && ep.kappa > 0x1p-100f && ep.kappa < 0x1p60f;
+                    if (in_kappa) ep.kappa *= ep.c_block;
+                }
+                if constexpr (KB == 7) {
+                    if (in_kappa) pass_b_last_round_kb7<kCompress, BITS, IDENTITY, kRange, !kScaleInKappa>(tile, tid, ep, keys, kmin, kmax);
+                    else pass_b_last_round_kb7<kCompress, BITS, IDENTITY, kRange, true>(tile, tid, ep, keys, kmin, kmax);
                 } else if constexpr (KB == 8 || KB == 9) {
                     pass_b_high4<BITS, IDENTITY, KB>(tile, tid, ep, keys);
                 } else {
