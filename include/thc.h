@@ -175,8 +175,8 @@ int thc_decompress(thc_ctx *ctx, const void *sum, uint32_t divisor, uint64_t d, 
 
 /* thc_aggregate followed by thc_decompress as one call, for a caller that holds all n workers'
  * packed indices on this GPU (the simulated cluster): Algorithm 2's PS line, Y = sum_i T[Z_i],
- * feeding the worker's estimate line and the inverse RHT (Algorithm 3) directly.  For RHT blocks
- * above 2^14 coordinates, 4-bit indices and table values below 128 this is one launch and the
+ * feeding the worker's estimate line and the inverse RHT (Algorithm 3) directly.  For
+ * 4-bit indices and table values below 128 this is one launch and the
  * sums never travel through memory; they are written (d_pad unsigned integers of acc_bits bits,
  * as thc_aggregate writes them) only if sum_or_null is given.  Elsewhere the call runs
  * thc_aggregate and thc_decompress (sums in the workspace unless a buffer is given).  `out` is bit for bit what the two calls give with divisor n.  The paper's
@@ -232,9 +232,9 @@ int thc_prepare_minmax(thc_ctx *ctx, const void *const *grads, uint32_t n, uint6
  * (the simulated cluster): same arguments and results as the two calls in a row, `scales`
  * (device, nblocks floats) being written here and usable by thc_decompress afterwards.
  * Section 5.3 observes that the norm exchange can overlap the RHT: only the quantiser needs M,
- * so where the block size is 2^16 (more than 2^22 coordinates over all workers) to 2^20, the input
- * fp32 and n small enough for the intermediate ring to stay in L2, the transform kernel sums the squares of the tiles it loads anyway and the
- * gradients are read from HBM once instead of twice.  Elsewhere this runs the two calls.
+ * so where the block size is 2^17 (more than 14 blocks over all workers) to 2^20, the input fp32
+ * and n small enough for the intermediate ring to stay in L2, the transform kernel sums the squares
+ * of the tiles it loads anyway and the gradients are read from HBM once instead of twice.  Elsewhere this runs the two calls.
  * The fp64 sums are added in a different (fixed) order than thc_prepare's, so a scale may
  * differ from thc_prepare's in the last bit.  */
 int thc_prepare_compress(thc_ctx *ctx, const void *const *grads, uint32_t n, uint32_t worker_base,
@@ -246,10 +246,9 @@ int thc_prepare_compress(thc_ctx *ctx, const void *const *grads, uint32_t n, uin
  * workers, the residual between what it compressed and what its own indices stand for,
  *     ef[i] = x_i - RHT^-1( m + T[Z_i] (M - m)/g ),
  * to be added to the next round's gradient (thc_accumulate_error).  fp32 contexts only
- * (THC_EUNSUPPORTED for bf16 inputs).  For RHT blocks above 2^14 coordinates this is one launch
- * over all workers (indices in, de-quantised in registers, inverse transform, x - result out);
- * for smaller blocks it is composed per worker of thc_aggregate with n = 1, thc_decompress with
- * divisor 1 and one subtraction.  Both give the same bits.
+ * (THC_EUNSUPPORTED for bf16 inputs).  One launch over all workers (indices in, de-quantised in
+ * registers, inverse transform, x - result out), with the bits of thc_aggregate with n = 1,
+ * thc_decompress with divisor 1 and one subtraction.
  *   grads    host array of n_local device pointers: the x_i that were compressed
  *   packed   host array of n_local device pointers: their packed indices
  *   ef       host array of n_local device pointers, d fp32 each, written

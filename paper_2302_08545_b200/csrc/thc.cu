@@ -909,7 +909,8 @@ static PipePlan plan_pipeline(const thc_ctx *ctx, uint64_t wb_count)
 static bool plan_pipeline_fused(const thc_ctx *ctx, uint64_t nblocks, uint32_t n, PipePlan *out)
 {
     const uint32_t k = ctx->cfg.log2_block;
-    if (k > 20u || ctx->cfg.in_dtype != THC_F32 || block_kernel_serves(k, (nblocks * n) << k)) return false;
+    // (2^16: 4 % at most)
+    if (k < 17u || k > 20u || ctx->cfg.in_dtype != THC_F32 || block_kernel_serves(k, (nblocks * n) << k)) return false;
     if (ctx->cfg.range_mode != THC_RANGE_NORM) return false;
     const uint64_t wb_count = nblocks * n;
     PipePlan p = plan_pipeline(ctx, wb_count);

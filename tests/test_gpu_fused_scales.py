@@ -7,7 +7,7 @@ from paper_2302_08545_b200 import workloads as W
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("k,nblk,n,bits", [(16, 70, 4, 4), (16, 300, 1, 2), (17, 16, 5, 8), (17, 130, 2, 4), (18, 20, 3, 3), (19, 9, 4, 1),
+@pytest.mark.parametrize("k,nblk,n,bits", [(17, 16, 5, 8), (17, 130, 2, 4), (18, 20, 3, 3), (19, 9, 4, 1),
                                            (18, 131, 1, 4)])
 def test_one_launch_equals_the_two_calls(k, nblk, n, bits):
     import torch
