@@ -34,7 +34,7 @@ from paper_2302_08545_b200 import workloads as W  # noqa: E402
 
 METRIC = "gradient GB/s per compress+aggregate+decompress round; % of HBM roofline"
 UNIT = "GB/s"
-KERNELS_PER_STEP = {"prepare": 2, "compress": 1, "prepare_compress": 1, "aggregate": 1, "decompress": 1}
+KERNELS_PER_STEP = {"prepare": 1, "compress": 1, "prepare_compress": 1, "aggregate": 1, "decompress": 1}
 # DRAM bytes per (worker, padded coordinate) of the compress kernel (n = 4, d = 2^24, b = 4) and of
 # its fused-scales variant (n = 8, d = 2^24, b = 4: its ring grows with n), measured with ncu
 # (profiles/thc_pipeline_kernel_d2p24_b4.md); traffic grows in proportion to n*d_pad, so a full

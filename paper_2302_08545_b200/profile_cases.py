@@ -7,7 +7,7 @@ buffer), warms the calls up, times them with CUDA events and prints one JSON lin
 `ncu -k regex:<kernel> -c <n>` the same command gives the counters of the kernels named below.
 
   case              calls (kernels)
-  tile14            prepare, compress, aggregate, decompress at B = 2^14 (rht_tile_kernel)
+  tile14            prepare, compress, aggregate, decompress at B = 2^14 (thc_block_kernel)
   quantize          thc_quantize_rotated (quantize_rotated_kernel)
   bf16k22           compress, aggregate, decompress for bf16 gradients at B = 2^22, n = 2
                     (thc_pipeline_kernel<bf16, KB = 9>, aggregate_b4w8, thc_pipeline_kernel<decompress>)
