@@ -265,8 +265,9 @@ int thc_accumulate_error(thc_ctx *ctx, float *const *grads, const float *const *
 int thc_status(thc_ctx *ctx, uint32_t *flags, void *stream);
 
 /* Test hook for the bounded waits of the large-block pipeline (no counterpart in the paper).
- * The next thc_compress / thc_decompress on this context starts its task queue at position
- * `count` instead of 0, so tasks that depend on the skipped ones can never be satisfied: the
+ * The next call on this context that transforms blocks above 2^14 takes the pipeline whatever
+ * their size and starts its task queue at position `count` instead of 0 (blocks of up to 2^14 have no
+ * queue: no effect), so tasks that depend on the skipped ones can never be satisfied: the
  * kernel must notice (about one second), set THC_STATUS_WAIT_TIMEOUT, and return with the
  * context still usable; the outputs of that call are undefined.  Synchronises the device. */
 int thc_debug_skip_tasks(thc_ctx *ctx, uint32_t count);

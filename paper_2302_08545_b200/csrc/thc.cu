@@ -693,7 +693,8 @@ struct thc_ctx {
     int device;                 // -1: no CUDA device, host-only context
     DeviceBlock *dev;
     PhiloxKeys keys;
-    bool pipeline_next;         // the queue of the next pipeline launch is set (thc_debug_skip_tasks)
+    bool pipeline_next;         // the queue of the next pipeline launch is set (thc_debug_skip_tasks); until then
+                                // blocks above 2^14 take the pipeline
     int sm_count;
     // Encoded tensor maps of recent launches, keyed by what they describe: a training loop calls
     // with the same buffers every step, and encoding up to n + 1 maps per call costs more host
@@ -1187,7 +1188,7 @@ static int cached_map(const thc_ctx *ctx, CUtensorMap *map, const void *base, ui
     return THC_OK;
 }
 
-static int launch_pipeline(const thc_ctx *ctx, pipe_kernel_t kern, bool compress_f32,
+static int launch_pipeline(thc_ctx *ctx, pipe_kernel_t kern, bool compress_f32,
                            const thc_sizes_t &sz, uint64_t d, uint32_t n_local, uint32_t worker_base, uint32_t round, uint32_t divisor,
                            const float *scales, void *workspace, const PtrArrayP &in,
                            const MutPtrArrayP &out, const MutPtrArrayP &rot, cudaStream_t st,
@@ -1281,13 +1282,16 @@ static int launch_pipeline(const thc_ctx *ctx, pipe_kernel_t kern, bool compress
         }
     }
     THC_CUDA(launch_after(kern, dim3(pl.grid), kPCtaThreads, smem, st, maps, P, in, out, rot, ctx->keys));
+    ctx->pipeline_next = false;
     return THC_OK;
 }
 
-// ---- blocks held in shared memory (RHT blocks of up to 2^16 coordinates)
+// ---- blocks held in shared memory (see block_kernel_serves).  Blocks of up to 2^14 have no other kernel: for
+// them thc_sizes reserves no ring, and below 2^13 the pipeline has no tile.
 static bool use_block_kernel(const thc_ctx *ctx, uint64_t coords)
 {
-    return !ctx->pipeline_next && block_kernel_serves(ctx->cfg.log2_block, coords);
+    const uint32_t k = ctx->cfg.log2_block;
+    return k <= (uint32_t)kChunkLog2 || (!ctx->pipeline_next && block_kernel_serves(k, coords));
 }
 
 // lut_bytes: table space in shared memory; keys: exact-range mode; agg_n: aggregate + decompress.
@@ -1459,7 +1463,6 @@ int thc_compress(thc_ctx *ctx, const void *const *grads, uint32_t n_local, uint3
         return launch_block(ctx, kern, bf16 ? kCompressBF16 : kCompressF32, quant_lut_bytes(ctx), sz, d, n_local, worker_base,
                             round, 1, scales, in, out, rot, st);
     }
-    ctx->pipeline_next = false;
     pipe_kernel_t kern = bf16 ? pick_pipe_kernel<kCompressBF16>(ctx->cfg.bits, ctx->identity, k)
                               : pick_pipe_kernel<kCompressF32>(ctx->cfg.bits, ctx->identity, k);
     return launch_pipeline(ctx, kern, !bf16, sz, d, n_local, worker_base, round, 1, scales, workspace,
@@ -1538,7 +1541,6 @@ int thc_decompress(thc_ctx *ctx, const void *sum, uint32_t divisor, uint64_t d, 
         return launch_block(ctx, kern, w == 8 ? kDecompress8 : w == 16 ? kDecompress16 : kDecompress32, 0, sz, d, 1, 0, round,
                             divisor, scales, pin, pout, prot, st);
     }
-    ctx->pipeline_next = false;
     pipe_kernel_t kern = w == 8 ? pick_pipe_kernel<kDecompress8>(4, true, k)
                        : w == 16 ? pick_pipe_kernel<kDecompress16>(4, true, k)
                                  : pick_pipe_kernel<kDecompress32>(4, true, k);

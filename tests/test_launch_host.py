@@ -1,0 +1,89 @@
+"""Host code of the launching calls on a fake CUDA runtime (tests/fake_cudart.c): which kernel a call launches,
+with what grid and shared memory.  Runs without a GPU, in child processes; no kernel is executed."""
+import os
+import subprocess
+import sys
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+# What a child process has at hand: contexts, buffers that are only addresses, and the log of launches.
+PRELUDE = """
+import ctypes, sys
+sys.path.insert(0, {root!r})
+from paper_2302_08545_b200 import thc, workloads as W
+fake = ctypes.CDLL(None)
+fake.fake_log.restype = ctypes.c_char_p
+
+class Space:
+    nbytes = 1 << 40
+    def data_ptr(self):
+        return 1 << 32
+
+ws = Space()
+buf = [(i + 1) << 20 for i in range(64)]
+
+def context(k, **kw):
+    return thc.Context(**dict(dict(bits=4, granularity=30, table=W.TABLES[(4, 30)], t_p=2.0, log2_block=k, seed=1), **kw))
+
+def log():
+    # [kind, kernel, numbers...] per line since the last call
+    rows = [line.split() for line in fake.fake_log().decode().splitlines()]
+    return [row[:2] + [int(v) for v in row[2:]] for row in rows]
+
+def kernels():
+    return ["block" if "block_kernel" in r[1] else "pipeline" if "pipeline_kernel" in r[1] else r[1]
+            for r in log() if r[0] == "launch"]
+
+def transforms(c, d, n=2):
+    x = buf[:n]
+    calls = [lambda: c.compress(x, d, 0, buf[0], x, ws, stream=0), lambda: c.decompress(buf[0], n, d, 0, buf[1], buf[2], ws, stream=0),
+             lambda: c.aggregate_decompress(x, d, 0, buf[0], buf[1], ws, stream=0)]
+    return calls + [lambda: c.error_feedback(x, x, d, 0, buf[0], x, ws, stream=0)]
+
+"""
+
+
+@pytest.fixture(scope="module")
+def child(tmp_path_factory):
+    so = str(tmp_path_factory.mktemp("fake") / "fake_cudart.so")
+    subprocess.run([os.environ.get("CC", "gcc"), "-O1", "-fPIC", "-shared", "-I/usr/local/cuda/include", "-o", so,
+                    os.path.join(ROOT, "tests", "fake_cudart.c")], check=True)
+
+    def run(code):
+        res = subprocess.run([sys.executable, "-c", PRELUDE.format(root=ROOT) + code], capture_output=True, text=True,
+                             env=dict(os.environ, LD_PRELOAD=so), timeout=300)
+        assert res.returncode == 0, res.stderr[-3000:]
+        return res.stdout
+    return run
+
+
+@pytest.mark.parametrize("k", [3, 12, 13, 14])
+def test_skipped_tasks_never_send_a_small_block_to_the_pipeline(child, k):
+    child(f"""
+k = {k}
+c = context(k)
+m = context(k, range_mode=1)
+for call in transforms(c, 1 << 15) + [lambda: m.prepare_minmax(buf[:2], 1 << 15, 0, buf[0], ws, stream=0)]:
+    for ctx in (c, m):
+        ctx.debug_skip_tasks(1)
+    call()
+    assert kernels() == ["block"], k
+""")
+
+
+@pytest.mark.parametrize("k", [15, 16, 17])
+def test_skipped_tasks_take_the_pipeline_once(child, k):
+    child(f"""
+k = {k}
+c = context(k)
+m = context(k, range_mode=1)
+for ctx, call in [(c, f) for f in transforms(c, 3 << k)] + [(m, lambda: m.prepare_minmax(buf[:2], 3 << k, 0, buf[0], ws, stream=0))]:
+    call()
+    assert kernels() == ["block"]
+    ctx.debug_skip_tasks(1)
+    call()
+    call()
+    assert kernels() == ["pipeline", "block"]
+""")
