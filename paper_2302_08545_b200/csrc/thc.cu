@@ -1034,27 +1034,33 @@ int thc_prepare(thc_ctx *ctx, const void *const *grads, uint32_t n, uint64_t d, 
     return THC_OK;
 }
 
-// cudaFuncSetAttribute is needed once per kernel and dynamic shared-memory size; remember
-// what has been set per (kernel, device); a larger request raises the recorded size.
-static int ensure_dynamic_smem(const void *kern, size_t smem)
+// The largest dynamic shared memory of any launch: a pipeline CTA, a tile of 2^14 or one of 2^13 with the
+// constants of 1024 blocks, each with a table of 256 entries.
+constexpr size_t kMaxDynamicSmem = 104u << 10;
+static_assert(1024 + 2 * kPElems * 4 + kPSignWords * 4 + 256 * kLutEntryBytes + kBlockConstMax * 8 <= kMaxDynamicSmem, "pipeline");
+static_assert(1024 + (4 << 14) + (1 << 14) / 4 + 16 + 256 * kLutEntryBytes <= kMaxDynamicSmem, "tile of 2^14");
+static_assert(1024 + (4 << 13) + (1 << 13) / 4 + 1024 * 16 + 256 * kLutEntryBytes <= kMaxDynamicSmem, "tile of 2^13");
+
+// Lets a kernel use more than the default 48 KB.  The limit is the same for every launch of every kernel, so
+// that no thread can lower it between another's call and its launch; what is done is remembered per kernel
+// and device, and done again (to the same effect) should the table be full.
+static int ensure_dynamic_smem(const void *kern)
 {
+    constexpr uint32_t kSlots = 2048;                  // of some 300 kernels
     static std::mutex guard;
-    std::lock_guard<std::mutex> lock(guard);
-    static const void *seen_kern[96];
-    static size_t seen_size[96];
-    static int seen_dev[96];
-    static int seen = 0;
+    static const void *seen_kern[kSlots];
+    static int seen_dev[kSlots];
+    static uint32_t used = 0;
     int dev = 0;
     THC_CUDA(cudaGetDevice(&dev));
-    for (int i = 0; i < seen; ++i)
-        if (seen_kern[i] == kern && seen_dev[i] == dev) {
-            if (seen_size[i] >= smem) return THC_OK;
-            THC_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-            seen_size[i] = smem;
-            return THC_OK;
-        }
-    THC_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    if (seen < 96) { seen_kern[seen] = kern; seen_size[seen] = smem; seen_dev[seen] = dev; ++seen; }
+    std::lock_guard<std::mutex> lock(guard);
+    uint32_t slot = (uint32_t)((reinterpret_cast<uintptr_t>(kern) >> 4) * 0x9E3779B9u + (uint32_t)dev) % kSlots;
+    while (seen_kern[slot] != nullptr) {               // never full: a quarter stays free
+        if (seen_kern[slot] == kern && seen_dev[slot] == dev) return THC_OK;
+        slot = (slot + 1u) % kSlots;
+    }
+    THC_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxDynamicSmem));
+    if (used < kSlots / 4 * 3) { seen_kern[slot] = kern; seen_dev[slot] = dev; ++used; }
     return THC_OK;
 }
 
@@ -1238,7 +1244,7 @@ static int launch_pipeline(thc_ctx *ctx, pipe_kernel_t kern, bool compress_f32,
     const uint64_t nblk_cached = sz.nblocks < (uint64_t)kBlockConstMax ? sz.nblocks : (uint64_t)kBlockConstMax;
     const size_t smem = (size_t)1024 + (size_t)2 * kPElems * 4 + kPSignWords * 4 +
                         (size_t)(ctx->cfg.granularity + 1) * kLutEntryBytes + (size_t)nblk_cached * 8;
-    { const int rc = ensure_dynamic_smem(reinterpret_cast<const void *>(kern), smem); if (rc != THC_OK) return rc; }
+    { const int rc = ensure_dynamic_smem(reinterpret_cast<const void *>(kern)); if (rc != THC_OK) return rc; }
     // Tensor maps: the ring (pass-B panels are fetched by TMA at every block size) and, for fp32 compress, every
     // worker's gradient viewed as rows of 32 floats (whole rows only; a ragged last tile is
     // loaded by the compute warps).
@@ -1329,7 +1335,7 @@ static int launch_block(const thc_ctx *ctx, const void *kern, PipeMode mode, siz
     P.agg_chunk = 255u / ctx->cfg.granularity;
     P.agg_acc_bits = ctx->acc_bits;
     const size_t smem = (size_t)1024 + tile * 4 + tile / 4 + (size_t)P.const_slots * 16 + lut_bytes;
-    { const int rc = ensure_dynamic_smem(kern, smem); if (rc != THC_OK) return rc; }
+    { const int rc = ensure_dynamic_smem(kern); if (rc != THC_OK) return rc; }
     TmaMaps maps;
     if ((d >> 5) >= 256) {
         for (uint32_t i = 0; i < n_local; ++i) {

@@ -87,3 +87,37 @@ for ctx, call in [(c, f) for f in transforms(c, 3 << k)] + [(m, lambda: m.prepar
     call()
     assert kernels() == ["pipeline", "block"]
 """)
+
+
+def test_shared_memory_limit_is_set_once_per_kernel_and_never_lowered(child):
+    """More kernels than any process of the other tests uses, each with launches of several sizes (tables of
+    different granularity), largest first: a limit that is set again for a smaller launch would let another
+    thread's larger one fail."""
+    out = child("""
+limit, sets, largest = {}, {}, {}
+for size in (255, 60, 255):
+    for k in (3, 9, 14, 15, 16, 17, 20, 22):
+        for bits in (1, 2, 3, 4, 8):
+            levels = 1 << bits
+            for g in {size, levels - 1}:
+                table = list(range(levels - 1)) + [g]
+                if g < levels - 1:
+                    continue
+                for dtype in (0, 1):
+                    for acc in (0, 32):
+                        c = context(k, bits=bits, granularity=g, table=table, in_dtype=dtype, acc_bits=acc)
+                        for call in transforms(c, 1 << max(k, 15))[:4 - dtype]:
+                            call()
+                        for row in log():
+                            if row[0] == "attr":
+                                sets[row[1]] = sets.get(row[1], 0) + 1
+                                limit[row[1]] = row[2]
+                            elif row[4] > 48 << 10:
+                                largest[row[1]] = max(row[4], largest.get(row[1], 0))
+                                assert limit[row[1]] >= row[4], row
+assert len(limit) > 180, len(limit)
+print(len(limit), max(sets.values()))
+assert max(sets.values()) == 1
+assert all(limit[f] >= largest[f] for f in largest)
+""")
+    assert out.split()[1] == "1"
