@@ -6,6 +6,7 @@
 #include "../../include/thc.h"
 #include "thc_device.cuh"
 
+#include <atomic>
 #include <math.h>
 #include <mutex>
 #include <new>
@@ -704,6 +705,8 @@ struct thc_ctx {
     mutable MapEntry map_cache[kMapCache];
     mutable int map_cache_used, map_cache_next;
     mutable std::mutex map_mutex;
+    // Per mode, what resident_units answered for this context's block kernel (0: not asked yet).
+    mutable std::atomic<uint32_t> resident[kPipeModes];
 };
 
 static thread_local cudaError_t g_last_cuda = cudaSuccess;
@@ -805,6 +808,7 @@ int thc_create(const thc_config *cfg, thc_ctx **out)
     ctx->sm_count = 148;
     ctx->map_cache_used = 0;
     ctx->map_cache_next = 0;
+    for (auto &r : ctx->resident) r.store(0u, std::memory_order_relaxed);
     uint32_t k0 = (uint32_t)cfg->seed, k1 = (uint32_t)(cfg->seed >> 32);
     for (int r = 0; r < 10; ++r) {
         ctx->keys.k[2 * r] = k0;
@@ -1300,6 +1304,29 @@ static bool use_block_kernel(const thc_ctx *ctx, uint64_t coords)
     return k <= (uint32_t)kChunkLog2 || (!ctx->pipeline_next && block_kernel_serves(k, coords));
 }
 
+// CTAs (clusters) of a block kernel that the GPU holds at a time, as the runtime counts them.  A tile of 2^13 with
+// a table of more than 167 entries leaves room for three CTAs per SM instead of four: with 592 CTAs in the grid,
+// each with a fixed share of the tasks, a quarter of them started when others had ended.  Compress with a 4-bit
+// table of 256 entries, 592 against 444 CTAs: 4 x 2^22 coordinates in blocks of 2^12 37.7 -> 34.5 us, 4 x 2^24
+// 123.7 -> 117.6, 8 x 3,000,001 in blocks of 2^13 50.7 -> 47.1; over 448 .. 3500 tiles 22 % faster to 5 % slower
+// (near 700 and 1000 tiles, where 592 leave the shorter last round).  Of clusters of eight there are fewer than the
+// SMs have room for, since a cluster stays within one GPC (2^16: 71, or 48 with such a table: 4 x 2^20 coordinates 28.1 -> 24.5 us).
+static int resident_units(const thc_ctx *ctx, PipeMode mode, const void *kern, const cudaLaunchConfig_t &shape, uint32_t e, uint32_t *units)
+{
+    *units = ctx->resident[mode].load(std::memory_order_relaxed);
+    if (*units != 0u) return THC_OK;
+    int n = 0;
+    if (e == 0u) {
+        THC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, (int)shape.blockDim.x, shape.dynamicSmemBytes));
+        n *= ctx->sm_count;
+    } else {
+        THC_CUDA(cudaOccupancyMaxActiveClusters(&n, kern, &shape));
+    }
+    *units = n > 0 ? (uint32_t)n : 1u;
+    ctx->resident[mode].store(*units, std::memory_order_relaxed);
+    return THC_OK;
+}
+
 // lut_bytes: table space in shared memory; keys: exact-range mode; agg_n: aggregate + decompress.
 static int launch_block(const thc_ctx *ctx, const void *kern, PipeMode mode, size_t lut_bytes, const thc_sizes_t &sz,
                         uint64_t d, uint32_t n_local, uint32_t worker_base, uint32_t round, uint32_t divisor,
@@ -1345,9 +1372,6 @@ static int launch_block(const thc_ctx *ctx, const void *kern, PipeMode mode, siz
             if (rc != THC_OK) return rc;
         }
     }
-    const uint32_t ctas_per_sm = tile_log2 == 13u ? 4u : 2u;
-    const uint32_t resident = ((uint32_t)ctx->sm_count * ctas_per_sm) >> e;       // clusters (CTAs where e = 0)
-    const uint32_t grid = (P.tasks < resident ? P.tasks : resident) << e;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -1356,12 +1380,18 @@ static int launch_block(const thc_ctx *ctx, const void *kern, PipeMode mode, siz
     attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof cfg);
-    cfg.gridDim = dim3(grid);
+    cfg.gridDim = dim3((unsigned)ctx->sm_count << 3);
     cfg.blockDim = dim3((unsigned)(tile / 64));
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cfg.attrs = attr;
     cfg.numAttrs = e != 0u ? 2 : 1;
+    cudaLaunchConfig_t shape = cfg;
+    shape.attrs = attr + 1;
+    shape.numAttrs = 1;
+    uint32_t resident = 0;
+    { const int rc = resident_units(ctx, mode, kern, shape, e, &resident); if (rc != THC_OK) return rc; }
+    cfg.gridDim = dim3((P.tasks < resident ? P.tasks : resident) << e);
     void *args[] = {&maps, &P, const_cast<PtrArrayP *>(&in), const_cast<MutPtrArrayP *>(&out), const_cast<MutPtrArrayP *>(&rot),
                     const_cast<PhiloxKeys *>(&ctx->keys)};
     THC_CUDA(cudaLaunchKernelExC(&cfg, kern, args));

@@ -69,7 +69,8 @@ enum PipeMode { kCompressF32, kCompressBF16, kDecompress8, kDecompress16, kDecom
                 kCompressF32Fused,     // fp32 compress that also computes the block scales (below)
                 kErrorFeedback,        // e_i = x_i - RHT^-1(X_i) from worker i's own packed indices
                 kRangeF32,             // exact min / max of the rotated coordinates per RHT block
-                kAggDecompress };      // decompress straight from the workers' packed indices (PS line + estimate line)
+                kAggDecompress,        // decompress straight from the workers' packed indices (PS line + estimate line)
+                kPipeModes };
 
 // Layout inside DeviceBlock::counters.  Every CTA hits `head` and `abort` for every task and
 // the completion counters of the slots in use: each gets its own 128-byte line (head, exited,

@@ -76,6 +76,26 @@ int cudaFuncSetAttribute(const void *f, int attr, int value)
     return 0;
 }
 
+/* What a B200 answers for kernels of 128 registers per thread: four CTAs of 128 threads or two of 256 per SM,
+ * less where shared memory is short; clusters of eight do not fill the SMs. */
+int cudaOccupancyMaxActiveBlocksPerMultiprocessor(int *n, const void *f, int threads, size_t smem)
+{
+    (void)f;
+    const int by_smem = (int)(233472 / (smem + 1024)), by_regs = 512 / threads;
+    *n = by_smem < by_regs ? by_smem : by_regs;
+    return 0;
+}
+
+int cudaOccupancyMaxActiveClusters(int *n, const void *f, const cudaLaunchConfig_t *c)
+{
+    static const int of_eight[5] = {0, 15, 33, 48, 71};
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, f, (int)c->blockDim.x, c->dynamicSmemBytes);
+    for (unsigned i = 0; i < c->numAttrs; ++i)
+        if (c->attrs[i].id == cudaLaunchAttributeClusterDimension)
+            *n = c->attrs[i].val.clusterDim.x == 8 ? of_eight[*n] : 148 * *n / (int)c->attrs[i].val.clusterDim.x;
+    return 0;
+}
+
 int cudaLaunchKernel(const void *f, struct dim3 g, struct dim3 b, void **args, size_t smem, void *st)
 {
     (void)args; (void)st;

@@ -121,3 +121,23 @@ assert max(sets.values()) == 1
 assert all(limit[f] >= largest[f] for f in largest)
 """)
     assert out.split()[1] == "1"
+
+
+@pytest.mark.parametrize("k,g,ctas", [
+    (3, 30, 592), (12, 30, 592), (12, 166, 592), (12, 167, 444), (12, 255, 444), (3, 255, 296), (14, 255, 296), (15, 255, 296),
+    (16, 166, 8 * 71), (16, 255, 8 * 48),
+])
+def test_grid_of_the_block_kernel_is_what_the_gpu_holds(child, k, g, ctas):
+    """The CTAs walk over the tasks in a fixed stride: one that has to wait for another to end doubles the time."""
+    child(f"""
+k, g, ctas = {k}, {g}, {ctas}
+c = context(k, granularity=g, table=W.TABLES[(4, 30)][:15] + (g,), workers=1)
+d = 64 << 16 if k == 16 else 1 << 26
+for _ in range(2):
+    c.compress(buf[:1], d, 0, buf[0], buf[:1], ws, stream=0)
+    assert [r[2] for r in log() if r[0] == "launch"] == [min(ctas, 8 * 64) if k == 16 else ctas]
+    c.decompress(buf[0], 1, d, 0, buf[1], buf[2], ws, stream=0)     # no table
+    assert [r[2] for r in log() if r[0] == "launch"] == [8 * 64 if k == 16 else 296 if k in (14, 15) else 592]
+    c.compress(buf[:1], 5, 0, buf[0], buf[:1], ws, stream=0)
+    assert [r[2] for r in log() if r[0] == "launch"] == [8 if k == 16 else 2 if k == 15 else 1]                                  # one tile or cluster
+""")
