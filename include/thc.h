@@ -232,7 +232,7 @@ int thc_prepare_minmax(thc_ctx *ctx, const void *const *grads, uint32_t n, uint6
  * (the simulated cluster): same arguments and results as the two calls in a row, `scales`
  * (device, nblocks floats) being written here and usable by thc_decompress afterwards.
  * Section 5.3 observes that the norm exchange can overlap the RHT: only the quantiser needs M,
- * so where the block size is 2^17 (more than 14 blocks over all workers) to 2^20, the input fp32
+ * so where the block size is 2^17 (more than some 15 blocks over all workers) to 2^20, the input fp32
  * and n small enough for the intermediate ring to stay in L2, the transform kernel sums the squares
  * of the tiles it loads anyway and the gradients are read from HBM once instead of twice.  Elsewhere this runs the two calls.
  * The fp64 sums are added in a different (fixed) order than thc_prepare's, so a scale may

@@ -697,6 +697,7 @@ struct thc_ctx {
     bool pipeline_next;         // the queue of the next pipeline launch is set (thc_debug_skip_tasks); until then
                                 // blocks above 2^14 take the pipeline
     int sm_count;
+    int lone_clusters;          // see block_kernel_serves; blocks of 2^17 only
     // Encoded tensor maps of recent launches, keyed by what they describe: a training loop calls
     // with the same buffers every step, and encoding up to n + 1 maps per call costs more host
     // time than a small launch takes on the device.
@@ -741,6 +742,56 @@ static cudaError_t launch_after(void (*kern)(P...), dim3 grid, unsigned threads,
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kern, P(args)...);
+}
+
+// No launch takes more dynamic shared memory: a pipeline CTA, a tile of 2^14 or one of 2^13 with the constants
+// of 1024 blocks, each with a table of 256 entries, take up to 101 KB.  (More than half an SM's 228 KB, so that
+// count_lone_clusters can ask for one CTA per SM.)
+constexpr size_t kMaxDynamicSmem = 120u << 10;
+static_assert(1024 + 2 * kPElems * 4 + kPSignWords * 4 + 256 * kLutEntryBytes + kBlockConstMax * 8 <= kMaxDynamicSmem, "pipeline");
+static_assert(1024 + (4 << 14) + (1 << 14) / 4 + 16 + 256 * kLutEntryBytes <= kMaxDynamicSmem, "tile of 2^14");
+static_assert(1024 + (4 << 13) + (1 << 13) / 4 + 1024 * 16 + 256 * kLutEntryBytes <= kMaxDynamicSmem, "tile of 2^13");
+
+// Lets a kernel use more than the default 48 KB.  The limit is the same for every launch of every kernel, so
+// that no thread can lower it between another's call and its launch; what is done is remembered per kernel
+// and device, and done again (to the same effect) should the table be full.
+static int ensure_dynamic_smem(const void *kern)
+{
+    constexpr uint32_t kSlots = 2048;                  // of some 300 kernels
+    static std::mutex guard;
+    static const void *seen_kern[kSlots];
+    static int seen_dev[kSlots];
+    static uint32_t used = 0;
+    int dev = 0;
+    THC_CUDA(cudaGetDevice(&dev));
+    std::lock_guard<std::mutex> lock(guard);
+    uint32_t slot = (uint32_t)((reinterpret_cast<uintptr_t>(kern) >> 4) * 0x9E3779B9u + (uint32_t)dev) % kSlots;
+    while (seen_kern[slot] != nullptr) {               // never full: a quarter stays free
+        if (seen_kern[slot] == kern && seen_dev[slot] == dev) return THC_OK;
+        slot = (slot + 1u) % kSlots;
+    }
+    THC_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxDynamicSmem));
+    if (used < kSlots / 4 * 3) { seen_kern[slot] = kern; seen_dev[slot] = dev; ++used; }
+    return THC_OK;
+}
+
+// Clusters of eight CTAs that find an SM for each CTA (15 on a B200 of 148 SMs: a cluster stays within one GPC).
+static cudaError_t count_lone_clusters(int sm_count, int *n)
+{
+    const void *kern = block_kernel(kDecompress8, 4, true, 17u);
+    if (ensure_dynamic_smem(kern) != THC_OK) return g_last_cuda;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = 1u << block_cluster_log2(block_kind(17u));
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cudaLaunchConfig_t shape;
+    memset(&shape, 0, sizeof shape);
+    shape.gridDim = dim3((unsigned)sm_count * attr.val.clusterDim.x);
+    shape.blockDim = dim3((1u << block_tile_log2(block_kind(17u))) / 64u);
+    shape.dynamicSmemBytes = kMaxDynamicSmem;
+    shape.attrs = &attr;
+    shape.numAttrs = 1;
+    return cudaOccupancyMaxActiveClusters(n, kern, &shape);
 }
 
 static bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
@@ -806,6 +857,7 @@ int thc_create(const thc_config *cfg, thc_ctx **out)
     ctx->device = -1;
     ctx->dev = nullptr;
     ctx->sm_count = 148;
+    ctx->lone_clusters = 15;
     ctx->map_cache_used = 0;
     ctx->map_cache_next = 0;
     for (auto &r : ctx->resident) r.store(0u, std::memory_order_relaxed);
@@ -844,6 +896,7 @@ int thc_create(const thc_config *cfg, thc_ctx **out)
         if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void **>(&ctx->dev), sizeof(DeviceBlock));
         if (e == cudaSuccess) e = cudaMemcpy(ctx->dev, h, sizeof(DeviceBlock), cudaMemcpyHostToDevice);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&ctx->sm_count, cudaDevAttrMultiProcessorCount, dev);
+        if (e == cudaSuccess && cfg->log2_block == 17) e = count_lone_clusters(ctx->sm_count, &ctx->lone_clusters);
         if (e != cudaSuccess) {
             if (ctx->dev) cudaFree(ctx->dev);
             delete h;
@@ -869,15 +922,23 @@ int thc_destroy(thc_ctx *ctx)
 
 static uint64_t round_up(uint64_t v, uint64_t a) { return (v + a - 1) / a * a; }
 
-// Which blocks are held in shared memory (thc_block.cu), by size and coordinates over all workers.
-// Blocks up to 2^15 always; 2^16 up to 2^22 coordinates over all workers, where the two-pass pipeline
-// has less than a task per CTA and its chain of queue, ring and counters is all latency: 8.8 us
-// instead of 13.9 on a block or two, 21 instead of 23 on 2^22 coordinates; on 2^24 the cluster's
-// gather makes it 74 against 53.  2^17 up to 14 blocks, the clusters of eight half SMs that are resident
-// at a time: 13.1 us instead of 19.1 on 12 blocks, 18.6 against 19.4 on 16.
-static bool block_kernel_serves(uint32_t k, uint64_t coords)
+// Which blocks are held in shared memory (thc_block.cu), by size and coordinates over all workers; the others
+// take the two-pass pipeline, whose chain of queue, ring and counters is all latency on a few blocks.
+// Blocks up to 2^15 always.  2^16 and 2^17 as long as the clusters run side by side.  us, cluster / pipeline:
+//   2^16   blocks          8           32           64           65           72           96
+//          compress    8.5 / 13.2  13.6 / 18.0  20.2 / 22.1  21.1 / 22.2  24.8 / 23.2  29.0 / 24.6
+//          decompress  7.3 / 11.6  12.4 / 16.3  18.7 / 20.6  19.4 / 20.7  21.1 / 21.8  29.0 / 23.1
+//   (71 clusters are resident, four CTAs to an SM; from 72 on there is a second wave.  The one-call tail is the
+//   exception, level at 64 and 0.6 to 1.9 us slower in clusters from 48 to 56; 2^24 coordinates 74 / 53.)
+//   2^17   blocks          8           14           15           16           18           32
+//          compress   12.3 / 14.9  13.3 / 18.2  13.3 / 18.2  18.6 / 18.3  19.5 / 18.5  25.4 / 22.5
+//          decompress 11.3 / 14.1  12.2 / 17.4  12.2 / 17.4  17.4 / 17.3  17.9 / 17.2  22.6 / 20.8
+//   (up to 15 clusters have an SM for each CTA; from 16 on two CTAs share one.  Scales + compress of 15 blocks:
+//   18.7 in two calls, 21.2 as one launch of the pipeline.)
+static bool block_kernel_serves(const thc_ctx *ctx, uint64_t coords)
 {
-    return k <= 15u || (k == 16u && coords <= (1ull << 22)) || (k == 17u && coords <= (14ull << 17));
+    const uint32_t k = ctx->cfg.log2_block;
+    return k <= 15u || (k == 16u && coords <= (1ull << 22)) || (k == 17u && coords <= (uint64_t)ctx->lone_clusters << 17);
 }
 
 // Schedule of the persistent pipeline for `wb_count` worker-blocks of 2^k coordinates:
@@ -915,7 +976,7 @@ static bool plan_pipeline_fused(const thc_ctx *ctx, uint64_t nblocks, uint32_t n
 {
     const uint32_t k = ctx->cfg.log2_block;
     // (2^16: 4 % at most)
-    if (k < 17u || k > 20u || ctx->cfg.in_dtype != THC_F32 || block_kernel_serves(k, (nblocks * n) << k)) return false;
+    if (k < 17u || k > 20u || ctx->cfg.in_dtype != THC_F32 || block_kernel_serves(ctx, (nblocks * n) << k)) return false;
     if (ctx->cfg.range_mode != THC_RANGE_NORM) return false;
     const uint64_t wb_count = nblocks * n;
     PipePlan p = plan_pipeline(ctx, wb_count);
@@ -1035,36 +1096,6 @@ int thc_prepare(thc_ctx *ctx, const void *const *grads, uint32_t n, uint64_t d, 
         THC_CUDA(launch_after(prepare_final_kernel, dim3((unsigned)((sz.nblocks + 3) / 4)), 128, 0, st, 
             partial, n, sz.nblocks, chunks_per_block, chunks_per_worker, t_p, k, scales, ctx->dev));
     }
-    return THC_OK;
-}
-
-// The largest dynamic shared memory of any launch: a pipeline CTA, a tile of 2^14 or one of 2^13 with the
-// constants of 1024 blocks, each with a table of 256 entries.
-constexpr size_t kMaxDynamicSmem = 104u << 10;
-static_assert(1024 + 2 * kPElems * 4 + kPSignWords * 4 + 256 * kLutEntryBytes + kBlockConstMax * 8 <= kMaxDynamicSmem, "pipeline");
-static_assert(1024 + (4 << 14) + (1 << 14) / 4 + 16 + 256 * kLutEntryBytes <= kMaxDynamicSmem, "tile of 2^14");
-static_assert(1024 + (4 << 13) + (1 << 13) / 4 + 1024 * 16 + 256 * kLutEntryBytes <= kMaxDynamicSmem, "tile of 2^13");
-
-// Lets a kernel use more than the default 48 KB.  The limit is the same for every launch of every kernel, so
-// that no thread can lower it between another's call and its launch; what is done is remembered per kernel
-// and device, and done again (to the same effect) should the table be full.
-static int ensure_dynamic_smem(const void *kern)
-{
-    constexpr uint32_t kSlots = 2048;                  // of some 300 kernels
-    static std::mutex guard;
-    static const void *seen_kern[kSlots];
-    static int seen_dev[kSlots];
-    static uint32_t used = 0;
-    int dev = 0;
-    THC_CUDA(cudaGetDevice(&dev));
-    std::lock_guard<std::mutex> lock(guard);
-    uint32_t slot = (uint32_t)((reinterpret_cast<uintptr_t>(kern) >> 4) * 0x9E3779B9u + (uint32_t)dev) % kSlots;
-    while (seen_kern[slot] != nullptr) {               // never full: a quarter stays free
-        if (seen_kern[slot] == kern && seen_dev[slot] == dev) return THC_OK;
-        slot = (slot + 1u) % kSlots;
-    }
-    THC_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxDynamicSmem));
-    if (used < kSlots / 4 * 3) { seen_kern[slot] = kern; seen_dev[slot] = dev; ++used; }
     return THC_OK;
 }
 
@@ -1301,7 +1332,7 @@ static int launch_pipeline(thc_ctx *ctx, pipe_kernel_t kern, bool compress_f32,
 static bool use_block_kernel(const thc_ctx *ctx, uint64_t coords)
 {
     const uint32_t k = ctx->cfg.log2_block;
-    return k <= (uint32_t)kChunkLog2 || (!ctx->pipeline_next && block_kernel_serves(k, coords));
+    return k <= (uint32_t)kChunkLog2 || (!ctx->pipeline_next && block_kernel_serves(ctx, coords));
 }
 
 // CTAs (clusters) of a block kernel that the GPU holds at a time, as the runtime counts them.  A tile of 2^13 with

@@ -1,6 +1,6 @@
 """Blocks held in shared memory (thc_block.cu) at the edges of their tiles: one coordinate more or
-less than a tile, several tiles per CTA, clusters (2^15, 2^16) and the size from which 2^16 blocks
-take the two-pass pipeline, for fp32 and bf16 gradients: every step against the oracle."""
+less than a tile, several tiles per CTA, clusters (2^15 .. 2^17) and the sizes from which 2^16 and 2^17
+blocks take the two-pass pipeline, for fp32 and bf16 gradients: every step against the oracle."""
 import numpy as np
 import pytest
 
@@ -15,6 +15,7 @@ pytestmark = pytest.mark.gpu
     (12, 5_000_001, 2, "f32", 4), (13, 8192, 1, "f32", 8), (13, 5_000_000, 2, "bf16", 1), (14, 16_385, 2, "f32", 4),
     (14, 5_100_003, 2, "f32", 4), (15, 32_769, 3, "bf16", 4), (15, 10_000_019, 1, "f32", 2), (16, 65_535, 2, "f32", 4),
     (16, 1 << 22, 1, "f32", 4), (16, (1 << 22) + 1, 1, "f32", 4), (16, 65_537, 20, "bf16", 4),
+    (17, 5 * (1 << 17) - 3, 3, "f32", 4), (17, 8 * (1 << 17) - 3, 2, "bf16", 4),
 ])
 def test_edges_of_tiles_and_clusters(k, d, n, dtype, bits):
     import torch

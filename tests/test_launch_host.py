@@ -141,3 +141,30 @@ for _ in range(2):
     c.compress(buf[:1], 5, 0, buf[0], buf[:1], ws, stream=0)
     assert [r[2] for r in log() if r[0] == "launch"] == [8 if k == 16 else 2 if k == 15 else 1]                                  # one tile or cluster
 """)
+
+
+@pytest.mark.parametrize("k,last", [(16, 64), (17, 15)])
+def test_largest_number_of_blocks_held_in_clusters(child, k, last):
+    """Up to `last` blocks over all workers are held in clusters, more take the pipeline; scales + compress is one
+    launch only where compress takes the pipeline."""
+    child(f"""
+k, last = {k}, {last}
+c = context(k)
+for blocks in (1, last, last + 1):
+    for n in (1, blocks):
+        d = blocks // n << k
+        x = buf[:1] * n
+        want = ["block" if blocks <= last else "pipeline"]
+        if n <= 64:
+            c.compress(x, d, 0, buf[0], x, ws, stream=0)
+            assert kernels() == want, (blocks, n)
+            c.error_feedback(x, x, d, 0, buf[0], x, ws, stream=0)
+            assert kernels() == want, (blocks, n)
+            fused = c.sizes(d, n).fused_scales
+            assert not fused or want == ["pipeline"]
+            c.prepare_compress(x, d, 0, buf[0], x, ws, stream=0)
+            assert len(kernels()) == 2 - fused
+        if n == 1:
+            c.decompress(buf[0], 1, d, 0, buf[1], buf[2], ws, stream=0)
+            assert kernels() == want, blocks
+""")
