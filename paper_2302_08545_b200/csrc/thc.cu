@@ -1,8 +1,8 @@
 // libthc: kernels and C ABI.  See include/thc.h for the contract of every entry point.
 //
-// Structure of the transform.  RHT blocks of up to 2^16 coordinates are held in shared memory by one
-// CTA or a cluster (thc_block.cuh); larger blocks go through the persistent two-pass pipeline of
-// thc_pipeline.cuh.
+// Structure of the transform.  RHT blocks of up to 2^15 coordinates, and few blocks of 2^16 or 2^17, are held
+// in shared memory by one CTA or a cluster (thc_block.cu; block_kernel_serves has the rule); the others go
+// through the persistent two-pass pipeline of thc_pipeline.cuh.
 #include "../../include/thc.h"
 #include "thc_device.cuh"
 
@@ -59,13 +59,6 @@ quantize_rotated_kernel(PtrArray rotated, MutPtrArray packed, uint64_t d_pad, ui
     }
 }
 
-// Fast path of the PS sum for 4-bit indices, 8-bit sums and table values below 128 (the
-// paper's prototype: 4-bit indices, 8-bit table values and sums, Section 3).  The 16 table
-// bytes sit in four registers; `prmt` looks four indices up at once.  A selector nibble with
-// bit 3 set makes prmt return the sign of the selected byte, i.e. 0 for values < 128, so the
-// low half of the table answers indices 0-7 and, with bit 3 flipped, the high half answers
-// 8-15; the two results are disjoint and are added into packed byte accumulators (no byte
-// can overflow because workers * g <= 255).
 // 32 bytes of sums to a 16-byte aligned address; in one store where it is 32-byte aligned, so that no
 // sector of 32 bytes reaches the L2 in two halves.
 __device__ __forceinline__ void store_sums32(uint4 *p, bool aligned32, const uint32_t (&v)[8])
@@ -79,6 +72,13 @@ __device__ __forceinline__ void store_sums32(uint4 *p, bool aligned32, const uin
     }
 }
 
+// Fast path of the PS sum for 4-bit indices, 8-bit sums and table values below 128 (the
+// paper's prototype: 4-bit indices, 8-bit table values and sums, Section 3).  The 16 table
+// bytes sit in four registers; `prmt` looks four indices up at once.  A selector nibble with
+// bit 3 set makes prmt return the sign of the selected byte, i.e. 0 for values < 128, so the
+// low half of the table answers indices 0-7 and, with bit 3 flipped, the high half answers
+// 8-15; the two results are disjoint and are added into packed byte accumulators (no byte
+// can overflow because workers * g <= 255).
 __global__ void __launch_bounds__(kThreads)
 aggregate_b4w8_kernel(PtrArray in, uint32_t n, uint64_t units32, const DeviceBlock *dev,
                       uint4 *__restrict__ sum)
@@ -1093,13 +1093,14 @@ int thc_prepare(thc_ctx *ctx, const void *const *grads, uint32_t n, uint64_t d, 
         THC_CUDA(launch_after(prepare_partial_kernel<false>, grid, kThreads, 0, st, in, d, chunk_log2, chunks_per_worker, partial, counters,
                                                                  chunks_per_block, t_p, k, scales, ctx->dev));
     if (counters == nullptr) {
-        THC_CUDA(launch_after(prepare_final_kernel, dim3((unsigned)((sz.nblocks + 3) / 4)), 128, 0, st, 
+        THC_CUDA(launch_after(prepare_final_kernel, dim3((unsigned)((sz.nblocks + 3) / 4)), 128, 0, st,
             partial, n, sz.nblocks, chunks_per_block, chunks_per_worker, t_p, k, scales, ctx->dev));
     }
     return THC_OK;
 }
 
-// ---- persistent pipeline dispatch (RHT blocks of 2^15 .. 2^24 coordinates)
+// ---- persistent pipeline dispatch (RHT blocks of 2^16 .. 2^22 coordinates that block_kernel_serves leaves; 2^15 only
+// after thc_debug_skip_tasks)
 typedef void (*pipe_kernel_t)(const TmaMaps, PipeParams, PtrArrayP, MutPtrArrayP, MutPtrArrayP, PhiloxKeys);
 
 template <int MODE, int KB>
@@ -1130,15 +1131,15 @@ static pipe_kernel_t pick_pipe_kernel_kb(uint32_t bits, bool identity)
     }
 }
 
-// The 2^20-coordinate block (the paper's 4 MB partition) gets the compile-time geometry.
+// The 2^20-coordinate block (the paper's 4 MB partition) gets the compile-time geometry in every mode.
 template <int MODE>
 static pipe_kernel_t pick_pipe_kernel(uint32_t bits, bool identity, uint32_t k)
 {
     if constexpr (MODE == kCompressF32 || MODE == kCompressBF16) {
-        // 2^21 and 2^22 (the largest configuration): the generic path with its geometry fixed at
-        // compile time
-        // (4-bit indices only, the width of every benchmark configuration with such blocks: each
-        // further instantiation costs build time)
+        // 2^21 and 2^22: geometry at compile time, pass B in two rounds (pass_b_low5, pass_b_high4).  4-bit
+        // indices only, the width of the configurations with such blocks.  The others would gain as
+        // much (4 x 2^26 fp32 coordinates, us: 2^21 b = 2 754 -> 638, b = 8 880 -> 786; 2^22 785 -> 674, 924 -> 833)
+        // and their 32 kernels would take a build from 131 to 164 s.
         if (k == 21 && bits == 4)
             return identity ? thc_pipeline_kernel<MODE, 4, true, 8> : thc_pipeline_kernel<MODE, 4, false, 8>;
         if (k == 22 && bits == 4)

@@ -1,4 +1,5 @@
-// Persistent dataflow kernel for RHT blocks larger than one shared-memory tile (k >= 15).
+// Persistent dataflow kernel for RHT blocks that are not held in shared memory (thc_block.cu): 2^16 .. 2^22, of
+// 2^16 and 2^17 only where there are many.  (2^15 gets here after thc_debug_skip_tasks alone, a test hook.)
 //
 // Work is cut into tasks of one 2^13-coordinate tile each, run by CTAs of 128 threads:
 //   A(wb, t)  pass A of tile t of worker-block wb: consecutive coordinates, stages of
@@ -59,7 +60,7 @@ constexpr int kPChunks = kPElems / 4;
 constexpr int kPThreads = 128;                // compute threads of a CTA
 constexpr int kPCtaThreads = 160;             // plus one control warp that runs the queue
 constexpr int kPSignWords = 512;            // sign words: two slots of 256 (pass A) or one of 512
-constexpr int kMaxRing = 320;                // ring slots: blocks of 2^15 need up to 280 to cover the tasks in flight
+constexpr int kMaxRing = 320;                // ring slots: blocks of 2^16 need up to 142 to cover the tasks in flight (2^15: 280)
 constexpr uint32_t kFusedBlocks = 160;       // fused scales: blocks in flight have counters of their own
 static_assert(2 * kFusedBlocks <= (uint32_t)kMaxRing, "the block counters share the tile counters' array");
 constexpr int kBlockConstMax = 256;         // per-block constants cached in shared memory
@@ -1026,7 +1027,8 @@ __device__ __forceinline__ void pass_b_high4(const float4 *tile, int tid, const 
 }
 
 // ------------------------------------------------------------------------------ the kernel
-// KB = 7 specialises the k = 20 geometry at compile time; KB = 0 reads it from the params.
+// KB = 7 specialises the k = 20 geometry at compile time, KB = 8 and 9 (compress) that of k = 21 and 22;
+// KB = 0 reads it from the params.
 template <int MODE, int BITS, bool IDENTITY, int KB>
 __global__ void __launch_bounds__(kPCtaThreads, 3)
 thc_pipeline_kernel(const __grid_constant__ TmaMaps maps, PipeParams P, PtrArrayP in,

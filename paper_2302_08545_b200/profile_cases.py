@@ -17,7 +17,8 @@ buffer), warms the calls up, times them with CUDA events and prints one JSON lin
   minmax            thc_prepare_minmax + compress in exact-range mode (thc_pipeline_kernel<range>)
   aggdec            thc_aggregate_decompress (thc_pipeline_kernel<aggregate + decompress>)
   fused             thc_prepare_compress, n = 8 (thc_pipeline_kernel<fused scales + compress>)
-  scan              compress and decompress of 4 x 2^26 fp32 coordinates for B = 2^15 .. 2^22 (one line each)
+  scan              compress, decompress and error feedback of 4 x 2^26 fp32 coordinates for B = 2^8 .. 2^22 (a
+                    line each; blocks held in shared memory up to 2^15, the two-pass pipeline above)
   cfg1 .. cfg4, cfg3b2   the benchmark configurations at full size, inputs generated on the device
                     (per-call times of the round, error feedback and the one-call tail included)
 """
@@ -29,7 +30,7 @@ import json
 from . import workloads as W
 
 
-W_PEAK = 6549.8   # GB/s: the machine's measured HBM copy rate (MEASURED_PEAKS.json), for the printed fraction
+W_PEAK = 6549.8   # GB/s: the measured HBM copy rate (MEASURED_PEAKS.json), for the printed fraction
 
 
 def _time(fn, iters, torch, stream):
@@ -49,11 +50,11 @@ def _time(fn, iters, torch, stream):
 
 
 def scan(iters: int):
-    """Block-size scan: the same 4 x 2^26 coordinates through every two-pass block size."""
+    """Block-size scan: the same 4 x 2^26 coordinates in blocks of every size."""
     import torch
     from . import runner
     stream = torch.cuda.current_stream()
-    for k in range(15, 23):
+    for k in (8, 10, *range(12, 23)):
         w = W.Workload(f"scan_k{k}", n=4, d=1 << 26, log2_block=k, bits=4, granularity=30,
                        table=W.TABLES[(4, 30)], data_seed=5)
         ctx = runner.context_for(w)
@@ -63,9 +64,11 @@ def scan(iters: int):
         tc = _time(lambda: r.compress(0), iters, torch, stream)
         r.aggregate()
         td = _time(lambda: r.decompress(0), iters, torch, stream)
-        print(json.dumps({"case": "scan", "log2_block": k, "compress_ms": round(tc, 4),
-                          "decompress_ms": round(td, 4), "status_flags": ctx.status()}), flush=True)
-        del r, ctx
+        ef = [torch.zeros(w.d, dtype=torch.float32, device=r.device) for _ in range(w.n)]
+        te = _time(lambda: ctx.error_feedback(r.grads, r.packed, w.d, 0, r.scales, ef, r.workspace), iters, torch, stream)
+        print(json.dumps({"case": "scan", "log2_block": k, "compress_ms": round(tc, 4), "decompress_ms": round(td, 4),
+                          "error_feedback_ms": round(te, 4), "status_flags": ctx.status()}), flush=True)
+        del r, ctx, ef
         torch.cuda.empty_cache()
 
 
