@@ -35,17 +35,17 @@ from paper_2302_08545_b200 import workloads as W  # noqa: E402
 METRIC = "gradient GB/s per compress+aggregate+decompress round; % of HBM roofline"
 UNIT = "GB/s"
 KERNELS_PER_STEP = {"prepare": 1, "compress": 1, "prepare_compress": 1, "aggregate": 1, "decompress": 1}
-# DRAM bytes per (worker, padded coordinate) of the compress kernel (n = 4, d = 2^24, b = 4) and of
+# DRAM bytes per (worker, padded coordinate) of the 2^20 compress kernel (n = 4, d = 2^24, b = 4) and of
 # its fused-scales variant (n = 8, d = 2^24, b = 4: its ring grows with n), measured with ncu
 # (profiles/thc_pipeline_kernel_d2p24_b4.md); traffic grows in proportion to n*d_pad, so a full
 # launch is this times n*d_pad.
-NCU_COMPRESS_DRAM_BYTES_PER_COORD = {("f32", 4): 5.296}
-NCU_FUSED_DRAM_BYTES_PER_COORD = {("f32", 4): 9.206}
+NCU_COMPRESS_DRAM_BYTES_PER_COORD = {("f32", 4): 5.222}
+NCU_FUSED_DRAM_BYTES_PER_COORD = {("f32", 4): 9.194}
 # Executed thread-instructions per (worker, padded coordinate) from the same captures
 # (smsp__inst_executed x 32 / coordinates): the kernel is bound by the shared-memory data pipe
 # and instruction issue rather than by HBM, so the issue rate is reported beside the HBM fraction.
-NCU_COMPRESS_THREAD_INST_PER_COORD = {("f32", 4): 46.1}
-NCU_FUSED_THREAD_INST_PER_COORD = {("f32", 4): 49.0}
+NCU_COMPRESS_THREAD_INST_PER_COORD = {("f32", 4): 45.3}
+NCU_FUSED_THREAD_INST_PER_COORD = {("f32", 4): 48.8}
 
 
 def pick_workload(name: str) -> W.Workload:
@@ -62,7 +62,7 @@ def measured_peaks():
     if os.path.exists(path):
         with open(path) as f:
             return float(json.load(f)["hbm_gbs"]), "measured (MEASURED_PEAKS.json)"
-    return 6650.0, "fallback (earlier pool measurement)"
+    return 6650.0, "fallback (an earlier measurement)"
 
 
 class ClockSampler:
@@ -433,12 +433,12 @@ def run_gpu(args):
     in_bytes_pad = w.n * w.d_pad * (4 if w.in_dtype == "f32" else 2)
     per_coord = (NCU_FUSED_DRAM_BYTES_PER_COORD if fused else NCU_COMPRESS_DRAM_BYTES_PER_COORD).get(
         (w.in_dtype, w.bits))
-    traffic = None if per_coord is None or w.log2_block < 15 else per_coord * w.n * w.d_pad
+    traffic = None if per_coord is None or w.log2_block != 20 else per_coord * w.n * w.d_pad
     clk = clocks.summary()
     inst = (NCU_FUSED_THREAD_INST_PER_COORD if fused else NCU_COMPRESS_THREAD_INST_PER_COORD).get(
         (w.in_dtype, w.bits))
     issue = None
-    if inst is not None and w.log2_block >= 15 and clk.get("sm_mhz"):
+    if inst is not None and w.log2_block == 20 and clk.get("sm_mhz"):
         sms = torch.cuda.get_device_properties(dev).multi_processor_count
         lane_peak = sms * 128 * clk["sm_mhz"] * 1e6
         lane_rate = inst * w.n * w.d_pad / (comp_ms * 1e-3)
