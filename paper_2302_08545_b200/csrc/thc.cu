@@ -1336,15 +1336,22 @@ static bool use_block_kernel(const thc_ctx *ctx, uint64_t coords)
     return k <= (uint32_t)kChunkLog2 || (!ctx->pipeline_next && block_kernel_serves(ctx, coords));
 }
 
-// CTAs (clusters) of a block kernel that the GPU holds at a time, as the runtime counts them.  A tile of 2^13 with
+// CTAs (clusters) of a block kernel that the GPU holds at a time.  A tile of 2^13 with
 // a table of more than 167 entries leaves room for three CTAs per SM instead of four: with 592 CTAs in the grid,
 // each with a fixed share of the tasks, a quarter of them started when others had ended.  Compress with a 4-bit
 // table of 256 entries, 592 against 444 CTAs: 4 x 2^22 coordinates in blocks of 2^12 37.7 -> 34.5 us, 4 x 2^24
 // 123.7 -> 117.6, 8 x 3,000,001 in blocks of 2^13 50.7 -> 47.1; over 448 .. 3500 tiles 22 % faster to 5 % slower
 // (near 700 and 1000 tiles, where 592 leave the shorter last round).  Of clusters of eight there are fewer than the
-// SMs have room for, since a cluster stays within one GPC (2^16: 71, or 48 with such a table: 4 x 2^20 coordinates 28.1 -> 24.5 us).
+// SMs have room for, since a cluster stays within one GPC (2^16: 48 with such a table: 4 x 2^20 coordinates 28.1 -> 24.5 us).
+// The runtime is asked only where shared memory leaves less room than the kernel's registers do (four CTAs
+// or two): that adds some 0.5 us to a context's first call.  Elsewhere no more clusters are launched than
+// there are (block_kernel_serves).
+constexpr size_t kSmemPerSm = 228u << 10, kSmemPerCta = 1024u + 256u;     // reserved and static
 static int resident_units(const thc_ctx *ctx, PipeMode mode, const void *kern, const cudaLaunchConfig_t &shape, uint32_t e, uint32_t *units)
 {
+    const uint32_t by_registers = shape.blockDim.x == 128u ? 4u : 2u;
+    *units = ((uint32_t)ctx->sm_count * by_registers) >> e;
+    if (shape.dynamicSmemBytes + kSmemPerCta <= kSmemPerSm / by_registers) return THC_OK;
     *units = ctx->resident[mode].load(std::memory_order_relaxed);
     if (*units != 0u) return THC_OK;
     int n = 0;
