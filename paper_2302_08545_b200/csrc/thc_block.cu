@@ -26,7 +26,7 @@
 // 669 -> 441 us, decompress 156 -> 95 us, error feedback 1310 -> 509 us; 2^14 681 -> 435, 155 -> 115,
 // 1316 -> 539 us.  In a cluster the gather binds (a tile of every CTA crosses the SM-to-SM network: 8740
 // cycles for the last round of a tile of 2^15 where one of 2^14 takes 1580): 2^15 is as fast as the
-// two-pass pipeline on large inputs (645 us; error feedback 985 -> 763 us) and takes 9.4 instead of 14 us on
+// two-pass pipeline on large inputs (645 us; error feedback 985 -> 763 us) and takes 9.3 instead of 13.1 us on
 // a few blocks; 2^16 and 2^17 pay only there (see block_kernel_serves).
 #include "thc_block.h"
 
