@@ -8,7 +8,8 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("k,nblk,n,bits", [(17, 16, 5, 8), (17, 130, 2, 4), (18, 20, 3, 3), (19, 9, 4, 1),
-                                           (18, 131, 1, 4)])
+                                           (18, 131, 1, 4), (17, 16, 1, 4), (18, 1, 1, 4), (18, 14, 3, 2),
+                                           (19, 2, 1, 8), (19, 6, 4, 4), (20, 2, 1, 1), (20, 4, 4, 4)])
 def test_one_launch_equals_the_two_calls(k, nblk, n, bits):
     import torch
     from paper_2302_08545_b200 import runner

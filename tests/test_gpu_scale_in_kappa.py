@@ -1,6 +1,7 @@
-"""Blocks whose 1/sqrt(B) is a power of two leave out the scaling of every coordinate where the clamp
-bound is of ordinary size: the indices without the rotated output (that path) and with it (the
-other one) equal each other and the oracle's, also for bounds far outside the ordinary sizes."""
+"""Compress of 2^20 blocks, whose 1/sqrt(B) is a power of two, leaves out the scaling of every coordinate where
+the clamp bound is of ordinary size: the indices without the rotated output (that path) and with it
+(the other one) equal each other and the oracle's, also for bounds far outside the ordinary sizes.
+Blocks of 2^22 scale every coordinate in both calls."""
 import numpy as np
 import pytest
 
