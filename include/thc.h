@@ -252,7 +252,7 @@ int thc_prepare_compress(thc_ctx *ctx, const void *const *grads, uint32_t n, uin
  *   grads    host array of n_local device pointers: the x_i that were compressed
  *   packed   host array of n_local device pointers: their packed indices
  *   ef       host array of n_local device pointers, d fp32 each, written
- *   workspace  as reported by thc_sizes (it includes room for one worker's table values)  */
+ *   workspace  as reported by thc_sizes                                                   */
 int thc_error_feedback(thc_ctx *ctx, const void *const *grads, const void *const *packed,
                        uint32_t n_local, uint64_t d, uint32_t round, const float *scales,
                        float *const *ef, void *workspace, uint64_t workspace_bytes, void *stream);

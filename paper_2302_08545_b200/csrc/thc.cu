@@ -1029,7 +1029,7 @@ int thc_sizes(const thc_ctx *ctx, uint64_t d, uint32_t n_local, thc_sizes_t *s)
             s->fused_scales = 1;
         }
     }
-    // scratch of prepare / the pipeline's ring, then one worker's table values (error feedback)
+    // scratch of prepare / the pipeline's ring, then the sums (thc_aggregate_decompress where it runs the two calls)
     s->workspace_bytes = round_up((prepare_ws > two_pass_ws ? prepare_ws : two_pass_ws) + 256, 256) +
                          round_up(s->sum_bytes, 256);
     return THC_OK;
