@@ -292,9 +292,13 @@ __device__ __forceinline__ uint32_t lut_lane_addr(const unsigned char *lut, int 
 // w0, w1: the four 16-bit variates.  `lut_addr` comes from lut_lane_addr (unused for the identity
 // table).  Returns the indices packed BITS apiece, coordinate 0 in the low bits: the compare is the
 // carry of an addition, and a multiply-add with carry shifts the indices so far, appends z0 and
-// adds it (0.7 instructions per coordinate less than compare and select).  With the 8-byte entries
-// the whole second word is added in, so the bits above 4 BITS are not defined (join_units cuts
-// them off).
+// adds it.  What is added for z0 is a whole word of which only the low half (table) or the low 24 bits
+// (identity: the bits of 2^23 + f) mean anything, so the bits above 4 BITS are not defined (join_units
+// cuts them off; 8 bits: the one 0x4B000000 that is left is taken off here).
+// Bound by dispatch slots.  What allows it is packed, two coordinates to an instruction; the variates are
+// inverted two at a time.  Cycles per coordinate of an SM's 128 lanes, alone, 12 warps per SM: 4 bits
+// 12.9 -> 11.5, 2 bits identity 10.5 -> 8.0, 1 bit 10.5 -> 4.5 (its f is 0 below u = 1, where 2^16 u is
+// above every variate, so the carry is the index).
 template <int BITS, bool IDENTITY>
 __device__ __forceinline__ uint32_t quantize4(float r0, float r1, float r2, float r3, float kappa, float offset,
                                               float gf, uint32_t w0, uint32_t w1, uint32_t lut_addr)
@@ -302,41 +306,63 @@ __device__ __forceinline__ uint32_t quantize4(float r0, float r1, float r2, floa
     constexpr bool kLut8 = LutKind<BITS, IDENTITY>::k8;
     const float r[4] = {r0, r1, r2, r3};
     const uint32_t words[2] = {w0, w1};
+    const float2 big = make_float2(8388608.0f, 8388608.0f), g2 = make_float2(gf, gf);
     uint32_t acc = 0u;
 #pragma unroll
-    for (int e = 3; e >= 0; --e) {
-        float u;
-        asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(u) : "f"(r[e]), "f"(kappa), "f"(offset));
-        const float t = __fmaf_rd(u, gf, 8388608.0f);          // 2^23 + floor(u * g)
-        // bits of 2^23 + u16
-        const uint32_t ub = (e & 1) ? __byte_perm(words[e >> 1], 0x4B000000u, 0x7432)
-                                    : __byte_perm(words[e >> 1], 0x4B000000u, 0x7410);
-        uint32_t zw;
-        float tau;
-        if (IDENTITY) {
-            zw = __float_as_uint(t) & 0xFFu;
-            const float delta = fmaf(u, gf, 8388608.0f - t);
-            tau = fmaf(delta, 65536.0f, 8388608.0f);
-        } else if (kLut8) {
-            const uint32_t a = __float_as_uint(t) * (uint32_t)kLutEntryBytes + lut_addr;
-            uint32_t x, y;
-            asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(x), "=r"(y) : "r"(a));
-            const float delta = fmaf(u, gf, __uint_as_float(y & 0xFFFF0000u));
-            tau = fmaf(delta, __uint_as_float(x), 8388608.0f);
-            zw = y;
+    for (int p = 1; p >= 0; --p) {
+        float2 u, tau;
+        asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(u.x) : "f"(r[2 * p]), "f"(kappa), "f"(offset));
+        asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(u.y) : "f"(r[2 * p + 1]), "f"(kappa), "f"(offset));
+        uint32_t zw[2] = {0u, 0u};
+        if (IDENTITY && BITS == 1) {
+            tau = __ffma2_rn(u, make_float2(65536.0f, 65536.0f), big);
         } else {
-            const uint32_t a = __float_as_uint(t) * (uint32_t)kLutEntryBytes + lut_addr;
-            uint32_t x, y, z, w;
-            asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(x), "=r"(y), "=r"(z), "=r"(w) : "r"(a));
-            const float delta = fmaf(u, gf, __uint_as_float(x));
-            tau = fmaf(delta, __uint_as_float(y), 8388608.0f);
-            zw = z;
+            const float2 t = __ffma2_rd(u, g2, big);           // 2^23 + floor(u * g)
+            if (IDENTITY) {
+                const float2 delta = __ffma2_rn(u, g2, __ffma2_rn(t, make_float2(-1.0f, -1.0f), big));
+                tau = __ffma2_rn(delta, make_float2(65536.0f, 65536.0f), big);
+                zw[0] = __float_as_uint(t.x);
+                zw[1] = __float_as_uint(t.y);
+            } else {
+                const float tf[2] = {t.x, t.y};
+                float nt[2], r16[2];
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const uint32_t a = __float_as_uint(tf[e]) * (uint32_t)kLutEntryBytes + lut_addr;
+                    uint32_t x, y;
+                    if (kLut8) {
+                        asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(x), "=r"(y) : "r"(a));
+                        nt[e] = __uint_as_float(y & 0xFFFF0000u);
+                        zw[e] = y;
+                    } else {
+                        uint32_t z, w;
+                        asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(y), "=r"(x), "=r"(z), "=r"(w) : "r"(a));
+                        nt[e] = __uint_as_float(y);
+                        zw[e] = z;
+                    }
+                    r16[e] = __uint_as_float(x);
+                }
+                const float2 delta = __ffma2_rn(u, g2, make_float2(nt[0], nt[1]));
+                tau.x = fmaf(delta.x, r16[0], 8388608.0f);
+                tau.y = fmaf(delta.y, r16[1], 8388608.0f);
+            }
         }
-        // carry out of tau + ~ub: ub < tau
-        asm("{\n\t.reg .u32 t;\n\tadd.cc.u32 t, %1, %2;\n\tmadc.lo.u32 %0, %0, %4, %3;\n\t}"
-            : "+r"(acc) : "r"(__float_as_uint(tau)), "r"(~ub), "r"(zw), "n"(1 << BITS));
+        const float tauf[2] = {tau.x, tau.y};
+        const uint32_t inv = ~words[p];
+#pragma unroll
+        for (int e = 1; e >= 0; --e) {
+            // ~ of the bits of 2^23 + u16
+            const uint32_t nub = __byte_perm(inv, 0xB4FFFFFFu, e ? 0x7632 : 0x7610);
+            // carry out of tau + ~ub: ub < tau
+            if (IDENTITY && BITS == 1)
+                asm("{\n\t.reg .u32 t;\n\tadd.cc.u32 t, %1, %2;\n\taddc.u32 %0, %0, %0;\n\t}"
+                    : "+r"(acc) : "r"(__float_as_uint(tauf[e])), "r"(nub));
+            else
+                asm("{\n\t.reg .u32 t;\n\tadd.cc.u32 t, %1, %2;\n\tmadc.lo.u32 %0, %0, %4, %3;\n\t}"
+                    : "+r"(acc) : "r"(__float_as_uint(tauf[e])), "r"(nub), "r"(zw[e]), "n"(1 << BITS));
+        }
     }
-    return acc;
+    return IDENTITY && BITS == 8 ? acc - 0x4B000000u : acc;
 }
 
 // Two groups of four indices as one unit of eight, coordinate 0 in the low bits.
