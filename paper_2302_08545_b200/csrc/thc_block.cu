@@ -669,7 +669,14 @@ thc_block_kernel(const __grid_constant__ TmaMaps maps, const __grid_constant__ B
         // cache); the second iteration's rows move down the register arrays
         const float gf = (float)P.granularity;
         const uint32_t my_lut = lut_lane_addr<LutKind<BITS, IDENTITY>::k8>(lut, tid);
+        // Offsets from the thread's first unit fit 32 bits; the rounding calls of a tile (of a cluster's block)
+        // share the high word of their counter (see EpilogueCtx).
+        const uint64_t limit = kForward ? P.d_pad : P.d;
+        const uint32_t left = j_out >= limit ? 0u : (uint32_t)min(limit - j_out, (uint64_t)1 << 31);
+        const uint32_t call_lo = (uint32_t)(j_out >> 3), call_hi = (uint32_t)(j_out >> 35);
         float *rot = kForward ? static_cast<float *>(rotated.p[cur_wl]) : nullptr;
+        if (rot != nullptr) rot += j_out;
+        unsigned char *packed = kQuant ? static_cast<unsigned char *>(outp.p[cur_wl]) + j_out / 8 * BITS : nullptr;
         uint32_t kmin = 0xFFFFFFFFu, kmax = 0u;
 #pragma unroll 1
         for (uint32_t half = 0; half < 2; ++half) {
@@ -677,17 +684,16 @@ thc_block_kernel(const __grid_constant__ TmaMaps maps, const __grid_constant__ B
             for (uint32_t mm = 0; mm < 4; ++mm) {
                 const uint32_t m = 4u * half + mm;
                 const uint32_t off = ((m & (C - 1u)) << kBLog2) + (m >> E) * (32u * kBRowStep);
-                const uint64_t j = j_out + off;
                 const float4 ra = scale4(a[mm], P.c_block), rb = scale4(b[mm], P.c_block);
                 if (kForward) {
-                    if (rot != nullptr && j < P.d_pad) {
-                        *reinterpret_cast<float4 *>(rot + j) = ra;
-                        *reinterpret_cast<float4 *>(rot + j + 4) = rb;
+                    if (rot != nullptr && off < left) {
+                        *reinterpret_cast<float4 *>(rot + off) = ra;
+                        *reinterpret_cast<float4 *>(rot + off + 4) = rb;
                     }
                     const float r[8] = {ra.x, ra.y, ra.z, ra.w, rb.x, rb.y, rb.z, rb.w};
                     if constexpr (kRange) {
                         uint32_t lo = 0xFFFFFFFFu, hi = 0u;
-                        if (j < P.d_pad) {
+                        if (off < left) {
 #pragma unroll
                             for (int e = 0; e < 8; ++e) {
                                 const uint32_t key = float_key(r[e]);
@@ -704,33 +710,33 @@ thc_block_kernel(const __grid_constant__ TmaMaps maps, const __grid_constant__ B
                                 lo = __reduce_min_sync(0xFFFFFFFFu, lo);
                                 hi = __reduce_max_sync(0xFFFFFFFFu, hi);
                             }
-                            if (j < P.d_pad && (k < 8u || lane == 0)) add_range(P.range_keys, P.nblocks, j >> k, lo, hi);
+                            if (off < left && (k < 8u || lane == 0)) add_range(P.range_keys, P.nblocks, (j_out + off) >> k, lo, hi);
                         }
                     } else {
                         const float2 kc = bc[KIND != 0 ? 0u : ((32u * rl + 8u * u + off) >> k)];
-                        const uint4 rnd = round_call(j, P.worker_base + cur_wl, P.round, keys);
+                        const uint4 rnd = philox4x32_10(call_lo + (off >> 3), call_hi, P.worker_base + cur_wl, P.round, keys);
                         const uint64_t z = quantize8<BITS, IDENTITY>(r, kc.x, kc.y, gf, rnd, my_lut);
-                        if (j < P.d_pad) store_unit<BITS>(static_cast<unsigned char *>(outp.p[cur_wl]), j, z);
+                        if (off < left) store_unit<BITS>(packed, off, z);
                     }
-                } else if (j < P.d) {
-                    float *out = static_cast<float *>(outp.p[kEF ? cur_wl : 0]);
-                    const float *xs = kEF ? static_cast<const float *>(rotated.p[cur_wl]) : nullptr;
+                } else if (off < left) {
+                    float *out = static_cast<float *>(outp.p[kEF ? cur_wl : 0]) + j_out;
+                    const float *xs = kEF ? static_cast<const float *>(rotated.p[cur_wl]) + j_out : nullptr;
                     const uint32_t word = ((m & (C - 1u)) << (kBLog2 - 5 - E)) + (uint32_t)rl + kBRowStep * (m >> E);
                     const uint32_t bits = sw[kBSignWords * par + word] >> (8 * u);
                     float4 oa = flip4(ra, bits), ob = flip4(rb, bits >> 4);
-                    if (j + 8 <= P.d) {
+                    if (off + 8 <= left) {
                         if (kEF) {
-                            const float4 xa = ld_global_once(reinterpret_cast<const float4 *>(xs + j));
-                            const float4 xb = ld_global_once(reinterpret_cast<const float4 *>(xs + j + 4));
+                            const float4 xa = ld_global_once(reinterpret_cast<const float4 *>(xs + off));
+                            const float4 xb = ld_global_once(reinterpret_cast<const float4 *>(xs + off + 4));
                             oa = make_float4(xa.x - oa.x, xa.y - oa.y, xa.z - oa.z, xa.w - oa.w);
                             ob = make_float4(xb.x - ob.x, xb.y - ob.y, xb.z - ob.z, xb.w - ob.w);
                         }
-                        *reinterpret_cast<float4 *>(out + j) = oa;
-                        *reinterpret_cast<float4 *>(out + j + 4) = ob;
+                        *reinterpret_cast<float4 *>(out + off) = oa;
+                        *reinterpret_cast<float4 *>(out + off + 4) = ob;
                     } else {
                         const float o[8] = {oa.x, oa.y, oa.z, oa.w, ob.x, ob.y, ob.z, ob.w};
                         for (int e = 0; e < 8; ++e)
-                            if (j + e < P.d) out[j + e] = kEF ? xs[j + e] - o[e] : o[e];
+                            if (off + e < left) out[off + e] = kEF ? xs[off + e] - o[e] : o[e];
                     }
                 }
             }
