@@ -1431,6 +1431,15 @@ static int launch_block(const thc_ctx *ctx, const void *kern, PipeMode mode, siz
     uint32_t resident = 0;
     { const int rc = resident_units(ctx, mode, kern, shape, e, &resident); if (rc != THC_OK) return rc; }
     cfg.gridDim = dim3((P.tasks < resident ? P.tasks : resident) << e);
+    // Tasks claimed from a counter instead of dealt out in a fixed stride: the CTAs of an SM do not progress evenly,
+    // and with fixed shares the mean CTA of a compress ended after four fifths of the time.  us, fixed / claimed, 4 x 2^25
+    // coordinates, 4 bits: compress in 2^12 blocks 222.0 / 202.4, 2^13 of bf16 236.8 / 211.6, 2^14 219.8 / 205.8, 2^15
+    // 327.0 / 308.5, error feedback 2^12 256.8 / 254.2 (2 x 2^28: 1006 / 976, decompress 342 / 333).  With few tasks to a
+    // CTA fixed shares put the last ones on different SMs: 3.7 to 5 tasks a CTA, compress with tiles of 2^13 44.8 / 43.6
+    // still, error feedback 53.3 / 54.9, with tiles of 2^14 30.5 / 32.4; decompress is level up to 7.
+    const bool quantises = mode == kCompressF32 || mode == kCompressBF16;
+    const uint32_t fixed = quantises && tile_log2 == 13u ? 2u : 8u;
+    P.head = P.tasks > (uint64_t)fixed * resident ? &reinterpret_cast<PipeCounters *>(ctx->dev->counters)->head : nullptr;
     void *args[] = {&maps, &P, const_cast<PtrArrayP *>(&in), const_cast<MutPtrArrayP *>(&out), const_cast<MutPtrArrayP *>(&rot),
                     const_cast<PhiloxKeys *>(&ctx->keys)};
     THC_CUDA(cudaLaunchKernelExC(&cfg, kern, args));

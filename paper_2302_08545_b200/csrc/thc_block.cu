@@ -14,14 +14,15 @@
 //            on the registers.  In a cluster these three stages are a round in place, and the
 //            last round takes the strides between the tiles: each thread gathers the same
 //            eight-coordinate unit from all CTAs and finishes 1 / C of the positions of every tile.
-// Stages above the block size are left out.  The CTAs walk over the tiles in a fixed stride; as
-// soon as the last round holds the tile in registers the next tile's TMA copy is started, so the
+// Stages above the block size are left out.  Few tiles per CTA are dealt out in a fixed stride,
+// more are claimed from a counter (see launch_block); as soon as the last round holds the tile in registers
+// the next tile's TMA copy is started, so the
 // epilogue hides it.
 //
 // What bounds it.  Timers in the kernel, 4 x 2^26 coordinates in blocks of 2^12, 4 bits: per tile a CTA spends
 // 2190 cycles on the load and the block constants, 2350 on round 1, 1650 on round 2 and its barrier, 1230 on
 // the last round and 5480 on the epilogue (Philox and the quantiser, bound by instruction issue), with four CTAs side by side
-// on an SM; and the CTAs, each with its fixed share of the tiles, run for 371 us of 465 on average.
+// on an SM; with fixed shares of the tiles the CTAs ran for 371 us of 465 on average, hence the counter.
 // Against five rounds through shared memory with a block barrier between them: blocks of 2^12 compress
 // 669 -> 441 us, decompress 156 -> 95 us, error feedback 1310 -> 509 us; 2^14 681 -> 435, 155 -> 115,
 // 1316 -> 539 us.  In a cluster the gather binds (a tile of every CTA crosses the SM-to-SM network: 8740
@@ -45,6 +46,12 @@ __device__ __forceinline__ float4 cluster_load(uint32_t addr)
 {
     float4 v;
     asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
+    return v;
+}
+__device__ __forceinline__ uint32_t cluster_load_u32(uint32_t addr)
+{
+    uint32_t v;
+    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
     return v;
 }
 
@@ -440,17 +447,27 @@ thc_block_kernel(const __grid_constant__ TmaMaps maps, const __grid_constant__ B
     float2 *blk_const = reinterpret_cast<float2 *>(smem + kBElems * 4 + 2 * kBSignWords * 4);   // likewise
     unsigned char *lut = smem + kBElems * 4 + 2 * kBSignWords * 4 + (size_t)P.const_slots * 16;
     __shared__ __align__(8) uint64_t s_full;
+    __shared__ uint32_t s_next;                        // the task after this one
 
     const int thread = threadIdx.x;
     const uint32_t k = P.k;
     const uint32_t rank = CLUSTER ? blockIdx.x & (C - 1u) : 0u;
-    const uint32_t stride = gridDim.x >> E;
     const uint64_t d_rows32 = P.d >> 5;
 
-    // tasks: tile (cluster: block) x worker, worker minor
+    // tasks: tile (cluster: block) x worker, worker minor.  Dealt out in a fixed stride, or, where P.head is
+    // given, claimed from it after the first two.
+    const uint32_t groups = gridDim.x >> E;
     uint32_t task = blockIdx.x >> E;
-    uint32_t unit = task / P.n_local, wl = task - unit * P.n_local;
-    const uint32_t unit_step = stride / P.n_local, wl_step = stride - unit_step * P.n_local;
+    uint32_t unit = task, wl = 0u;
+    auto split_task = [&]() {
+        if (kForward || kEF) {                         // (the others have one vector)
+            unit = task / P.n_local;
+            wl = task - unit * P.n_local;
+        } else {
+            unit = task;
+        }
+    };
+    split_task();
     auto tile_coord = [&](uint32_t u) -> uint64_t { return ((uint64_t)((u << E) + rank)) << kBLog2; };
     // Thread 0: whole tiles of a gradient come by TMA.
     auto by_tma = [&](uint32_t u) -> bool { return kForward && (tile_coord(u) >> 5) + kBSignWords <= d_rows32; };
@@ -520,6 +537,10 @@ thc_block_kernel(const __grid_constant__ TmaMaps maps, const __grid_constant__ B
         float4 *wtile = tile + 512 * warp;
         const uint32_t par = n & 1u;
         const uint64_t j0 = tile_coord(unit);
+        // the task after this one, handed round by the barrier in front of the last round
+        const bool claims = P.head != nullptr && task >= groups && tid == 0 && rank == 0u;
+        uint32_t claimed = 0u;
+        if (claims) claimed = groups * 2u + atomicAdd(P.head, 1u);
         // ---- constants of the tile's blocks
         float2 *bc = blk_const + par * P.const_slots;
         const uint32_t blk0 = (uint32_t)(j0 >> k);
@@ -616,6 +637,7 @@ thc_block_kernel(const __grid_constant__ TmaMaps maps, const __grid_constant__ B
         } else {
             mid_round5(wtile, lane);
         }
+        if (claims) s_next = claimed;
         __syncthreads();
 
         // ---- last round.  Thread (rl, u) owns the unit u of eight coordinates of rows rl + kBRowStep m: lanes 0-7 of
@@ -647,10 +669,11 @@ thc_block_kernel(const __grid_constant__ TmaMaps maps, const __grid_constant__ B
         const uint32_t cur_wl = wl;
         const uint64_t j_out = !CLUSTER ? j0 + 32u * rl + 8u * u
                                        : ((uint64_t)unit << k) + ((uint64_t)rank << (kBLog2 - E)) + 32u * rl + 8u * u;
-        task += stride;
-        unit += unit_step;
-        wl += wl_step;
-        if (wl >= P.n_local) { wl -= P.n_local; ++unit; }
+        // (the task after the next one is stored behind the barrier below; a cluster reads its first CTA's)
+        if (task < groups || P.head == nullptr) task += groups;
+        else if (!CLUSTER) task = s_next;
+        else task = cluster_load_u32(cluster_map((uint32_t)__cvta_generic_to_shared(&s_next), 0));
+        if (task < P.tasks) split_task();
         fence_proxy_async();                           // these reads before the next load's writes
         if (!CLUSTER) {
             __syncthreads();
@@ -756,7 +779,8 @@ thc_block_kernel(const __grid_constant__ TmaMaps maps, const __grid_constant__ B
             if (lane == 0) add_range(P.range_keys, P.nblocks, j_out >> k, kmin, kmax);
         }
     }
-    if (kRange && P.range_out != nullptr) {
+    // the last CTA clears the task counter for the next launch and finishes the ranges
+    if (P.head != nullptr || (kRange && P.range_out != nullptr)) {
         __shared__ uint32_t s_left;
         __threadfence();
         __syncthreads();
@@ -764,8 +788,11 @@ thc_block_kernel(const __grid_constant__ TmaMaps maps, const __grid_constant__ B
         __syncthreads();
         if (s_left == gridDim.x - 1) {
             __threadfence();
-            finish_ranges(P.range_keys, P.nblocks, P.range_out, P.dev, thread, kBThreads);
-            if (thread == 0) *P.exited = 0u;
+            if (kRange && P.range_out != nullptr) finish_ranges(P.range_keys, P.nblocks, P.range_out, P.dev, thread, kBThreads);
+            if (thread == 0) {
+                if (P.head != nullptr) *P.head = 0u;
+                *P.exited = 0u;
+            }
         }
     }
 }

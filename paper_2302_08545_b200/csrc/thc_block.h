@@ -29,7 +29,8 @@ struct BlockParams {
     uint32_t const_slots;      // blocks a tile can overlap
     uint32_t *range_keys;      // range mode: see add_range
     float   *range_out;        // ... finished by the last CTA (or null: by range_final_kernel)
-    uint32_t *exited;          // ... which this counter finds (zero between launches)
+    uint32_t *head;            // counter of claimed tasks, or null: fixed stride (see launch_block)
+    uint32_t *exited;          // CTAs that have ended (both are zero between launches)
     uint32_t agg_n;            // aggregate + decompress: workers whose table values are summed
     uint32_t agg_chunk;        // ... and how many of them before a byte could overflow
     uint32_t agg_acc_bits;     // ... and the width of the sums written on request (outp.p[1])

@@ -47,3 +47,9 @@ def test_edges_of_tiles_and_clusters(k, d, n, dtype, bits):
         z = O.unpack(r.packed[n - 1].cpu().numpy(), r.sz.d_pad, bits)
         e = O.error_feedback(x[n - 1], z, scl, c, 5)
         assert np.array_equal(ef[n - 1].cpu().numpy().view(np.uint32), e.view(np.uint32))
+
+
+@pytest.mark.parametrize("k,d", [(12, 9 * 592 * 8192 + 5), (14, 8 * 296 * 16_384 + 1), (15, 9 * 148 * 32_768 + 3)])
+def test_tasks_claimed_from_the_counter(k, d):
+    """So many tasks per CTA that every mode claims them; each call of the round needs the counter at zero again."""
+    test_edges_of_tiles_and_clusters(k, d, 1, "f32", 4)
