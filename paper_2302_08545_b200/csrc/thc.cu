@@ -706,8 +706,9 @@ struct thc_ctx {
     mutable MapEntry map_cache[kMapCache];
     mutable int map_cache_used, map_cache_next;
     mutable std::mutex map_mutex;
-    // Per mode, what resident_units answered for this context's block kernel (0: not asked yet).
-    mutable std::atomic<uint32_t> resident[kPipeModes];
+    // Per mode, what resident_units answered for this context's block kernel (0: not asked yet); then for clusters
+    // of one CTA per worker.
+    mutable std::atomic<uint32_t> resident[kPipeModes + kScalesMaxWorkers + 1];
 };
 
 static thread_local cudaError_t g_last_cuda = cudaSuccess;
@@ -941,6 +942,26 @@ static bool block_kernel_serves(const thc_ctx *ctx, uint64_t coords)
     return k <= 15u || (k == 16u && coords <= (1ull << 22)) || (k == 17u && coords <= (uint64_t)ctx->lone_clusters << 17);
 }
 
+// Scales and compress in one launch for blocks held in shared memory by one CTA: the gradients are read once, and the
+// clusters of one CTA per worker need no memory to exchange their sums in and no wait but the hardware's.  Up to
+// eight workers, the cluster size that every GPU can place; below 2^8 a thread's 64 coordinates span several blocks.
+// us, two calls / one launch, 4 bits, workers x coordinates:
+//                    2 x 3000    8 x 300,000  1 x 3 M      3 x 3 M      8 x 3 M      1 x 20 M     3 x 20 M     8 x 20 M
+//   fp32  2^11       8.9 / 8.1   13.6 / 10.8  13.7 / 10.4  26.2 / 22.8  62.1 / 53.0  53.4 / 40.4  134 / 115    340 / 295
+//         2^13       9.8 / 8.2   12.4 / 11.1  13.9 / 10.2  26.0 / 23.2  60.0 / 53.3  51.3 / 42.3  133 / 118    338 / 304
+//         2^14      11.1 / 9.7   15.5 / 12.7  15.7 / 11.8  26.2 / 23.5  61.3 / 62.7  52.0 / 43.5  137 / 129    348 / 344
+//   bf16  2^11       9.2 / 8.3   13.3 / 11.4  13.3 / 10.6  25.5 / 23.4  59.3 / 54.0  55.3 / 43.4  136 / 123    334 / 314
+//         2^13      10.5 / 8.6   12.2 / 11.5  13.8 / 10.6  25.7 / 23.8  55.8 / 55.8  47.7 / 45.1  122 / 126    307 / 319
+//         2^14      11.1 / 9.8   15.1 / 13.0  15.2 / 11.9  25.1 / 24.3  53.9 / 64.2  46.8 / 44.9  121 / 134    307 / 364
+//   (bf16 has half the bytes to save; with tiles of 2^14 there are two CTAs to an SM, and fewer to cover the wait for the slowest
+//   worker.)  Inputs of one wave of tiles always gain: the launch and its latency.
+static bool block_scales_serve(const thc_ctx *ctx, uint64_t coords, uint32_t n)
+{
+    const uint32_t k = ctx->cfg.log2_block;
+    if (k < kScalesMinLog2 || k > (uint32_t)kChunkLog2 || n > kScalesMaxWorkers || ctx->cfg.range_mode != THC_RANGE_NORM) return false;
+    return k <= 12u || coords <= (1ull << 22) || (ctx->cfg.in_dtype == THC_F32 && (k == 13u || n <= 6u));
+}
+
 // Schedule of the persistent pipeline for `wb_count` worker-blocks of 2^k coordinates:
 // how far pass B trails pass A (lag, in worker-blocks) and how many ring slots that needs.
 struct PipePlan { uint32_t grid, lag, ring; };
@@ -1029,6 +1050,7 @@ int thc_sizes(const thc_ctx *ctx, uint64_t d, uint32_t n_local, thc_sizes_t *s)
             s->fused_scales = 1;
         }
     }
+    if (block_scales_serve(ctx, s->d_pad * n_local, n_local)) s->fused_scales = 1;
     // scratch of prepare / the pipeline's ring, then the sums (thc_aggregate_decompress where it runs the two calls)
     s->workspace_bytes = round_up((prepare_ws > two_pass_ws ? prepare_ws : two_pass_ws) + 256, 256) +
                          round_up(s->sum_bytes, 256);
@@ -1347,30 +1369,32 @@ static bool use_block_kernel(const thc_ctx *ctx, uint64_t coords)
 // or two): that adds some 0.5 us to a context's first call.  Elsewhere no more clusters are launched than
 // there are (block_kernel_serves).
 constexpr size_t kSmemPerSm = 228u << 10, kSmemPerCta = 1024u + 256u;     // reserved and static
-static int resident_units(const thc_ctx *ctx, PipeMode mode, const void *kern, const cudaLaunchConfig_t &shape, uint32_t e, uint32_t *units)
+static int resident_units(const thc_ctx *ctx, uint32_t entry, const void *kern, const cudaLaunchConfig_t &shape, uint32_t cluster, uint32_t *units)
 {
     const uint32_t by_registers = shape.blockDim.x == 128u ? 4u : 2u;
-    *units = ((uint32_t)ctx->sm_count * by_registers) >> e;
-    if (shape.dynamicSmemBytes + kSmemPerCta <= kSmemPerSm / by_registers) return THC_OK;
-    *units = ctx->resident[mode].load(std::memory_order_relaxed);
+    *units = (uint32_t)ctx->sm_count * by_registers / cluster;
+    if (entry < (uint32_t)kPipeModes && shape.dynamicSmemBytes + kSmemPerCta <= kSmemPerSm / by_registers) return THC_OK;
+    *units = ctx->resident[entry].load(std::memory_order_relaxed);
     if (*units != 0u) return THC_OK;
     int n = 0;
-    if (e == 0u) {
+    if (cluster == 1u) {
         THC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, (int)shape.blockDim.x, shape.dynamicSmemBytes));
         n *= ctx->sm_count;
     } else {
         THC_CUDA(cudaOccupancyMaxActiveClusters(&n, kern, &shape));
     }
     *units = n > 0 ? (uint32_t)n : 1u;
-    ctx->resident[mode].store(*units, std::memory_order_relaxed);
+    ctx->resident[entry].store(*units, std::memory_order_relaxed);
     return THC_OK;
 }
 
-// lut_bytes: table space in shared memory; keys: exact-range mode; agg_n: aggregate + decompress.
+// lut_bytes: table space in shared memory; keys: exact-range mode; agg_n: aggregate + decompress; scales_out: scales and
+// compress in one launch.
 static int launch_block(const thc_ctx *ctx, const void *kern, PipeMode mode, size_t lut_bytes, const thc_sizes_t &sz,
                         uint64_t d, uint32_t n_local, uint32_t worker_base, uint32_t round, uint32_t divisor,
                         const float *scales, const PtrArrayP &in, const MutPtrArrayP &out, const MutPtrArrayP &rot,
-                        cudaStream_t st, uint32_t *keys = nullptr, uint32_t agg_n = 0, float *range_out = nullptr)
+                        cudaStream_t st, uint32_t *keys = nullptr, uint32_t agg_n = 0, float *range_out = nullptr,
+                        float *scales_out = nullptr)
 {
     const uint32_t k = ctx->cfg.log2_block;
     BlockParams P;
@@ -1383,7 +1407,10 @@ static int launch_block(const thc_ctx *ctx, const void *kern, PipeMode mode, siz
     P.d_pad = sz.d_pad;
     P.scales = scales;
     P.dev = ctx->dev;
-    P.tasks = (uint32_t)(units * n_local);
+    P.tasks = (uint32_t)(scales_out != nullptr ? units : units * n_local);
+    P.scales_out = scales_out;
+    P.t_p = ctx->cfg.t_p;
+    P.sqrt_block = sqrt((double)(1ull << k));
     P.n_local = n_local;
     P.k = k;
     P.granularity = ctx->cfg.granularity;
@@ -1406,8 +1433,8 @@ static int launch_block(const thc_ctx *ctx, const void *kern, PipeMode mode, siz
     if ((d >> 5) >= 256) {
         for (uint32_t i = 0; i < n_local; ++i) {
             int rc = THC_OK;
-            if (mode == kCompressBF16) rc = cached_map(ctx, &maps.in[i], in.p[i], 32u, d >> 5, 64u, 64u, 32u, true);
-            else if (mode == kCompressF32 || mode == kRangeF32) rc = cached_map(ctx, &maps.in[i], in.p[i], 32u, d >> 5, 128u, 256u);
+            if (mode == kCompressBF16 || mode == kCompressBF16Fused) rc = cached_map(ctx, &maps.in[i], in.p[i], 32u, d >> 5, 64u, 64u, 32u, true);
+            else if (mode == kCompressF32 || mode == kCompressF32Fused || mode == kRangeF32) rc = cached_map(ctx, &maps.in[i], in.p[i], 32u, d >> 5, 128u, 256u);
             if (rc != THC_OK) return rc;
         }
     }
@@ -1415,29 +1442,31 @@ static int launch_block(const thc_ctx *ctx, const void *kern, PipeMode mode, siz
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = 1u << e;
+    const uint32_t cluster = scales_out != nullptr ? n_local : 1u << e;
+    attr[1].val.clusterDim.x = cluster;
     attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof cfg);
-    cfg.gridDim = dim3((unsigned)ctx->sm_count << 3);
+    cfg.gridDim = dim3((unsigned)ctx->sm_count * 8u * cluster);
     cfg.blockDim = dim3((unsigned)(tile / 64));
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cfg.attrs = attr;
-    cfg.numAttrs = e != 0u ? 2 : 1;
+    cfg.numAttrs = cluster != 1u ? 2 : 1;
     cudaLaunchConfig_t shape = cfg;
     shape.attrs = attr + 1;
     shape.numAttrs = 1;
     uint32_t resident = 0;
-    { const int rc = resident_units(ctx, mode, kern, shape, e, &resident); if (rc != THC_OK) return rc; }
-    cfg.gridDim = dim3((P.tasks < resident ? P.tasks : resident) << e);
+    { const int rc = resident_units(ctx, scales_out != nullptr ? kPipeModes + cluster : (uint32_t)mode,
+                                                 kern, shape, cluster, &resident); if (rc != THC_OK) return rc; }
+    cfg.gridDim = dim3((P.tasks < resident ? P.tasks : resident) * cluster);
     // Tasks claimed from a counter instead of dealt out in a fixed stride: the CTAs of an SM do not progress evenly,
     // and with fixed shares the mean CTA of a compress ended after four fifths of the time.  us, fixed / claimed, 4 x 2^25
     // coordinates, 4 bits: compress in 2^12 blocks 222.0 / 202.4, 2^13 of bf16 236.8 / 211.6, 2^14 219.8 / 205.8, 2^15
     // 327.0 / 308.5, error feedback 2^12 256.8 / 254.2 (2 x 2^28: 1006 / 976, decompress 342 / 333).  With few tasks to a
     // CTA fixed shares put the last ones on different SMs: 3.7 to 5 tasks a CTA, compress with tiles of 2^13 44.8 / 43.6
     // still, error feedback 53.3 / 54.9, with tiles of 2^14 30.5 / 32.4; decompress is level up to 7.
-    const bool quantises = mode == kCompressF32 || mode == kCompressBF16;
+    const bool quantises = mode == kCompressF32 || mode == kCompressBF16 || scales_out != nullptr;
     const uint32_t fixed = quantises && tile_log2 == 13u ? 2u : 8u;
     P.head = P.tasks > (uint64_t)fixed * resident ? &reinterpret_cast<PipeCounters *>(ctx->dev->counters)->head : nullptr;
     void *args[] = {&maps, &P, const_cast<PtrArrayP *>(&in), const_cast<MutPtrArrayP *>(&out), const_cast<MutPtrArrayP *>(&rot),
@@ -1564,7 +1593,8 @@ int thc_prepare_compress(thc_ctx *ctx, const void *const *grads, uint32_t n, uin
     thc_sizes_t sz;
     if ((rc = thc_sizes(ctx, d, n, &sz)) != THC_OK) return rc;
     PipePlan pf;
-    if (!plan_pipeline_fused(ctx, sz.nblocks, n, &pf)) {
+    const bool in_block = block_scales_serve(ctx, sz.d_pad * n, n);
+    if (!in_block && !plan_pipeline_fused(ctx, sz.nblocks, n, &pf)) {
         rc = thc_prepare(ctx, grads, n, d, scales, workspace, workspace_bytes, stream);
         if (rc != THC_OK) return rc;
         return thc_compress(ctx, grads, n, worker_base, d, round, scales, packed, rotated, workspace,
@@ -1587,6 +1617,11 @@ int thc_prepare_compress(thc_ctx *ctx, const void *const *grads, uint32_t n, uin
             if (!aligned16(rotated[i])) return THC_EINVAL;
             prot.p[i] = rotated[i];
         }
+    }
+    if (in_block) {
+        const PipeMode mode = ctx->cfg.in_dtype == THC_BF16 ? kCompressBF16Fused : kCompressF32Fused;
+        return launch_block(ctx, block_kernel(mode, ctx->cfg.bits, ctx->identity, ctx->cfg.log2_block), mode, quant_lut_bytes(ctx), sz, d, n,
+                            worker_base, round, 1, scales, pin, pout, prot, static_cast<cudaStream_t>(stream), nullptr, 0, nullptr, scales);
     }
     pipe_kernel_t kern = ctx->cfg.log2_block == 20 ? pick_pipe_kernel_kb<kCompressF32Fused, 7>(ctx->cfg.bits, ctx->identity)
                                                     : pick_pipe_kernel_kb<kCompressF32Fused, 0>(ctx->cfg.bits, ctx->identity);

@@ -48,6 +48,12 @@ __device__ __forceinline__ float4 cluster_load(uint32_t addr)
     asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
     return v;
 }
+__device__ __forceinline__ double cluster_load_f64(uint32_t addr)
+{
+    double v;
+    asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(addr) : "memory");
+    return v;
+}
 __device__ __forceinline__ uint32_t cluster_load_u32(uint32_t addr)
 {
     uint32_t v;
@@ -122,8 +128,10 @@ __device__ __forceinline__ void low_stages_store(float4 *wtile, const LowRows &l
 
 // ... of a gradient.  fp32 rows lie in the tile; the bf16 rows of a warp (64 rows of 64 bytes in the
 // 64-byte swizzle) in the upper half of its 8 KB, and are widened exactly.
-template <bool BF16>
-__device__ __forceinline__ void low_round_gradient(float4 *wtile, const uint32_t *wsw, int lane, uint32_t k)
+// With SQ the sum of squares of the lane's 64 inputs (fp64, four interleaved partial sums combined
+// in a fixed order) is returned.
+template <bool BF16, bool SQ>
+__device__ __forceinline__ double low_round_gradient(float4 *wtile, const uint32_t *wsw, int lane, uint32_t k)
 {
     const LowRows lr = low_rows(lane);
     float4 v[16];
@@ -149,10 +157,23 @@ __device__ __forceinline__ void low_round_gradient(float4 *wtile, const uint32_t
 #pragma unroll
         for (int m = 0; m < 16; ++m) v[m] = *low_chunk(wtile, lr, m);
     }
+    double sq = 0.0;
+    if (SQ) {
+        double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
+#pragma unroll
+        for (int m = 0; m < 16; ++m) {
+            a0 = fma((double)v[m].x, (double)v[m].x, a0);
+            a1 = fma((double)v[m].y, (double)v[m].y, a1);
+            a2 = fma((double)v[m].z, (double)v[m].z, a2);
+            a3 = fma((double)v[m].w, (double)v[m].w, a3);
+        }
+        sq = (a0 + a1) + (a2 + a3);
+    }
     const uint32_t w0 = wsw[lr.first], w1 = wsw[lr.first ^ 1];
 #pragma unroll
     for (int m = 0; m < 8; ++m) { v[m] = flip4(v[m], w0 >> (m * 4)); v[8 + m] = flip4(v[8 + m], w1 >> (m * 4)); }
     low_stages_store(wtile, lr, v, k);
+    return sq;
 }
 
 // (step, base) of the estimate line for chunk m of a row: rows of 32 coordinates hold several blocks
@@ -416,6 +437,60 @@ __device__ __forceinline__ void unit_gather(uint32_t own, uint32_t row, uint32_t
     }
 }
 
+// ------------------------------------------------------------------------ scales
+// Scales and compress in one launch: the sums of squares come from round 1's registers, go to shared memory and are
+// exchanged between the workers' CTAs while round 2 runs; the scales are ready before the epilogue, which alone needs
+// them.  What it adds to a compress (4 x 2^25 coordinates in 2^12 blocks: 202 -> 246 us) is the conversion to fp64, which runs at an
+// eighth of the issue rate and fills its own unit in round 1, three dispatch slots per coordinate, and the
+// wait for the slowest of the cluster; the launch it replaces took 83 us.
+// Scales of the tile's blocks (Section 5.3: M = t_p max_i ||x_i|| / sqrt(B)) from the sums of squares in the shared memory of
+// the n_local CTAs of the cluster, and the quantiser's constants into `bc`.  sq: address of the own sums, one per
+// block or, from 2^11 on, per 2^11 coordinates; they are added in ascending order.  Every CTA does it for itself;
+// `store`: this one writes the scales.
+template <int TILE_LOG2>
+__device__ __forceinline__ void block_scales(const BlockParams &P, uint32_t sq, uint32_t blk0, float2 *bc, bool store, int tid)
+{
+    const uint32_t k = P.k, blocks = 1u << (TILE_LOG2 - k);
+    double s = 0.0;                                    // largest sum of squares; a NaN sticks
+    uint32_t b;
+    bool live;
+    if (k <= 10u) {
+        b = (uint32_t)tid;                             // a thread per block
+        live = b < blocks;
+        if (live) {
+            for (uint32_t i = 0; i < P.n_local; ++i) {
+                const double v = cluster_load_f64(cluster_map(sq + 8u * b, i));
+                if (v > s || v != v) s = v;
+            }
+        }
+    } else {
+        b = (uint32_t)tid >> 5;                        // a warp per block, a lane per worker
+        live = b < blocks;
+        const uint32_t lane = (uint32_t)tid & 31u, parts = 1u << (k - 11u);
+        if (live && lane < P.n_local) {
+            const uint32_t a = cluster_map(sq + 8u * parts * b, lane);
+#pragma unroll 4
+            for (uint32_t c = 0; c < parts; ++c) s += cluster_load_f64(a + 8u * c);
+        }
+#pragma unroll
+        for (int off = 1; off < (int)kScalesMaxWorkers; off <<= 1) {
+            const double v = __shfl_xor_sync(0xFFFFFFFFu, s, off);
+            if (v > s || v != v) s = v;
+        }
+        live = live && lane == 0u;
+    }
+    if (!live) return;
+    float M = (float)(P.t_p * sqrt(s) / P.sqrt_block);
+    uint32_t flags = 0;
+    if (!isfinite(M)) { M = 0.0f; flags |= THC_STATUS_NONFINITE; }
+    if (M == 0.0f) flags |= THC_STATUS_ZERO_BLOCK;
+    bc[b] = compress_constants(BlockRange{-M, M});
+    if (store && blk0 + b < P.nblocks) {
+        P.scales_out[blk0 + b] = M;
+        if (flags) atomicOr(&P.dev->status, flags);
+    }
+}
+
 // ------------------------------------------------------------------------ the kernel
 // KIND: see block_kind.
 template <int MODE, int BITS, bool IDENTITY, int KIND>
@@ -433,8 +508,12 @@ thc_block_kernel(const __grid_constant__ TmaMaps maps, const __grid_constant__ B
     constexpr int kBRowStep = kBSignWords / 8;         // rows between the registers of the last round
     constexpr bool kEF = MODE == kErrorFeedback;
     constexpr bool kRange = MODE == kRangeF32;
-    constexpr bool kF32In = MODE == kCompressF32 || kRange;
-    constexpr bool kForward = kF32In || MODE == kCompressBF16;
+    // Scales in the same launch: the n_local CTAs of a cluster hold the same tile of all workers and exchange
+    // its sums of squares.
+    constexpr bool kScales = MODE == kCompressF32Fused || MODE == kCompressBF16Fused;
+    constexpr bool kBF16In = MODE == kCompressBF16 || MODE == kCompressBF16Fused;
+    constexpr bool kF32In = MODE == kCompressF32 || MODE == kCompressF32Fused || kRange;
+    constexpr bool kForward = kF32In || kBF16In;
     constexpr bool kQuant = kForward && !kRange;
     constexpr int kFRep = BITS <= 4 ? 32 : 8;
     extern __shared__ __align__(1024) unsigned char block_smem_raw[];
@@ -447,20 +526,22 @@ thc_block_kernel(const __grid_constant__ TmaMaps maps, const __grid_constant__ B
     float2 *blk_const = reinterpret_cast<float2 *>(smem + kBElems * 4 + 2 * kBSignWords * 4);   // likewise
     unsigned char *lut = smem + kBElems * 4 + 2 * kBSignWords * 4 + (size_t)P.const_slots * 16;
     __shared__ __align__(8) uint64_t s_full;
-    __shared__ uint32_t s_next;                        // the task after this one
+    __shared__ uint32_t s_next[2];                     // the task after this one
+    __shared__ double s_sq[2][!kScales ? 1 : KIND == 0 ? kBElems >> kScalesMinLog2 : kBElems >> 11];    // sums of squares, by task parity
 
     const int thread = threadIdx.x;
     const uint32_t k = P.k;
-    const uint32_t rank = CLUSTER ? blockIdx.x & (C - 1u) : 0u;
+    const uint32_t group = kScales ? P.n_local : C;    // CTAs that take a task together
+    const uint32_t rank = kScales ? blockIdx.x % group : CLUSTER ? blockIdx.x & (C - 1u) : 0u;
     const uint64_t d_rows32 = P.d >> 5;
 
     // tasks: tile (cluster: block) x worker, worker minor.  Dealt out in a fixed stride, or, where P.head is
     // given, claimed from it after the first two.
-    const uint32_t groups = gridDim.x >> E;
-    uint32_t task = blockIdx.x >> E;
-    uint32_t unit = task, wl = 0u;
+    const uint32_t groups = kScales ? gridDim.x / group : gridDim.x >> E;
+    uint32_t task = kScales ? blockIdx.x / group : blockIdx.x >> E;
+    uint32_t unit = task, wl = kScales ? rank : 0u;
     auto split_task = [&]() {
-        if (kForward || kEF) {                         // (the others have one vector)
+        if (!kScales && (kForward || kEF)) {            // (the others have one vector)
             unit = task / P.n_local;
             wl = task - unit * P.n_local;
         } else {
@@ -468,7 +549,7 @@ thc_block_kernel(const __grid_constant__ TmaMaps maps, const __grid_constant__ B
         }
     };
     split_task();
-    auto tile_coord = [&](uint32_t u) -> uint64_t { return ((uint64_t)((u << E) + rank)) << kBLog2; };
+    auto tile_coord = [&](uint32_t u) -> uint64_t { return ((uint64_t)((u << E) + (CLUSTER ? rank : 0u))) << kBLog2; };
     // Thread 0: whole tiles of a gradient come by TMA.
     auto by_tma = [&](uint32_t u) -> bool { return kForward && (tile_coord(u) >> 5) + kBSignWords <= d_rows32; };
     auto start_load = [&](uint32_t u, uint32_t w) {
@@ -544,7 +625,7 @@ thc_block_kernel(const __grid_constant__ TmaMaps maps, const __grid_constant__ B
         // ---- constants of the tile's blocks
         float2 *bc = blk_const + par * P.const_slots;
         const uint32_t blk0 = (uint32_t)(j0 >> k);
-        if (!kRange) {
+        if (!kRange && !kScales) {
             for (uint32_t b = tid; b < P.const_slots; b += kBThreads) {
                 float2 c = make_float2(0.f, 0.f);
                 if (blk0 + b < P.nblocks) {
@@ -607,8 +688,18 @@ thc_block_kernel(const __grid_constant__ TmaMaps maps, const __grid_constant__ B
                 }
                 __syncwarp();
             }
-            if (MODE == kCompressBF16 && tma) low_round_gradient<true>(wtile, sw + 64 * warp, lane, k);
-            else low_round_gradient<false>(wtile, sw + 64 * warp, lane, k);
+            double sq;
+            if (kBF16In && tma) sq = low_round_gradient<true, kScales>(wtile, sw + 64 * warp, lane, k);
+            else sq = low_round_gradient<false, kScales>(wtile, sw + 64 * warp, lane, k);
+            if constexpr (kScales) {
+                // a lane has 64 consecutive coordinates: 2^(k-6) lanes to a block, at most the warp
+                const uint32_t parts_log2 = min(k, 11u);
+                for (uint32_t b = 0; b + 6u < parts_log2; ++b) sq += __shfl_xor_sync(0xFFFFFFFFu, sq, 1 << b);
+                if ((lane & ((1 << (parts_log2 - 6u)) - 1)) == 0) s_sq[par][(2048u * warp + 64u * lane) >> parts_log2] = sq;
+                if (claims) s_next[par] = claimed;
+                __syncwarp();
+                cluster_arrive();
+            }
         } else {
             const uint64_t jw = j0 + 2048u * warp;
             const int coords = jw + 2048u <= P.d_pad ? 2048 : jw < P.d_pad ? (int)(P.d_pad - jw) : 0;
@@ -637,7 +728,7 @@ thc_block_kernel(const __grid_constant__ TmaMaps maps, const __grid_constant__ B
         } else {
             mid_round5(wtile, lane);
         }
-        if (claims) s_next = claimed;
+        if (!kScales && claims) s_next[0] = claimed;
         __syncthreads();
 
         // ---- last round.  Thread (rl, u) owns the unit u of eight coordinates of rows rl + kBRowStep m: lanes 0-7 of
@@ -665,14 +756,22 @@ thc_block_kernel(const __grid_constant__ TmaMaps maps, const __grid_constant__ B
             const uint32_t row = (rank << (kBLog2 - 5 - E)) + (uint32_t)rl, ca = (uint32_t)((2 * u) ^ x) << 4, cb = (uint32_t)((2 * u + 1) ^ x) << 4;
             unit_gather<E, kBRowStep>(own, row, ca, cb, a, b);
         }
+        uint32_t next_task = 0u;
+        if constexpr (kScales) {
+            // every worker's sums of squares of this tile are in place
+            cluster_wait();
+            if (P.head != nullptr && task >= groups) next_task = cluster_load_u32(cluster_map((uint32_t)__cvta_generic_to_shared(&s_next[par]), 0));
+            block_scales<kBLog2>(P, (uint32_t)__cvta_generic_to_shared(s_sq[par]), blk0, bc, wl == 0u, tid);
+        }
         // ---- the tile is in registers: start the next task's load
         const uint32_t cur_wl = wl;
         const uint64_t j_out = !CLUSTER ? j0 + 32u * rl + 8u * u
                                        : ((uint64_t)unit << k) + ((uint64_t)rank << (kBLog2 - E)) + 32u * rl + 8u * u;
         // (the task after the next one is stored behind the barrier below; a cluster reads its first CTA's)
         if (task < groups || P.head == nullptr) task += groups;
-        else if (!CLUSTER) task = s_next;
-        else task = cluster_load_u32(cluster_map((uint32_t)__cvta_generic_to_shared(&s_next), 0));
+        else if (kScales) task = next_task;
+        else if (!CLUSTER) task = s_next[0];
+        else task = cluster_load_u32(cluster_map((uint32_t)__cvta_generic_to_shared(&s_next[0]), 0));
         if (task < P.tasks) split_task();
         fence_proxy_async();                           // these reads before the next load's writes
         if (!CLUSTER) {
@@ -779,6 +878,7 @@ thc_block_kernel(const __grid_constant__ TmaMaps maps, const __grid_constant__ B
             if (lane == 0) add_range(P.range_keys, P.nblocks, j_out >> k, kmin, kmax);
         }
     }
+    if (kScales) { cluster_arrive(); cluster_wait(); }  // (the others read this CTA's sums)
     // the last CTA clears the task counter for the next launch and finishes the ranges
     if (P.head != nullptr || (kRange && P.range_out != nullptr)) {
         __shared__ uint32_t s_left;
@@ -801,7 +901,10 @@ template <int MODE, int KIND>
 static const void *pick(uint32_t bits, bool identity)
 {
 #define THC_BLK(B, I) reinterpret_cast<const void *>(thc_block_kernel<MODE, B, I, KIND>)
-    if constexpr (MODE == kErrorFeedback) {
+    constexpr bool fused = MODE == kCompressF32Fused || MODE == kCompressBF16Fused;
+    if constexpr (fused && KIND > 1) {
+        return nullptr;
+    } else if constexpr (MODE == kErrorFeedback) {
         switch (bits) {
         case 1: return THC_BLK(1, true);
         case 2: return THC_BLK(2, true);
@@ -809,7 +912,7 @@ static const void *pick(uint32_t bits, bool identity)
         case 4: return THC_BLK(4, true);
         default: return THC_BLK(8, true);
         }
-    } else if constexpr (MODE == kCompressF32 || MODE == kCompressBF16) {
+    } else if constexpr (MODE == kCompressF32 || MODE == kCompressBF16 || fused) {
         switch (bits) {
         case 1: return identity ? THC_BLK(1, true) : THC_BLK(1, false);
         case 2: return identity ? THC_BLK(2, true) : THC_BLK(2, false);
@@ -829,6 +932,8 @@ static const void *pick_mode(PipeMode mode, uint32_t bits, bool identity)
     switch (mode) {
     case kCompressF32: return pick<kCompressF32, KIND>(bits, identity);
     case kCompressBF16: return pick<kCompressBF16, KIND>(bits, identity);
+    case kCompressF32Fused: return pick<kCompressF32Fused, KIND>(bits, identity);
+    case kCompressBF16Fused: return pick<kCompressBF16Fused, KIND>(bits, identity);
     case kDecompress8: return pick<kDecompress8, KIND>(bits, identity);
     case kDecompress16: return pick<kDecompress16, KIND>(bits, identity);
     case kDecompress32: return pick<kDecompress32, KIND>(bits, identity);

@@ -11,6 +11,10 @@ __host__ __device__ constexpr int block_kind(uint32_t k) { return k <= 13u ? 0 :
 __host__ __device__ constexpr int block_tile_log2(int kind) { return kind == 0 || kind == 3 ? 13 : 14; }
 __host__ __device__ constexpr uint32_t block_cluster_log2(int kind) { return kind == 2 ? 1u : kind >= 3 ? 3u : 0u; }
 
+// Scales and compress in one launch (kinds 0 and 1): block sizes from 2^8 on, up to this many workers (a cluster of one
+// CTA per worker, of the size that every GPU can hold).
+constexpr uint32_t kScalesMinLog2 = 8, kScalesMaxWorkers = 8;
+
 struct BlockParams {
     uint64_t d;
     uint64_t d_pad;
@@ -31,6 +35,8 @@ struct BlockParams {
     float   *range_out;        // ... finished by the last CTA (or null: by range_final_kernel)
     uint32_t *head;            // counter of claimed tasks, or null: fixed stride (see launch_block)
     uint32_t *exited;          // CTAs that have ended (both are zero between launches)
+    float   *scales_out;       // scales + compress: = scales, written by the kernel; tasks are tiles of all workers
+    double   t_p, sqrt_block;
     uint32_t agg_n;            // aggregate + decompress: workers whose table values are summed
     uint32_t agg_chunk;        // ... and how many of them before a byte could overflow
     uint32_t agg_acc_bits;     // ... and the width of the sums written on request (outp.p[1])

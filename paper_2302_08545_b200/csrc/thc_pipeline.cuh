@@ -71,6 +71,7 @@ enum PipeMode { kCompressF32, kCompressBF16, kDecompress8, kDecompress16, kDecom
                 kErrorFeedback,        // e_i = x_i - RHT^-1(X_i) from worker i's own packed indices
                 kRangeF32,             // exact min / max of the rotated coordinates per RHT block
                 kAggDecompress,        // decompress straight from the workers' packed indices (PS line + estimate line)
+                kCompressBF16Fused,    // bf16 compress that also computes the block scales (thc_block.cu only)
                 kPipeModes };
 
 // Layout inside DeviceBlock::counters.  Every CTA hits `head` and `abort` for every task and

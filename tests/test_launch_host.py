@@ -168,3 +168,35 @@ for blocks in (1, last, last + 1):
             c.decompress(buf[0], 1, d, 0, buf[1], buf[2], ws, stream=0)
             assert kernels() == want, blocks
 """)
+
+
+@pytest.mark.parametrize("k,n,dtype,small,large", [
+    (7, 2, 0, 2, 2), (8, 1, 0, 1, 1), (8, 8, 1, 1, 1), (8, 9, 0, 2, 2), (12, 5, 1, 1, 1), (13, 3, 1, 1, 2), (13, 8, 0, 1, 1),
+    (14, 6, 0, 1, 1), (14, 7, 0, 1, 2), (14, 1, 1, 1, 2), (14, 9, 1, 2, 2), (15, 2, 0, 2, 2),
+])
+def test_scales_and_compress_of_blocks_in_shared_memory(child, k, n, dtype, small, large):
+    """One launch, in clusters of one CTA per worker, exactly where thc_sizes says so; what the two calls refuse is
+    refused there too, before anything is launched."""
+    child(f"""
+k, n, dtype, small, large = {k}, {n}, {dtype}, {small}, {large}
+c = context(k, in_dtype=dtype)
+x = buf[:n]
+for d, launches in ((5, small), (1 << 15, small), (20_000_003, large)):
+    c.prepare_compress(x, d, 0, buf[0], x, ws, stream=0)
+    rows = [r for r in log() if r[0] == "launch"]
+    assert len(rows) == launches and c.sizes(d, n).fused_scales == (launches == 1)
+    if launches == 1:
+        assert "block_kernel" in rows[0][1] and rows[0][5] == n and rows[0][2] % n == 0
+class Short(Space):
+    nbytes = c.sizes(5, n).workspace_bytes - 1
+m = context(k, range_mode=1)
+for ctx, grads, scales, packed, space in [(c, [8] * n, buf[0], x, ws), (c, x, buf[0], [0] * n, ws), (c, x, 0, x, ws), (c, x, buf[0], x, Short()),
+                                          (m, x, buf[0], x, ws)]:
+    try:
+        ctx.prepare_compress(grads, 5, 0, scales, packed, space, stream=0)
+        assert False
+    except thc.ThcError:
+        pass
+    assert small == 2 or log() == []
+    log()
+""")
