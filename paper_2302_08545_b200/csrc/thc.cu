@@ -1671,6 +1671,23 @@ int thc_decompress(thc_ctx *ctx, const void *sum, uint32_t divisor, uint64_t d, 
 // packed indices all sit in this GPU's memory (Algorithm 2: the PS line Y = sum_i T[Z_i] feeding
 // the worker's estimate line and the inverse RHT): pass A of the inverse transform adds up the
 // table values itself, so the sums need not travel through HBM; they are written only on request.
+// Whether the two calls are faster where the sums are wanted too: a thread's first round waits for the indices of all
+// workers, some at a time, and the pipeline and the tiles of 2^14 have fewer threads to cover that.  us, two calls / one:
+//                     4 workers    8            10           16           24           32
+//   2^ 8  3000        6.7 / 4.9    6.7 / 5.6    6.8 / 6.4    7.3 / 6.9    8.8 / 8.3    10.2 / 9.8
+//   2^12  2^22       13.3 / 10.5  13.7 / 11.4  18.3 / 14.1  19.2 / 15.9  24.1 / 20.2   29.0 / 24.7
+//   2^14  2^24       45.9 / 41.1  48.0 / 48.5  66.3 / 57.2  72.0 / 67.9  86.4 / 90.8  100.5 / 112.9
+//   2^16  2^20       12.9 / 12.4  13.5 / 13.2  14.8 / 14.5  16.1 / 15.2  18.0 / 17.2   19.8 / 19.2   (clusters)
+//   2^17  2^20       13.7 / 13.8  14.3 / 14.8  15.8 / 16.3  17.0 / 17.5  18.9 / 19.9   20.3 / 22.2   (clusters)
+//   2^20  25.6 M     86.6 / 76.1  90.1 / 87.1   115 / 100    125 / 129    146 / 165     168 / 202
+//   2^22  2^26        271 / 236    283 / 255    343 / 284    362 / 352    429 / 442     477 / 528
+static bool two_call_tail(const thc_ctx *ctx, uint64_t d_pad, uint32_t n)
+{
+    const uint32_t k = ctx->cfg.log2_block;
+    if (use_block_kernel(ctx, d_pad)) return k == 17u || ((k == 14u || k == 15u) && n > 16u);
+    return n > 12u;
+}
+
 int thc_aggregate_decompress(thc_ctx *ctx, const void *const *packed, uint32_t n, uint64_t d, uint32_t round,
                              const float *scales, float *outp, void *sum_or_null, void *workspace,
                              uint64_t workspace_bytes, void *stream)
@@ -1684,7 +1701,8 @@ int thc_aggregate_decompress(thc_ctx *ctx, const void *const *packed, uint32_t n
     if (outp == nullptr || scales == nullptr || !aligned16(outp)) return THC_EINVAL;
     if (sum_or_null != nullptr && !aligned16(sum_or_null)) return THC_EINVAL;
     const uint32_t k = ctx->cfg.log2_block;
-    if (ctx->cfg.bits != 4 || ctx->cfg.granularity >= 128 || sz.d_pad % 32 != 0) {
+    if (ctx->cfg.bits != 4 || ctx->cfg.granularity >= 128 || sz.d_pad % 32 != 0 ||
+        (sum_or_null != nullptr && two_call_tail(ctx, sz.d_pad, n))) {
         // index widths without the byte-lane look-up (there the one launch is
         // slower than the two): the two calls; the sums go to the caller's buffer or to the workspace
         // (without a buffer the sums take the end of the workspace; thc_decompress checks that what

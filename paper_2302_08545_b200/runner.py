@@ -88,5 +88,8 @@ class Round:
             if with_prepare:
                 self.prepare(stream)
             self.compress(rnd, stream)
-        self.aggregate(stream)
-        self.decompress(rnd, stream)
+        if fused:
+            self.aggregate_decompress(rnd, want_sums=True, stream=stream)
+        else:
+            self.aggregate(stream)
+            self.decompress(rnd, stream)

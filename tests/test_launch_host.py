@@ -200,3 +200,17 @@ for ctx, grads, scales, packed, space in [(c, [8] * n, buf[0], x, ws), (c, x, bu
     assert small == 2 or log() == []
     log()
 """)
+
+
+@pytest.mark.parametrize("k,d,n,launches", [
+    (12, 1 << 24, 32, 1), (14, 1 << 20, 16, 1), (14, 1 << 20, 17, 2), (15, 1 << 20, 17, 2), (16, 1 << 20, 32, 1), (16, 1 << 24, 13, 2),
+    (17, 1 << 20, 2, 2), (17, 1 << 23, 12, 1), (20, 1 << 22, 12, 1), (20, 1 << 22, 13, 2),
+])
+def test_one_call_tail_is_two_launches_where_these_are_faster(child, k, d, n, launches):
+    """With the sums wanted; without them it is one launch for 4-bit indices."""
+    child(f"""
+c = context({k}, workers=32)
+for total, want in ((buf[2], {launches}), (None, 1)):
+    c.aggregate_decompress(buf[:{n}], {d}, 0, buf[0], buf[1], ws, total=total, stream=0)
+    assert len(kernels()) == want
+""")
