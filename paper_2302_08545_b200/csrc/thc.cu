@@ -1942,6 +1942,9 @@ int thc_debug_skip_tasks(thc_ctx *ctx, uint32_t count)
     int rc = check_launch_ctx(ctx);
     if (rc != THC_OK) return rc;
     THC_CUDA(cudaDeviceSynchronize());
+    // (blocks that have no pipeline claim their tiles from the same counter: a start that no pipeline launch takes
+    // up and clears would make the next such launch leave tiles out)
+    if (ctx->cfg.log2_block <= (uint32_t)kChunkLog2) return THC_OK;
     PipeCounters *pc = reinterpret_cast<PipeCounters *>(ctx->dev->counters);
     THC_CUDA(cudaMemcpy(&pc->head, &count, sizeof count, cudaMemcpyHostToDevice));
     ctx->pipeline_next = true;

@@ -2,7 +2,8 @@
  * tests/test_launch_host.py: the host code of the library runs as with a GPU, no kernel is executed, and
  * launches and attribute calls are written to a log, one line each.
  *   attr <kernel> <bytes>                           cudaFuncSetAttribute
- *   launch <kernel> <grid.x> <threads> <bytes> <cluster>
+ *   launch <kernel> <grid.x> <threads> <bytes> <cluster> [<claims>]
+ * (claims, of the block kernels: 1 where the launch is given the counter that tasks are claimed from)
  */
 #include <driver_types.h>
 #include <stddef.h>
@@ -50,7 +51,18 @@ int cudaGetDeviceCount(int *n) { *n = 1; return 0; }
 int cudaGetDevice(int *d) { *d = 0; return 0; }
 int cudaGetLastError(void) { return 0; }
 const char *cudaGetErrorString(int e) { (void)e; return "fake"; }
-int cudaMalloc(void **p, size_t n) { *p = aligned_alloc(256, (n + 255) & ~(size_t)255); return *p ? 0 : 2; }
+
+/* What a context keeps on the device: the last allocation, which tests look into. */
+static unsigned char *device_block;
+static size_t device_block_bytes;
+void *fake_device_block(size_t *bytes) { *bytes = device_block_bytes; return device_block; }
+int cudaMalloc(void **p, size_t n)
+{
+    *p = aligned_alloc(256, (n + 255) & ~(size_t)255);
+    device_block = *p;
+    device_block_bytes = n;
+    return *p ? 0 : 2;
+}
 int cudaFree(void *p) { free(p); return 0; }
 int cudaMemcpy(void *d, const void *s, size_t n, int kind) { (void)kind; memcpy(d, s, n); return 0; }
 int cudaMemcpyAsync(void *d, const void *s, size_t n, int kind, void *st) { (void)kind; (void)st; memcpy(d, s, n); return 0; }
@@ -103,12 +115,22 @@ int cudaLaunchKernel(const void *f, struct dim3 g, struct dim3 b, void **args, s
     return 0;
 }
 
+/* BlockParams (the second argument): the context's device block, and two of its counters side by side, the one that
+ * tasks are claimed from, or null, and that of the CTAs that have ended. */
+static int block_claims(void **args)
+{
+    const uintptr_t *word = args[1], dev = word[3];
+    for (int i = 4; i < 16; ++i) if (word[i] == dev + 256) return word[i - 1] == dev + 128;
+    return -1;
+}
+
 int cudaLaunchKernelExC(const cudaLaunchConfig_t *c, const void *f, void **args)
 {
-    (void)args;
     unsigned cluster = 1;
     for (unsigned i = 0; i < c->numAttrs; ++i) if (c->attrs[i].id == cudaLaunchAttributeClusterDimension) cluster = c->attrs[i].val.clusterDim.x;
-    LOG("launch %s %u %u %zu %u\n", kernel_name(f), c->gridDim.x, c->blockDim.x, c->dynamicSmemBytes, cluster);
+    LOG("launch %s %u %u %zu %u", kernel_name(f), c->gridDim.x, c->blockDim.x, c->dynamicSmemBytes, cluster);
+    if (strstr(kernel_name(f), "block_kernel") != NULL) LOG(" %d", block_claims(args));
+    LOG("\n");
     return 0;
 }
 

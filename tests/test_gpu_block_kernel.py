@@ -53,3 +53,23 @@ def test_edges_of_tiles_and_clusters(k, d, n, dtype, bits):
 def test_tasks_claimed_from_the_counter(k, d):
     """So many tasks per CTA that every mode claims them; each call of the round needs the counter at zero again."""
     test_edges_of_tiles_and_clusters(k, d, 1, "f32", 4)
+
+
+def test_skipped_tasks_leave_no_tile_out():
+    """The hook for the pipeline's waits has no effect on blocks that claim their tiles from the same counter."""
+    import torch
+    from paper_2302_08545_b200 import runner
+    d = 3 * 592 * 8192
+    w = W.Workload("plain", n=1, d=d, log2_block=12, bits=4, granularity=30, table=W.TABLES[(4, 30)], data_seed=1)
+    ctx = runner.context_for(w)
+    r = runner.Round(ctx, 1, d)
+    W.fill_torch(w, r.grads)
+    r.prepare()
+    r.compress(3)
+    want = r.packed[0].clone()
+    r.packed[0].fill_(0xAA)
+    ctx.debug_skip_tasks(3)
+    r.compress(3)
+    torch.cuda.synchronize()
+    assert ctx.status() == 0
+    assert torch.equal(r.packed[0], want)

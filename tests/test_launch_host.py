@@ -73,6 +73,29 @@ for call in transforms(c, 1 << 15) + [lambda: m.prepare_minmax(buf[:2], 1 << 15,
 """)
 
 
+@pytest.mark.parametrize("k", [3, 12, 14])
+def test_skipped_tasks_leave_the_counter_of_claimed_tiles_alone(child, k):
+    """Launches with many tiles claim them from a counter of the context: all of them, from the first on."""
+    child(f"""
+k = {k}
+fake.fake_device_block.restype = ctypes.c_void_p
+size = ctypes.c_size_t()
+for mode in (0, 1):
+    c = context(k, range_mode=mode)
+    block = lambda: ctypes.string_at(fake.fake_device_block(ctypes.byref(size)), size.value)
+    before = block()
+    assert before[128:132] == bytes(4)
+    c.debug_skip_tasks(3)
+    for d in (5, 1 << 25):
+        c.compress(buf[:3], d, 0, buf[0], buf[:3], ws, stream=0)
+    assert [r[6] for r in log() if r[0] == "launch"] == [0, 1]
+    assert block() == before
+c = context(20)
+c.debug_skip_tasks(3)
+assert block()[128:132] == bytes([3, 0, 0, 0])
+""")
+
+
 @pytest.mark.parametrize("k", [15, 16, 17])
 def test_skipped_tasks_take_the_pipeline_once(child, k):
     child(f"""
