@@ -1701,31 +1701,27 @@ int thc_aggregate_decompress(thc_ctx *ctx, const void *const *packed, uint32_t n
     if (outp == nullptr || scales == nullptr || !aligned16(outp)) return THC_EINVAL;
     if (sum_or_null != nullptr && !aligned16(sum_or_null)) return THC_EINVAL;
     const uint32_t k = ctx->cfg.log2_block;
-    if (ctx->cfg.bits != 4 || ctx->cfg.granularity >= 128 || sz.d_pad % 32 != 0 ||
-        (sum_or_null != nullptr && two_call_tail(ctx, sz.d_pad, n))) {
-        // index widths without the byte-lane look-up (there the one launch is
-        // slower than the two): the two calls; the sums go to the caller's buffer or to the workspace
-        // (without a buffer the sums take the end of the workspace; thc_decompress checks that what
-        // is left in front of them is enough for it)
-        uint64_t ws_for_decompress = workspace_bytes;
-        void *sum = sum_or_null;
-        if (sum == nullptr) {
-            if (workspace == nullptr || !aligned16(workspace)) return THC_EINVAL;
-            const uint64_t room = round_up(sz.sum_bytes, 256);
-            if (workspace_bytes < room) return THC_EWORKSPACE;
-            ws_for_decompress = (workspace_bytes - room) & ~(uint64_t)255;
-            sum = static_cast<unsigned char *>(workspace) + ws_for_decompress;
-        }
-        if ((rc = thc_aggregate(ctx, packed, n, d, sum, stream)) != THC_OK) return rc;
-        return thc_decompress(ctx, sum, n, d, round, scales, outp, workspace, ws_for_decompress, stream);
+    // index widths without the byte-lane look-up (there the one launch is slower than the two), and see
+    // two_call_tail: the sums go to the caller's buffer or take the end of the workspace
+    const bool two_calls = ctx->cfg.bits != 4 || ctx->cfg.granularity >= 128 || sz.d_pad % 32 != 0 ||
+                           (sum_or_null != nullptr && two_call_tail(ctx, sz.d_pad, n));
+    // What is refused is refused before the first launch.  Without a buffer room for the sums is asked for where
+    // the one launch needs no workspace too: the same rule for all configurations.
+    uint64_t ws_left = workspace_bytes;
+    if (sum_or_null == nullptr && (two_calls || k <= (uint32_t)kChunkLog2)) {
+        const uint64_t room = round_up(sz.sum_bytes, 256);
+        if (workspace == nullptr || !aligned16(workspace)) return THC_EINVAL;
+        if (workspace_bytes < room) return THC_EWORKSPACE;
+        ws_left = (workspace_bytes - room) & ~(uint64_t)255;
     }
     if (k > (uint32_t)kChunkLog2) {
         if (workspace == nullptr || !aligned16(workspace)) return THC_EINVAL;
-        if (workspace_bytes < pipeline_workspace_need(ctx, sz.nblocks, sz.nblocks)) return THC_EWORKSPACE;
-    } else if (sum_or_null == nullptr) {
-        // needed by configurations that run the two calls: the same rule for all
-        if (workspace == nullptr || !aligned16(workspace)) return THC_EINVAL;
-        if (workspace_bytes < round_up(sz.sum_bytes, 256)) return THC_EWORKSPACE;
+        if (ws_left < pipeline_workspace_need(ctx, sz.nblocks, sz.nblocks)) return THC_EWORKSPACE;
+    }
+    if (two_calls) {
+        void *sum = sum_or_null != nullptr ? sum_or_null : static_cast<unsigned char *>(workspace) + ws_left;
+        if ((rc = thc_aggregate(ctx, packed, n, d, sum, stream)) != THC_OK) return rc;
+        return thc_decompress(ctx, sum, n, d, round, scales, outp, workspace, ws_left, stream);
     }
     PtrArrayP pin;
     MutPtrArrayP pout, prot;

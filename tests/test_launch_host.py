@@ -237,3 +237,29 @@ for total, want in ((buf[2], {launches}), (None, 1)):
     c.aggregate_decompress(buf[:{n}], {d}, 0, buf[0], buf[1], ws, total=total, stream=0)
     assert len(kernels()) == want
 """)
+
+
+@pytest.mark.parametrize("k,bits,d,n", [(17, 4, 1 << 20, 2), (20, 4, 1 << 22, 13), (20, 2, 1 << 22, 2), (15, 4, 1 << 20, 17)])
+def test_one_call_tail_refuses_before_it_launches(child, k, bits, d, n):
+    """Where it runs the two calls too: a missing, misaligned or short workspace leaves the caller's sums alone."""
+    child(f"""
+g = {{2: 3, 4: 30}}[{bits}]
+c = context({k}, bits={bits}, granularity=g, table=W.TABLES[({bits}, g)], workers=32)
+def space(nbytes, address=1 << 32):
+    s = Space()
+    s.nbytes, s.data_ptr = nbytes, lambda: address
+    return s
+sz = c.sizes({d}, 1)
+enough = sz.workspace_bytes
+log()
+for total in (buf[2], None):
+    for ws in (space(0, 0), space(enough, 8), space(255)):
+        try:
+            c.aggregate_decompress(buf[:{n}], {d}, 0, buf[0], buf[1], ws, total=total, stream=0)
+            assert False
+        except thc.ThcError:
+            pass
+        assert log() == []
+    c.aggregate_decompress(buf[:{n}], {d}, 0, buf[0], buf[1], space(enough), total=total, stream=0)
+    assert len(kernels()) == (2 if total or {bits} == 2 else 1)
+""")
