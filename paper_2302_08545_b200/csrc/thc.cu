@@ -1672,20 +1672,40 @@ int thc_decompress(thc_ctx *ctx, const void *sum, uint32_t divisor, uint64_t d, 
 // the worker's estimate line and the inverse RHT): pass A of the inverse transform adds up the
 // table values itself, so the sums need not travel through HBM; they are written only on request.
 // Whether the two calls are faster where the sums are wanted too: a thread's first round waits for the indices of all
-// workers, some at a time, and the pipeline and the tiles of 2^14 have fewer threads to cover that.  us, two calls / one:
-//                     4 workers    8            10           16           24           32
-//   2^ 8  3000        6.7 / 4.9    6.7 / 5.6    6.8 / 6.4    7.3 / 6.9    8.8 / 8.3    10.2 / 9.8
-//   2^12  2^22       13.3 / 10.5  13.7 / 11.4  18.3 / 14.1  19.2 / 15.9  24.1 / 20.2   29.0 / 24.7
-//   2^14  2^24       45.9 / 41.1  48.0 / 48.5  66.3 / 57.2  72.0 / 67.9  86.4 / 90.8  100.5 / 112.9
-//   2^16  2^20       12.9 / 12.4  13.5 / 13.2  14.8 / 14.5  16.1 / 15.2  18.0 / 17.2   19.8 / 19.2   (clusters)
-//   2^17  2^20       13.7 / 13.8  14.3 / 14.8  15.8 / 16.3  17.0 / 17.5  18.9 / 19.9   20.3 / 22.2   (clusters)
-//   2^20  25.6 M     86.6 / 76.1  90.1 / 87.1   115 / 100    125 / 129    146 / 165     168 / 202
-//   2^22  2^26        271 / 236    283 / 255    343 / 284    362 / 352    429 / 442     477 / 528
+// workers, some at a time, and the pipeline and the tiles of 2^14 have fewer threads to cover that.  Two launches win
+// where the tail is latency (few tiles) and where many workers' loads queue up, one launch where the tiles fill the
+// GPU once.  (Pipeline, up to 2^24 coordinates: the two cross between 12 and 17 workers, by up to 4 % either way at 13
+// to 16; the line is 12 for all of them.)  us, two calls / one:
+//                     4 workers    8            13           14           16           17           20           24           32
+//   2^ 8  3000        6.7 / 4.9    6.7 / 5.6                              7.3 / 6.9                              8.8 / 8.3    10.2 / 9.8
+//   2^12  2^22       13.3 / 10.5  13.7 / 11.4                            19.2 / 15.9                            24.1 / 20.2   29.0 / 24.7
+//   2^14  2^20        9.3 / 8.5    9.9 / 9.5   11.4 / 11.7  11.5 / 12.1  11.7 / 12.2  12.6 / 13.0  12.9 / 13.6  13.4 / 14.6   15.1 / 17.0
+//         2^22       14.0 / 11.6  15.2 / 13.2  20.1 / 16.8  20.4 / 17.6  20.9 / 18.1  23.7 / 19.4  24.2 / 20.6  25.6 / 22.4   30.4 / 26.3
+//         2^24       46.1 / 40.7  48.3 / 48.5  69.6 / 62.9  70.8 / 66.1  73.0 / 68.4  80.9 / 73.5  83.0 / 80.5  87.5 / 90.0    101 / 115
+//         2^26        155 / 137    164 / 162    243 / 209    246 / 220    259 / 230    289 / 242    301 / 262    323 / 301     383 / 397
+//   2^15  2^20       12.3 / 11.6  12.8 / 12.6  14.5 / 14.8  14.7 / 15.3  14.9 / 15.3  15.8 / 16.1  16.0 / 16.6  16.5 / 17.7   18.2 / 20.1
+//         2^22       19.3 / 16.1  20.2 / 17.5  25.1 / 21.0  25.4 / 21.6  26.1 / 22.3  28.7 / 23.5  29.3 / 24.7  30.7 / 26.2   35.6 / 30.3
+//         2^24       55.8 / 50.0  58.0 / 58.1  81.3 / 72.0  82.8 / 75.2  84.8 / 76.0  93.1 / 80.7  94.5 / 85.0  98.7 / 95.1    112 / 119
+//   2^16  2^20       13.2 / 12.5  13.8 / 13.3  15.3 / 14.9  15.4 / 15.3  15.6 / 15.3  16.6 / 15.8  16.9 / 16.4  17.3 / 17.4   18.9 / 19.4   (clusters)
+//   2^17  2^20       13.7 / 14.0  14.3 / 15.0  16.2 / 17.1  16.4 / 17.7  16.6 / 17.7  17.5 / 18.5  17.8 / 19.0  18.3 / 20.0   19.9 / 22.4   (clusters)
+//         11 blocks  15.2 / 14.8  15.6 / 15.7  18.0 / 18.0  18.1 / 18.5  18.2 / 18.6  19.7 / 19.4  19.8 / 19.9  20.2 / 21.0   22.1 / 23.4
+//         15 blocks  15.6 / 14.9  16.1 / 15.9  18.5 / 18.2  18.6 / 18.7  18.9 / 18.7  20.2 / 19.5  20.5 / 20.0  21.1 / 21.1   23.9 / 23.5
+//   2^16  2^24       62.5 / 55.8  64.9 / 62.8  83.1 / 80.1  84.2 / 82.6  86.8 / 88.8  94.7 / 94.6  96.4 / 104    101 / 117     115 / 143   (pipeline)
+//   2^18  2^26        205 / 194    215 / 218    288 / 284    293 / 291    304 / 312    330 / 329    338 / 360    358 / 405     408 / 499
+//   2^20  2^22       26.3 / 23.7  26.8 / 25.5  31.4 / 30.2  31.9 / 31.1  32.5 / 32.3  35.8 / 34.3  36.1 / 37.2  38.5 / 42.0   42.9 / 52.7
+//         25.6 M     86.8 / 75.7  90.8 / 86.5   120 / 115    122 / 118    126 / 127    138 / 136    141 / 148    149 / 166     171 / 202
+//   2^21  2^24       67.5 / 58.7  70.0 / 67.2  88.2 / 89.2  89.0 / 92.3  92.0 / 99.0  99.3 / 105    102 / 113    106 / 125     120 / 150
+//         2^26        236 / 211    247 / 238    315 / 304    318 / 309    329 / 328    358 / 346    366 / 369    384 / 406     439 / 497
+//   2^22  2^24       75.5 / 64.6  77.5 / 72.0  95.4 / 92.7  96.1 / 96.2  99.0 / 103    107 / 109    109 / 118    113 / 130     128 / 152
+//         2^26        271 / 235    282 / 255    349 / 313    353 / 322    365 / 342    392 / 361    399 / 387    417 / 429     472 / 524
 static bool two_call_tail(const thc_ctx *ctx, uint64_t d_pad, uint32_t n)
 {
     const uint32_t k = ctx->cfg.log2_block;
-    if (use_block_kernel(ctx, d_pad)) return k == 17u || ((k == 14u || k == 15u) && n > 16u);
-    return n > 12u;
+    if (use_block_kernel(ctx, d_pad)) {
+        if (k == 14u || k == 15u) return d_pad <= (1ull << 20) ? n > 16u : d_pad > (1ull << 22) && n > 24u;
+        return k == 17u && (d_pad <= 9ull << 17 || n > 13u);
+    }
+    return n > (d_pad <= (1ull << 24) ? 12u : k == 22u ? 18u : 14u);
 }
 
 int thc_aggregate_decompress(thc_ctx *ctx, const void *const *packed, uint32_t n, uint64_t d, uint32_t round,

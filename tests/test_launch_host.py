@@ -239,6 +239,19 @@ for total, want in ((buf[2], {launches}), (None, 1)):
 """)
 
 
+@pytest.mark.parametrize("k,d,n,launches", [
+    (14, 1 << 24, 24, 1), (14, 1 << 24, 25, 2), (14, 1 << 22, 32, 1), (15, 1 << 22, 32, 1), (15, 1 << 24, 17, 1), (15, 1 << 24, 32, 2),
+    (17, 9 << 17, 2, 2), (17, 10 << 17, 13, 1), (17, 10 << 17, 14, 2), (18, 1 << 25, 14, 1), (18, 1 << 25, 15, 2),
+    (22, 1 << 24, 13, 2), (22, 1 << 25, 18, 1), (22, 1 << 25, 19, 2),
+])
+def test_one_call_tail_by_the_number_of_tiles(child, k, d, n, launches):
+    child(f"""
+c = context({k}, workers=32)
+c.aggregate_decompress(buf[:{n}], {d}, 0, buf[0], buf[1], ws, total=buf[2], stream=0)
+assert len(kernels()) == {launches}
+""")
+
+
 @pytest.mark.parametrize("k,bits,d,n", [(17, 4, 1 << 20, 2), (20, 4, 1 << 22, 13), (20, 2, 1 << 22, 2), (15, 4, 1 << 20, 17)])
 def test_one_call_tail_refuses_before_it_launches(child, k, bits, d, n):
     """Where it runs the two calls too: a missing, misaligned or short workspace leaves the caller's sums alone."""
