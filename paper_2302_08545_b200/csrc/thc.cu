@@ -1468,7 +1468,13 @@ static int launch_block(const thc_ctx *ctx, const void *kern, PipeMode mode, siz
     // still, error feedback 53.3 / 54.9, with tiles of 2^14 30.5 / 32.4; decompress is level up to 7.
     const bool quantises = mode == kCompressF32 || mode == kCompressBF16 || scales_out != nullptr;
     const uint32_t fixed = quantises && tile_log2 == 13u ? 2u : 8u;
-    P.head = P.tasks > (uint64_t)fixed * resident ? &reinterpret_cast<PipeCounters *>(ctx->dev->counters)->head : nullptr;
+    P.head = nullptr;
+    if (P.tasks > (uint64_t)fixed * resident) {
+        P.head = &reinterpret_cast<PipeCounters *>(ctx->dev->counters)->head;
+        kern = block_kernel(mode, ctx->cfg.bits, ctx->identity, k, true);
+        const int rc = ensure_dynamic_smem(kern);
+        if (rc != THC_OK) return rc;
+    }
     void *args[] = {&maps, &P, const_cast<PtrArrayP *>(&in), const_cast<MutPtrArrayP *>(&out), const_cast<MutPtrArrayP *>(&rot),
                     const_cast<PhiloxKeys *>(&ctx->keys)};
     THC_CUDA(cudaLaunchKernelExC(&cfg, kern, args));

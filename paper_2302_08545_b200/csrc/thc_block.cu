@@ -492,8 +492,8 @@ __device__ __forceinline__ void block_scales(const BlockParams &P, uint32_t sq, 
 }
 
 // ------------------------------------------------------------------------ the kernel
-// KIND: see block_kind.
-template <int MODE, int BITS, bool IDENTITY, int KIND>
+// KIND: see block_kind.  CLAIMS: tasks can be claimed from P.head (see block_claims).
+template <int MODE, int BITS, bool IDENTITY, int KIND, bool CLAIMS>
 __global__ void __launch_bounds__(block_tile_log2(KIND) == 13 ? 128 : 256, block_tile_log2(KIND) == 13 ? 4 : 2)
 thc_block_kernel(const __grid_constant__ TmaMaps maps, const __grid_constant__ BlockParams P,
                  const __grid_constant__ PtrArrayP in, const __grid_constant__ MutPtrArrayP outp,
@@ -540,12 +540,13 @@ thc_block_kernel(const __grid_constant__ TmaMaps maps, const __grid_constant__ B
     const uint32_t groups = kScales ? gridDim.x / group : gridDim.x >> E;
     uint32_t task = kScales ? blockIdx.x / group : blockIdx.x >> E;
     uint32_t unit = task, wl = kScales ? rank : 0u;
+    constexpr bool kVectors = !kScales && (kForward || kEF);      // (the others have one, or one to a CTA)
+    const uint32_t unit_step = groups / P.n_local, wl_step = groups - unit_step * P.n_local;
     auto split_task = [&]() {
-        if (!kScales && (kForward || kEF)) {            // (the others have one vector)
+        unit = task;
+        if (kVectors) {
             unit = task / P.n_local;
             wl = task - unit * P.n_local;
-        } else {
-            unit = task;
         }
     };
     split_task();
@@ -619,7 +620,7 @@ thc_block_kernel(const __grid_constant__ TmaMaps maps, const __grid_constant__ B
         const uint32_t par = n & 1u;
         const uint64_t j0 = tile_coord(unit);
         // the task after this one, handed round by the barrier in front of the last round
-        const bool claims = P.head != nullptr && task >= groups && tid == 0 && rank == 0u;
+        const bool claims = CLAIMS && P.head != nullptr && task >= groups && tid == 0 && rank == 0u;
         uint32_t claimed = 0u;
         if (claims) claimed = groups * 2u + atomicAdd(P.head, 1u);
         // ---- constants of the tile's blocks
@@ -760,7 +761,7 @@ thc_block_kernel(const __grid_constant__ TmaMaps maps, const __grid_constant__ B
         if constexpr (kScales) {
             // every worker's sums of squares of this tile are in place
             cluster_wait();
-            if (P.head != nullptr && task >= groups) next_task = cluster_load_u32(cluster_map((uint32_t)__cvta_generic_to_shared(&s_next[par]), 0));
+            if (CLAIMS && P.head != nullptr && task >= groups) next_task = cluster_load_u32(cluster_map((uint32_t)__cvta_generic_to_shared(&s_next[par]), 0));
             block_scales<kBLog2>(P, (uint32_t)__cvta_generic_to_shared(s_sq[par]), blk0, bc, wl == 0u, tid);
         }
         // ---- the tile is in registers: start the next task's load
@@ -768,11 +769,22 @@ thc_block_kernel(const __grid_constant__ TmaMaps maps, const __grid_constant__ B
         const uint64_t j_out = !CLUSTER ? j0 + 32u * rl + 8u * u
                                        : ((uint64_t)unit << k) + ((uint64_t)rank << (kBLog2 - E)) + 32u * rl + 8u * u;
         // (the task after the next one is stored behind the barrier below; a cluster reads its first CTA's)
-        if (task < groups || P.head == nullptr) task += groups;
-        else if (kScales) task = next_task;
-        else if (!CLUSTER) task = s_next[0];
-        else task = cluster_load_u32(cluster_map((uint32_t)__cvta_generic_to_shared(&s_next[0]), 0));
-        if (task < P.tasks) split_task();
+        if (!CLAIMS) {
+            task += groups;
+            if (kVectors) {
+                unit += unit_step;
+                wl += wl_step;
+                if (wl >= P.n_local) { wl -= P.n_local; ++unit; }
+            } else {
+                unit = task;
+            }
+        } else {
+            if (task < groups || P.head == nullptr) task += groups;
+            else if (kScales) task = next_task;
+            else if (!CLUSTER) task = s_next[0];
+            else task = cluster_load_u32(cluster_map((uint32_t)__cvta_generic_to_shared(&s_next[0]), 0));
+            if (task < P.tasks) split_task();
+        }
         fence_proxy_async();                           // these reads before the next load's writes
         if (!CLUSTER) {
             __syncthreads();
@@ -880,7 +892,7 @@ thc_block_kernel(const __grid_constant__ TmaMaps maps, const __grid_constant__ B
     }
     if (kScales) { cluster_arrive(); cluster_wait(); }  // (the others read this CTA's sums)
     // the last CTA clears the task counter for the next launch and finishes the ranges
-    if (P.head != nullptr || (kRange && P.range_out != nullptr)) {
+    if ((CLAIMS && P.head != nullptr) || (kRange && P.range_out != nullptr)) {
         __shared__ uint32_t s_left;
         __threadfence();
         __syncthreads();
@@ -890,17 +902,30 @@ thc_block_kernel(const __grid_constant__ TmaMaps maps, const __grid_constant__ B
             __threadfence();
             if (kRange && P.range_out != nullptr) finish_ranges(P.range_keys, P.nblocks, P.range_out, P.dev, thread, kBThreads);
             if (thread == 0) {
-                if (P.head != nullptr) *P.head = 0u;
+                if (CLAIMS && P.head != nullptr) *P.head = 0u;
                 *P.exited = 0u;
             }
         }
     }
 }
 
-template <int MODE, int KIND>
+// Which kernels can claim their tasks.  The claim costs error feedback, the exact range and aggregate + decompress 0.1 to
+// 0.4 us a launch even where nothing is claimed (with / without, 4 bits: error feedback of 2 x 3000 in 2^11 blocks
+// 5.46 / 5.06 us, of 4 x 3 M in 2^12 28.1 / 27.7; range 6.17 / 5.88; aggregate + decompress 4.85 / 4.65): they have a kernel
+// of each.  Compress loses 0.1 us (and has most of the kernels), decompress is level.  Clusters of eight have two tasks
+// each at most and claim none: compress, error feedback and the range do without the code (bf16 with 3 bits, seven blocks of
+// 2^17 from two workers, 14.6 / 13.5 us), decompress and the tail are 0.2 to 0.5 us of 11 to 13 faster as compiled with it.
+constexpr bool block_claims(int mode, int kind, bool wanted)
+{
+    const bool both = mode == kErrorFeedback || mode == kRangeF32 || mode == kAggDecompress;
+    const bool inverse = mode == kDecompress8 || mode == kDecompress16 || mode == kDecompress32 || mode == kAggDecompress;
+    return kind < 3 ? wanted || !both : inverse;
+}
+
+template <int MODE, int KIND, bool WANTED>
 static const void *pick(uint32_t bits, bool identity)
 {
-#define THC_BLK(B, I) reinterpret_cast<const void *>(thc_block_kernel<MODE, B, I, KIND>)
+#define THC_BLK(B, I) reinterpret_cast<const void *>(thc_block_kernel<MODE, B, I, KIND, block_claims(MODE, KIND, WANTED)>)
     constexpr bool fused = MODE == kCompressF32Fused || MODE == kCompressBF16Fused;
     if constexpr (fused && KIND > 1) {
         return nullptr;
@@ -926,32 +951,40 @@ static const void *pick(uint32_t bits, bool identity)
 #undef THC_BLK
 }
 
-template <int KIND>
+template <int KIND, bool WANTED>
 static const void *pick_mode(PipeMode mode, uint32_t bits, bool identity)
 {
     switch (mode) {
-    case kCompressF32: return pick<kCompressF32, KIND>(bits, identity);
-    case kCompressBF16: return pick<kCompressBF16, KIND>(bits, identity);
-    case kCompressF32Fused: return pick<kCompressF32Fused, KIND>(bits, identity);
-    case kCompressBF16Fused: return pick<kCompressBF16Fused, KIND>(bits, identity);
-    case kDecompress8: return pick<kDecompress8, KIND>(bits, identity);
-    case kDecompress16: return pick<kDecompress16, KIND>(bits, identity);
-    case kDecompress32: return pick<kDecompress32, KIND>(bits, identity);
-    case kErrorFeedback: return pick<kErrorFeedback, KIND>(bits, identity);
-    case kRangeF32: return pick<kRangeF32, KIND>(bits, identity);
-    case kAggDecompress: return pick<kAggDecompress, KIND>(bits, identity);
+    case kCompressF32: return pick<kCompressF32, KIND, WANTED>(bits, identity);
+    case kCompressBF16: return pick<kCompressBF16, KIND, WANTED>(bits, identity);
+    case kCompressF32Fused: return pick<kCompressF32Fused, KIND, WANTED>(bits, identity);
+    case kCompressBF16Fused: return pick<kCompressBF16Fused, KIND, WANTED>(bits, identity);
+    case kDecompress8: return pick<kDecompress8, KIND, WANTED>(bits, identity);
+    case kDecompress16: return pick<kDecompress16, KIND, WANTED>(bits, identity);
+    case kDecompress32: return pick<kDecompress32, KIND, WANTED>(bits, identity);
+    case kErrorFeedback: return pick<kErrorFeedback, KIND, WANTED>(bits, identity);
+    case kRangeF32: return pick<kRangeF32, KIND, WANTED>(bits, identity);
+    case kAggDecompress: return pick<kAggDecompress, KIND, WANTED>(bits, identity);
     default: return nullptr;
     }
 }
 
-const void *block_kernel(PipeMode mode, uint32_t bits, bool identity, uint32_t k)
+const void *block_kernel(PipeMode mode, uint32_t bits, bool identity, uint32_t k, bool claims)
 {
+    if (claims) {
+        switch (block_kind(k)) {
+        case 0: return pick_mode<0, true>(mode, bits, identity);
+        case 1: return pick_mode<1, true>(mode, bits, identity);
+        case 2: return pick_mode<2, true>(mode, bits, identity);
+        default: break;
+        }
+    }
     switch (block_kind(k)) {
-    case 0: return pick_mode<0>(mode, bits, identity);
-    case 1: return pick_mode<1>(mode, bits, identity);
-    case 2: return pick_mode<2>(mode, bits, identity);
-    case 3: return pick_mode<3>(mode, bits, identity);
-    default: return pick_mode<4>(mode, bits, identity);
+    case 0: return pick_mode<0, false>(mode, bits, identity);
+    case 1: return pick_mode<1, false>(mode, bits, identity);
+    case 2: return pick_mode<2, false>(mode, bits, identity);
+    case 3: return pick_mode<3, false>(mode, bits, identity);
+    default: return pick_mode<4, false>(mode, bits, identity);
     }
 }
 

@@ -43,7 +43,7 @@ struct BlockParams {
 };
 
 // The kernel for a mode, index width and block size (signature: TmaMaps, BlockParams, PtrArrayP,
-// MutPtrArrayP outputs, MutPtrArrayP rotated, PhiloxKeys).
-const void *block_kernel(PipeMode mode, uint32_t bits, bool identity, uint32_t k);
+// MutPtrArrayP outputs, MutPtrArrayP rotated, PhiloxKeys); with claims, the one for launches that are given P.head.
+const void *block_kernel(PipeMode mode, uint32_t bits, bool identity, uint32_t k, bool claims = false);
 
 }  // namespace thc
