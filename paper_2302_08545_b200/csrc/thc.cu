@@ -1365,9 +1365,9 @@ static bool use_block_kernel(const thc_ctx *ctx, uint64_t coords)
 // 123.7 -> 117.6, 8 x 3,000,001 in blocks of 2^13 50.7 -> 47.1; over 448 .. 3500 tiles 22 % faster to 5 % slower
 // (near 700 and 1000 tiles, where 592 leave the shorter last round).  Of clusters of eight there are fewer than the
 // SMs have room for, since a cluster stays within one GPC (2^16: 48 with such a table: 4 x 2^20 coordinates 28.1 -> 24.5 us).
-// The runtime is asked only where shared memory leaves less room than the kernel's registers do (four CTAs
-// or two): that adds some 0.5 us to a context's first call.  Elsewhere no more clusters are launched than
-// there are (block_kernel_serves).
+// The runtime is asked where shared memory leaves less room than the kernel's registers do (four CTAs
+// or two) and for the clusters of scales + compress, whose number depends on the workers: that adds some 0.5 us to a
+// context's first call.  Elsewhere no more clusters are launched than there are (block_kernel_serves).
 constexpr size_t kSmemPerSm = 228u << 10, kSmemPerCta = 1024u + 256u;     // reserved and static
 static int resident_units(const thc_ctx *ctx, uint32_t entry, const void *kern, const cudaLaunchConfig_t &shape, uint32_t cluster, uint32_t *units)
 {
@@ -1461,13 +1461,30 @@ static int launch_block(const thc_ctx *ctx, const void *kern, PipeMode mode, siz
                                                  kern, shape, cluster, &resident); if (rc != THC_OK) return rc; }
     cfg.gridDim = dim3((P.tasks < resident ? P.tasks : resident) * cluster);
     // Tasks claimed from a counter instead of dealt out in a fixed stride: the CTAs of an SM do not progress evenly,
-    // and with fixed shares the mean CTA of a compress ended after four fifths of the time.  us, fixed / claimed, 4 x 2^25
-    // coordinates, 4 bits: compress in 2^12 blocks 222.0 / 202.4, 2^13 of bf16 236.8 / 211.6, 2^14 219.8 / 205.8, 2^15
-    // 327.0 / 308.5, error feedback 2^12 256.8 / 254.2 (2 x 2^28: 1006 / 976, decompress 342 / 333).  With few tasks to a
-    // CTA fixed shares put the last ones on different SMs: 3.7 to 5 tasks a CTA, compress with tiles of 2^13 44.8 / 43.6
-    // still, error feedback 53.3 / 54.9, with tiles of 2^14 30.5 / 32.4; decompress is level up to 7.
-    const bool quantises = mode == kCompressF32 || mode == kCompressBF16 || scales_out != nullptr;
-    const uint32_t fixed = quantises && tile_log2 == 13u ? 2u : 8u;
+    // and with fixed shares the mean CTA of a compress ended after four fifths of the time.  With few tasks to a CTA fixed
+    // shares put the last ones on different SMs; in clusters the claim is read from the first CTA.  us, fixed / claimed,
+    // 4 bits, by tasks to a CTA (cluster) that the GPU holds:
+    //                               2.1          2.9          3.9          4.5          4.9          5.5          6.5          7.5
+    //   tile 2^13  compress         20.7 / 22.0  26.6 / 28.5  34.1 / 33.9  38.3 / 39.9  41.5 / 42.3  45.7 / 44.8  53.4 / 53.3  60.9 / 60.2
+    //              8 workers, bf16  19.5 / 20.9  25.7 / 25.8  33.4 / 33.4  37.7 / 39.4  41.6 / 43.6  45.6 / 45.1  53.4 / 54.0  61.3 / 60.8
+    //   + scales   1 worker         22.7 / 23.8  29.9 / 31.9  38.8 / 38.1               47.5 / 46.5  51.4 / 52.8  60.0 / 59.1
+    //              2 workers        23.7 / 25.1  31.1 / 31.9  39.8 / 39.7               48.8 / 47.5  52.0 / 53.7  61.1 / 62.3
+    //              4 workers        22.9 / 24.5  31.6 / 32.8  41.1 / 42.4               50.0 / 49.2  53.0 / 55.1  65.1 / 64.2
+    //              8 workers        22.9 / 24.2  31.2 / 32.5  41.0 / 42.7               50.1 / 50.4  56.3 / 55.6  65.7 / 64.6
+    //                               6.5          7.5          8.5          10.5         13.5         17.5         24.5         40
+    //              error feedback   66.9 / 67.8  76.5 / 76.6  86.0 / 86.0   103 / 104    130 / 130    168 / 166    234 / 228    384 / 374
+    //              decompress                                 57.3 / 57.1  69.0 / 69.4  88.1 / 86.9   114 / 111    157 / 152    262 / 246
+    //   tile 2^14  compress         56.0 / 53.4  63.4 / 62.4  71.3 / 67.0  86.1 / 83.6   108 / 105    138 / 132    190 / 183    303 / 296
+    //              + 4 workers' scales  74.1 / 69.4  84.3 / 78.6  94.3 / 88.0
+    //              error feedback   74.5 / 70.8  82.9 / 79.6  93.0 / 90.7   113 / 111    141 / 139    180 / 174    246 / 241    400 / 393
+    //              decompress                                 68.4 / 69.1  83.6 / 82.1   105 / 104    135 / 132    186 / 182    302 / 290
+    //   2 x 2^14   compress         78.0 / 79.0  89.3 / 91.2   100 / 104    123 / 122    157 / 155    202 / 198    282 / 275    458 / 441
+    //   (cluster)  error feedback   96.2 / 98.0   111 / 112    125 / 127    152 / 155    193 / 196    248 / 250    344 / 343    561 / 550
+    //              decompress                                  100 / 103    123 / 125    158 / 160    204 / 204    283 / 280    462 / 452
+    //              aggregate + dec.                            101 / 104    123 / 126    158 / 162    204 / 207    284 / 284    463 / 456
+    const bool quantises = mode == kCompressF32 || mode == kCompressBF16;
+    const uint32_t fixed = e != 0u ? (quantises ? 10u : 20u)
+                         : tile_log2 != 13u ? 8u : scales_out != nullptr ? 6u : quantises ? 5u : 8u;
     P.head = nullptr;
     if (P.tasks > (uint64_t)fixed * resident) {
         P.head = &reinterpret_cast<PipeCounters *>(ctx->dev->counters)->head;

@@ -276,3 +276,29 @@ for total in (buf[2], None):
     c.aggregate_decompress(buf[:{n}], {d}, 0, buf[0], buf[1], space(enough), total=total, stream=0)
     assert len(kernels()) == (2 if total or {bits} == 2 else 1)
 """)
+
+
+@pytest.mark.parametrize("k,n,mode,tasks_to_a_cta,claims", [
+    (12, 1, "compress", 5, 0), (12, 3, "compress", 5.1, 1), (14, 1, "compress", 8, 0), (14, 2, "compress", 8.1, 1),
+    (12, 3, "error_feedback", 8, 0), (12, 3, "error_feedback", 8.1, 1), (14, 1, "prepare_minmax", 8, 0), (14, 1, "prepare_minmax", 8.1, 1),
+    (12, 1, "decompress", 8, 0), (12, 1, "decompress", 8.1, 1), (15, 2, "compress", 10, 0), (15, 1, "compress", 10.1, 1),
+    (15, 2, "error_feedback", 20, 0), (15, 2, "error_feedback", 20.1, 1), (15, 1, "decompress", 20.1, 1),
+    (11, 2, "prepare_compress", 6.1, 1), (12, 1, "prepare_compress", 6, 0), (14, 4, "prepare_compress", 8.1, 1), (8, 8, "prepare_compress", 6.1, 1),
+])
+def test_which_launches_claim_their_tasks(child, k, n, mode, tasks_to_a_cta, claims):
+    child(f"""
+k, n, mode = {k}, {n}, "{mode}"
+tile = 13 if k <= 13 else max(k, 14)                                # of a CTA, or of a cluster
+ctas = 592 if k <= 13 else 296 if k == 14 else 148
+c = context(k, workers=n, range_mode=int(mode == "prepare_minmax"))
+x = buf[:n]
+d = int({tasks_to_a_cta} * ctas / n) << tile
+assert d * n >> tile == int({tasks_to_a_cta} * ctas / n) * n
+dict(compress=lambda: c.compress(x, d, 0, buf[0], x, ws, stream=0),
+     prepare_compress=lambda: c.prepare_compress(x, d, 0, buf[0], x, ws, stream=0),
+     prepare_minmax=lambda: c.prepare_minmax(x, d, 0, buf[0], ws, stream=0),
+     decompress=lambda: c.decompress(buf[0], n, d, 0, buf[1], buf[2], ws, stream=0),
+     error_feedback=lambda: c.error_feedback(x, x, d, 0, buf[0], x, ws, stream=0))[mode]()
+rows = [r for r in log() if r[0] == "launch"]
+assert len(rows) == 1 and rows[0][6] == {claims}, rows
+""")
