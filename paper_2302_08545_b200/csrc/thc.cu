@@ -32,7 +32,7 @@ quantize_rotated_kernel(PtrArray rotated, MutPtrArray packed, uint64_t d_pad, ui
     extern __shared__ __align__(16) unsigned char qr_smem[];
     unsigned char *lut = qr_smem;
     float2 *bc = reinterpret_cast<float2 *>(qr_smem + (size_t)(granularity + 1) * kLutEntryBytes);
-    if (!IDENTITY) lut_fill<LutKind<BITS, IDENTITY>::k8>(lut, dev, granularity, threadIdx.x, kThreads);
+    if (!IDENTITY) lut_fill(lut, dev, granularity, threadIdx.x, kThreads);
     depend_on_previous();
     const uint64_t nblocks = d_pad >> k;
     const uint32_t cached = nblocks < (uint64_t)kQrBlockCache ? (uint32_t)nblocks : (uint32_t)kQrBlockCache;
@@ -43,7 +43,7 @@ quantize_rotated_kernel(PtrArray rotated, MutPtrArray packed, uint64_t d_pad, ui
     const float *rot = static_cast<const float *>(rotated.p[wl]);
     unsigned char *pk = static_cast<unsigned char *>(packed.p[wl]);
     const float gf = (float)granularity;
-    const uint32_t my_lut = lut_lane_addr<LutKind<BITS, IDENTITY>::k8>(lut, threadIdx.x);
+    const uint32_t my_lut = lut_lane_addr(lut, threadIdx.x);
     for (uint64_t u = (uint64_t)blockIdx.x * kThreads + threadIdx.x; u < d_pad / 8;
          u += (uint64_t)gridDim.x * kThreads) {
         const uint64_t j = u * 8;
@@ -1148,7 +1148,7 @@ static pipe_kernel_t pick_pipe_kernel_kb(uint32_t bits, bool identity)
         case 2: return identity ? thc_pipeline_kernel<MODE, 2, true, KB> : thc_pipeline_kernel<MODE, 2, false, KB>;
         case 3: return identity ? thc_pipeline_kernel<MODE, 3, true, KB> : thc_pipeline_kernel<MODE, 3, false, KB>;
         case 4: return identity ? thc_pipeline_kernel<MODE, 4, true, KB> : thc_pipeline_kernel<MODE, 4, false, KB>;
-        default: return identity ? thc_pipeline_kernel<MODE, 8, true, KB> : thc_pipeline_kernel<MODE, 8, false, KB>;
+        default: return thc_pipeline_kernel<MODE, 8, true, KB>;      // (the only table, see validate_config)
         }
     }
 }
@@ -1814,7 +1814,7 @@ int thc_quantize_rotated(thc_ctx *ctx, const float *const *rotated, uint32_t n_l
     case 2: if (ctx->identity) THC_QR(2, true); else THC_QR(2, false); break;
     case 3: if (ctx->identity) THC_QR(3, true); else THC_QR(3, false); break;
     case 4: if (ctx->identity) THC_QR(4, true); else THC_QR(4, false); break;
-    default: if (ctx->identity) THC_QR(8, true); else THC_QR(8, false); break;
+    default: THC_QR(8, true); break;              // (the only table, see validate_config)
     }
 #undef THC_QR
     return THC_OK;

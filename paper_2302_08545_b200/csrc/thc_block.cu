@@ -590,7 +590,7 @@ thc_block_kernel(const __grid_constant__ TmaMaps maps, const __grid_constant__ B
         mbar_init(&s_full, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (kQuant && !IDENTITY) lut_fill<LutKind<BITS, IDENTITY>::k8>(lut, P.dev, P.granularity, thread, kBThreads);
+    if (kQuant && !IDENTITY) lut_fill(lut, P.dev, P.granularity, thread, kBThreads);
     if (kEF) {
         // table values as floats, one copy per lane (8 copies for 8-bit indices)
         for (int i = thread; i < (1 << BITS) * kFRep; i += kBThreads)
@@ -802,7 +802,7 @@ thc_block_kernel(const __grid_constant__ TmaMaps maps, const __grid_constant__ B
         // ---- epilogue: two iterations over four rows (unrolled over all eight it does not fit the instruction
         // cache); the second iteration's rows move down the register arrays
         const float gf = (float)P.granularity;
-        const uint32_t my_lut = lut_lane_addr<LutKind<BITS, IDENTITY>::k8>(lut, tid);
+        const uint32_t my_lut = lut_lane_addr(lut, tid);
         // Offsets from the thread's first unit fit 32 bits; the rounding calls of a tile (of a cluster's block)
         // share the high word of their counter (see EpilogueCtx).
         const uint64_t limit = kForward ? P.d_pad : P.d;
@@ -943,7 +943,7 @@ static const void *pick(uint32_t bits, bool identity)
         case 2: return identity ? THC_BLK(2, true) : THC_BLK(2, false);
         case 3: return identity ? THC_BLK(3, true) : THC_BLK(3, false);
         case 4: return identity ? THC_BLK(4, true) : THC_BLK(4, false);
-        default: return identity ? THC_BLK(8, true) : THC_BLK(8, false);
+        default: return THC_BLK(8, true);              // (the only table there is)
         }
     } else {
         return THC_BLK(4, true);

@@ -249,37 +249,23 @@ __device__ __forceinline__ float4 flip4(float4 v, uint32_t bits)
 // The quantiser's table in shared memory, indexed by f = floor(u g): what the rounding rule
 // needs about the table interval [T[z0], T[z0+1]] that holds f.  Consecutive entries are 128
 // bytes apart and every entry is replicated over lanes so that a warp's look-ups (random f per
-// lane) never meet in a bank:
-//   indices of up to 4 bits   16 copies of 8 bytes   (R16 = 65536 / gap as fp32,
-//                                                     bf16(-T[z0]) << 16 | z0: table values up to
-//                                                     255 are exact in bf16)
-//   8-bit indices              8 copies of 16 bytes  (-T[z0] as fp32, R16, z0, 0)
+// lane) never meet in a bank: 16 copies of 8 bytes (R16 = 65536 / gap as fp32, bf16(-T[z0]) << 16 | z0: table
+// values up to 255 are exact in bf16).  Indices of 8 bits need none: 256 rising values up to g <= 255 are the identity.
 constexpr int kLutEntryBytes = 128;
 
-template <int BITS, bool IDENTITY>
-struct LutKind { static constexpr bool k8 = !IDENTITY && BITS <= 4; };
-
-template <bool LUT8>
 __device__ __forceinline__ void lut_fill(unsigned char *lut, const DeviceBlock *dev, uint32_t g, int tid, int nthreads)
 {
-    if (LUT8) {
-        for (int idx = tid; idx < (int)(g + 1) * 16; idx += nthreads) {
-            const uint4 e = dev->lut[idx / 16];
-            reinterpret_cast<uint2 *>(lut)[idx] = make_uint2(e.y, (e.x & 0xFFFF0000u) | e.z);
-        }
-    } else {
-        for (int idx = tid; idx < (int)(g + 1) * 8; idx += nthreads)
-            reinterpret_cast<uint4 *>(lut)[idx] = dev->lut[idx / 8];
+    for (int idx = tid; idx < (int)(g + 1) * 16; idx += nthreads) {
+        const uint4 e = dev->lut[idx / 16];
+        reinterpret_cast<uint2 *>(lut)[idx] = make_uint2(e.y, (e.x & 0xFFFF0000u) | e.z);
     }
 }
 
 // Shared-space byte address of this lane's copy of entry 0, minus 0x4B000000 * 128: the bits of
 // the float 2^23 + f, times 128, plus this value is the address of entry f.
-template <bool LUT8>
 __device__ __forceinline__ uint32_t lut_lane_addr(const unsigned char *lut, int lane)
 {
-    const uint32_t copy = LUT8 ? (uint32_t)(lane & 15) * 8u : (uint32_t)(lane & 7) * 16u;
-    return (uint32_t)__cvta_generic_to_shared(lut) + copy - 0x4B000000u * (uint32_t)kLutEntryBytes;
+    return (uint32_t)__cvta_generic_to_shared(lut) + (uint32_t)(lane & 15) * 8u - 0x4B000000u * (uint32_t)kLutEntryBytes;
 }
 
 // Stochastic quantisation of four consecutive rotated coordinates to table indices
@@ -303,7 +289,7 @@ template <int BITS, bool IDENTITY>
 __device__ __forceinline__ uint32_t quantize4(float r0, float r1, float r2, float r3, float kappa, float offset,
                                               float gf, uint32_t w0, uint32_t w1, uint32_t lut_addr)
 {
-    constexpr bool kLut8 = LutKind<BITS, IDENTITY>::k8;
+    static_assert(IDENTITY || BITS <= 4, "8 bits: identity");
     const float r[4] = {r0, r1, r2, r3};
     const uint32_t words[2] = {w0, w1};
     const float2 big = make_float2(8388608.0f, 8388608.0f), g2 = make_float2(gf, gf);
@@ -330,16 +316,9 @@ __device__ __forceinline__ uint32_t quantize4(float r0, float r1, float r2, floa
                 for (int e = 0; e < 2; ++e) {
                     const uint32_t a = __float_as_uint(tf[e]) * (uint32_t)kLutEntryBytes + lut_addr;
                     uint32_t x, y;
-                    if (kLut8) {
-                        asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(x), "=r"(y) : "r"(a));
-                        nt[e] = __uint_as_float(y & 0xFFFF0000u);
-                        zw[e] = y;
-                    } else {
-                        uint32_t z, w;
-                        asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(y), "=r"(x), "=r"(z), "=r"(w) : "r"(a));
-                        nt[e] = __uint_as_float(y);
-                        zw[e] = z;
-                    }
+                    asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(x), "=r"(y) : "r"(a));
+                    nt[e] = __uint_as_float(y & 0xFFFF0000u);
+                    zw[e] = y;
                     r16[e] = __uint_as_float(x);
                 }
                 const float2 delta = __ffma2_rn(u, g2, make_float2(nt[0], nt[1]));

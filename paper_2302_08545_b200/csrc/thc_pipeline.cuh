@@ -1094,7 +1094,7 @@ thc_pipeline_kernel(const __grid_constant__ TmaMaps maps, PipeParams P, PtrArray
         mbar_init(&s_done, kPThreads);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (kCompress && !IDENTITY && !kRange) lut_fill<LutKind<BITS, IDENTITY>::k8>(lut, P.dev, P.granularity, tid, kPCtaThreads);
+    if (kCompress && !IDENTITY && !kRange) lut_fill(lut, P.dev, P.granularity, tid, kPCtaThreads);
     // error feedback: table values as floats, one copy per lane (8 copies for 8-bit indices)
     constexpr int kFRep = BITS <= 4 ? 32 : 8;
     float *ftab = reinterpret_cast<float *>(lut);
@@ -1508,7 +1508,7 @@ thc_pipeline_kernel(const __grid_constant__ TmaMaps maps, PipeParams P, PtrArray
                 const uint64_t j_tile = r * B + ((uint64_t)idx << (kPLog2 - kb));
                 EpilogueCtx ep;
                 ep.kappa = bc.x; ep.half_g = bc.y; ep.gf = (float)P.granularity; ep.c_block = P.c_block;
-                ep.lut = lut_lane_addr<LutKind<BITS, IDENTITY>::k8>(lut, tid);
+                ep.lut = lut_lane_addr(lut, tid);
                 ep.worker = P.worker_base + wl; ep.round = P.round;
                 ep.call_lo = (uint32_t)(j_tile >> 3); ep.call_hi = (uint32_t)(r * B >> 35);
                 float *rot = static_cast<float *>(rotated.p[wl]);
