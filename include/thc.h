@@ -233,11 +233,17 @@ int thc_prepare_minmax(thc_ctx *ctx, const void *const *grads, uint32_t n, uint6
  * (the simulated cluster): same arguments and results as the two calls in a row, `scales`
  * (device, nblocks floats) being written here and usable by thc_decompress afterwards.
  * Section 5.3 observes that the norm exchange can overlap the RHT: only the quantiser needs M,
- * so where the block size is 2^17 (more than some 15 blocks over all workers) to 2^20, the input fp32
- * and n small enough for the intermediate ring to stay in L2, the transform kernel sums the squares
- * of the tiles it loads anyway and the gradients are read from HBM once instead of twice.  Elsewhere this runs the two calls.
- * The fp64 sums are added in a different (fixed) order than thc_prepare's, so a scale may
- * differ from thc_prepare's in the last bit.  */
+ * so the transform kernel sums the squares of the tiles it loads anyway and the gradients are read from
+ * HBM once instead of twice:
+ *   - blocks of 2^8 .. 2^14, up to eight workers, fp32 or bf16; large inputs in blocks of 2^13 and 2^14
+ *     (more than 2^22 coordinates over all workers) only in fp32, in 2^14 blocks up to six workers;
+ *   - blocks of 2^17 (more than some 15 over all workers) to 2^20, fp32, n small enough for the
+ *     intermediate ring to stay in L2.
+ * thc_sizes reports it as fused_scales = 1; elsewhere this runs the two calls (THC_RANGE_MINMAX contexts have no such
+ * scales: THC_EUNSUPPORTED).
+ * In the one launch the fp64 sums are added in a different (fixed) order than thc_prepare's, so a scale
+ * may differ from thc_prepare's in the last bit: ranks whose indices are to be summed take their scales
+ * from the same call.  */
 int thc_prepare_compress(thc_ctx *ctx, const void *const *grads, uint32_t n, uint32_t worker_base,
                          uint64_t d, uint32_t round, float *scales, void *const *packed,
                          float *const *rotated_or_null, void *workspace, uint64_t workspace_bytes,
@@ -267,8 +273,8 @@ int thc_status(thc_ctx *ctx, uint32_t *flags, void *stream);
 
 /* Test hook for the bounded waits of the large-block pipeline (no counterpart in the paper).
  * The next call on this context that transforms blocks above 2^14 takes the pipeline whatever
- * their size and starts its task queue at position `count` instead of 0 (blocks of up to 2^14 have no
- * queue: no effect), so tasks that depend on the skipped ones can never be satisfied: the
+ * their size and starts its task queue at position `count` instead of 0 (blocks of up to 2^14 do not
+ * take the pipeline: no effect), so tasks that depend on the skipped ones can never be satisfied: the
  * kernel must notice (about one second), set THC_STATUS_WAIT_TIMEOUT, and return with the
  * context still usable; the outputs of that call are undefined.  Synchronises the device. */
 int thc_debug_skip_tasks(thc_ctx *ctx, uint32_t count);

@@ -19,15 +19,15 @@
 // the next tile's TMA copy is started, so the
 // epilogue hides it.
 //
-// What bounds it.  Timers in the kernel, 4 x 2^26 coordinates in blocks of 2^12, 4 bits: per tile a CTA spends
-// 2190 cycles on the load and the block constants, 2350 on round 1, 1650 on round 2 and its barrier, 1230 on
-// the last round and 5480 on the epilogue (Philox and the quantiser, bound by instruction issue), with four CTAs side by side
-// on an SM; with fixed shares of the tiles the CTAs ran for 371 us of 465 on average, hence the counter.
-// Against five rounds through shared memory with a block barrier between them: blocks of 2^12 compress
-// 669 -> 441 us, decompress 156 -> 95 us, error feedback 1310 -> 509 us; 2^14 681 -> 435, 155 -> 115,
-// 1316 -> 539 us.  In a cluster the gather binds (a tile of every CTA crosses the SM-to-SM network: 8740
+// What bounds it.  Timers in the kernel, 4 x 2^26 coordinates in blocks of 2^12, 4 bits, before the quantiser was
+// packed: per tile a CTA spent 2190 cycles on the load and the block constants, 2350 on round 1, 1650 on round 2 and its
+// barrier, 1230 on the last round and 5480 on the epilogue (Philox and the quantiser, bound by instruction issue), with
+// four CTAs side by side on an SM; with fixed shares of the tiles the CTAs ran for 371 us of 465 on average, hence the counter.
+// Now (five rounds through shared memory with a block barrier between them in front): blocks of 2^12 compress
+// 669 -> 400 us, decompress 156 -> 93 us, error feedback 1310 -> 499 us; 2^14 681 -> 408, 155 -> 111,
+// 1316 -> 531 us.  In a cluster the gather binds (a tile of every CTA crosses the SM-to-SM network: 8740
 // cycles for the last round of a tile of 2^15 where one of 2^14 takes 1580): 2^15 is as fast as the
-// two-pass pipeline on large inputs (645 us; error feedback 985 -> 763 us) and takes 9.3 instead of 13.1 us on
+// two-pass pipeline on large inputs (611 us; error feedback 985 -> 758 us) and takes 9.3 instead of 13.1 us on
 // a few blocks; 2^16 and 2^17 pay only there (see block_kernel_serves).
 #include "thc_block.h"
 
