@@ -55,11 +55,56 @@ def test_tasks_claimed_from_the_counter(k, d):
     test_edges_of_tiles_and_clusters(k, d, 1, "f32", 4)
 
 
+def _claimed(tile_log2, n, per_cta=8):
+    """A vector of which n have more than per_cta tiles for each CTA that the GPU can hold: they are claimed."""
+    import torch
+    ctas = torch.cuda.get_device_properties(0).multi_processor_count * (4 if tile_log2 == 13 else 2)
+    return (per_cta * ctas // n + 1 << tile_log2) + 5
+
+
+@pytest.mark.parametrize("k,n", [(12, 3), (15, 2)])
+def test_tasks_of_several_workers_claimed_from_the_counter(k, n):
+    """Error feedback too: a claimed task is a tile and a worker."""
+    test_edges_of_tiles_and_clusters(k, _claimed(13, n) if k == 12 else _claimed(14, n, 20), n, "f32", 4)
+
+
+def test_exact_range_with_claimed_tasks():
+    """The last CTA clears the counter of the claimed tasks and finishes the ranges: twice, against the extremes of
+    the rotated coordinates that the call hands out, and compress and error feedback on these ranges."""
+    import torch
+    from paper_2302_08545_b200 import runner
+    k, d = 14, _claimed(14, 1)
+    w = W.Workload("plain", n=1, d=d, log2_block=k, bits=4, granularity=30, table=W.TABLES[(4, 30)], data_seed=1)
+    ctx = runner.context_for(w, exact_range=True)
+    r = runner.Round(ctx, 1, d, want_rotated=True)
+    nb = r.sz.nblocks
+    assert nb <= 4096                                   # finished in the same launch
+    for call in range(2):
+        W.fill_torch(w, r.grads, seed_offset=call)
+        r.scales.fill_(-7.0)
+        r.rotated[0].fill_(float("nan"))
+        r.prepare_minmax(call)
+        torch.cuda.synchronize()
+        assert ctx.status() == 0
+        blocks = r.rotated[0].view(nb, 1 << k)
+        assert torch.equal(r.scales[:nb], blocks.amin(1)) and torch.equal(r.scales[nb:], blocks.amax(1))
+        r.compress(call)
+        one = r.packed[0].clone()
+        r.quantize_rotated(call)
+        assert torch.equal(one, r.packed[0])
+    x = r.grads[0].cpu().numpy()
+    c = O.Config(bits=4, granularity=30, table=tuple(w.table), t_p=w.t_p, log2_block=k, seed=w.seed)
+    lo, hi = O.ranges(x[None], c, 1)
+    got = r.scales.cpu().numpy()
+    assert np.array_equal(got[:nb].view(np.uint32), lo.view(np.uint32))
+    assert np.array_equal(got[nb:].view(np.uint32), hi.view(np.uint32))
+
+
 def test_skipped_tasks_leave_no_tile_out():
     """The hook for the pipeline's waits has no effect on blocks that claim their tiles from the same counter."""
     import torch
     from paper_2302_08545_b200 import runner
-    d = 3 * 592 * 8192
+    d = _claimed(13, 1)
     w = W.Workload("plain", n=1, d=d, log2_block=12, bits=4, granularity=30, table=W.TABLES[(4, 30)], data_seed=1)
     ctx = runner.context_for(w)
     r = runner.Round(ctx, 1, d)

@@ -82,3 +82,40 @@ def test_blocks_in_shared_memory_one_launch_equals_the_two_calls(k, d, n, dtype,
         r.compress(call)
         torch.cuda.synchronize()
         assert all(torch.equal(a, b) for a, b in zip(p, r.packed))
+
+
+@pytest.mark.parametrize("k,n,dtype,bits", [(14, 1, "f32", 4), (14, 4, "f32", 2), (11, 2, "bf16", 3), (8, 8, "f32", 4)])
+def test_blocks_in_shared_memory_with_claimed_clusters(k, n, dtype, bits):
+    """More than eight (tiles of 2^13: six) tasks for each cluster that the GPU can hold."""
+    import torch
+    ctas = torch.cuda.get_device_properties(0).multi_processor_count * (2 if k == 14 else 4)
+    tile_log2, per_cluster = (14, 8) if k == 14 else (13, 6)
+    d = (per_cluster * ctas // n + 1 << tile_log2) + 5
+    test_blocks_in_shared_memory_one_launch_equals_the_two_calls(k, d, n, dtype, bits)
+
+
+@pytest.mark.parametrize("k,d,n,dtype", [(8, 8192 * 3 + 77, 3, "f32"), (12, 100_003, 2, "bf16"), (14, 50_000, 5, "f32")])
+def test_blocks_in_shared_memory_rotated_and_worker_base(k, d, n, dtype):
+    """The rotated coordinates, and the random numbers of workers that do not begin at 0."""
+    import torch
+    from paper_2302_08545_b200 import runner
+    w = W.Workload("plain", n=n, d=d, log2_block=k, bits=4, granularity=30, table=W.TABLES[(4, 30)], in_dtype=dtype, data_seed=k)
+    ctx = runner.context_for(w)
+    r = runner.Round(ctx, n, d, dtype, want_rotated=True)
+    assert r.sz.fused_scales == 1
+    W.fill_torch(w, r.grads)
+    got = []
+    for base in (5, 0):
+        for t in r.rotated:
+            t.fill_(float("nan"))
+        ctx.prepare_compress(r.grads, d, 2, r.scales, r.packed, r.workspace, rotated=r.rotated, worker_base=base)
+        p, rot = [t.clone() for t in r.packed], [t.clone() for t in r.rotated]
+        for t in r.packed:
+            t.fill_(0xAA)
+        ctx.compress(r.grads, d, 2, r.scales, r.packed, r.workspace, rotated=r.rotated, worker_base=base)
+        torch.cuda.synchronize()
+        assert ctx.status() == 0
+        assert all(torch.equal(a, b) for a, b in zip(p, r.packed))
+        assert all(torch.equal(a.view(torch.int32), b.view(torch.int32)) for a, b in zip(rot, r.rotated))
+        got.append(p[0])
+    assert not torch.equal(got[0], got[1])
