@@ -1482,9 +1482,12 @@ static int launch_block(const thc_ctx *ctx, const void *kern, PipeMode mode, siz
     //   (cluster)  error feedback   96.2 / 98.0   111 / 112    125 / 127    152 / 155    193 / 196    248 / 250    344 / 343    561 / 550
     //              decompress                                  100 / 103    123 / 125    158 / 160    204 / 204    283 / 280    462 / 452
     //              aggregate + dec.                            101 / 104    123 / 126    158 / 162    204 / 207    284 / 284    463 / 456
-    const bool quantises = mode == kCompressF32 || mode == kCompressBF16;
-    const uint32_t fixed = e != 0u ? (quantises ? 10u : 20u)
-                         : tile_log2 != 13u ? 8u : scales_out != nullptr ? 6u : quantises ? 5u : 8u;
+    //   exact range     2^13       45.7 / 47.6               57.9 / 59.9  70.2 / 70.7  88.0 / 88.5   111 / 111    152 / 150
+    //                   2^14       49.4 / 47.9               60.5 / 58.1  73.5 / 71.2  92.9 / 89.7   111 / 108    150 / 146
+    //                   2 x 2^14   69.9 / 71.7               90.5 / 92.3   110 / 112    139 / 138    178 / 176    247 / 242
+    const bool quantises = mode == kCompressF32 || mode == kCompressBF16, range = mode == kRangeF32;
+    const uint32_t fixed = e != 0u ? (quantises || range ? 10u : 20u)
+                         : tile_log2 != 13u ? 8u : scales_out != nullptr ? 6u : quantises ? 5u : range ? 16u : 8u;
     P.head = nullptr;
     if (P.tasks > (uint64_t)fixed * resident) {
         P.head = &reinterpret_cast<PipeCounters *>(ctx->dev->counters)->head;

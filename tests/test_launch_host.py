@@ -282,6 +282,7 @@ for total in (buf[2], None):
     (12, 1, "compress", 5, 0), (12, 3, "compress", 5.1, 1), (14, 1, "compress", 8, 0), (14, 2, "compress", 8.1, 1),
     (12, 3, "error_feedback", 8, 0), (12, 3, "error_feedback", 8.1, 1), (14, 1, "prepare_minmax", 8, 0), (14, 1, "prepare_minmax", 8.1, 1),
     (12, 1, "decompress", 8, 0), (12, 1, "decompress", 8.1, 1), (15, 2, "compress", 10, 0), (15, 1, "compress", 10.1, 1),
+    (15, 1, "prepare_minmax", 10, 0), (15, 1, "prepare_minmax", 10.1, 1),
     (15, 2, "error_feedback", 20, 0), (15, 2, "error_feedback", 20.1, 1), (15, 1, "decompress", 20.1, 1),
     (11, 2, "prepare_compress", 6.1, 1), (12, 1, "prepare_compress", 6, 0), (14, 4, "prepare_compress", 8.1, 1), (8, 8, "prepare_compress", 6.1, 1),
 ])
@@ -299,6 +300,6 @@ dict(compress=lambda: c.compress(x, d, 0, buf[0], x, ws, stream=0),
      prepare_minmax=lambda: c.prepare_minmax(x, d, 0, buf[0], ws, stream=0),
      decompress=lambda: c.decompress(buf[0], n, d, 0, buf[1], buf[2], ws, stream=0),
      error_feedback=lambda: c.error_feedback(x, x, d, 0, buf[0], x, ws, stream=0))[mode]()
-rows = [r for r in log() if r[0] == "launch"]
+rows = [r for r in log() if r[0] == "launch" and "block_kernel" in r[1]]
 assert len(rows) == 1 and rows[0][6] == {claims}, rows
 """)
